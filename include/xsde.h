@@ -321,9 +321,8 @@ int xsde_integrate_host(xsde_problem *prob, const void *psi_in, void *psi_out, i
  * XSDE_ADJOINT_MAX_BYTES bytes of workspace (environment variable, default
  * 2 GiB) all segments are recomputed at once before the reverse sweep; else one
  * at a time during it, in a buffer of one segment.  Each path runs on one CTA
- * with 8 points per thread, or 4 when the problem's kernel variant is one of
- * the 1D 4- or 2-point shapes (xsde_set_kernel_variant) or, at the default
- * variant 0, when there are fewer paths than SMs.  Asynchronous on
+ * with 4 points per thread, or 8 when the problem's kernel variant is one of
+ * the 1D 8-point shapes 1-3 and 6 (xsde_set_kernel_variant).  Asynchronous on
  * `stream`. */
 int xsde_adjoint(xsde_problem *prob, const xsde_vector *psi0, const xsde_vector *target, double dt, int64_t nsteps,
                  int32_t ckpt_every, double *loss, double *dLdV, void *dLdpsi0, void *stream);
@@ -408,11 +407,13 @@ int xsde_synchronize(xsde_problem *prob, void *stream);
  *     one path) or twice (3, at most 256 threads) as many; variants 4 and 5
  *     give each thread 4 or 2 points (radix-4 or radix-2 stages, so a path
  *     spreads over more warps) with the default paths per CTA for that shape;
- *     variant 0 is compiled for 512 resident threads per SM in complex64 (at
- *     most 128 registers a thread, a few values spilled: more warps to hide
- *     the exchanges' latency) and with all its registers in complex128;
- *     variant 6 is variant 0 with the other choice; where a bound applies a
- *     variant repeats another;
+ *     the 8-point default is compiled for 512 resident threads per SM in
+ *     complex64 (at most 128 registers a thread, a few values spilled: more
+ *     warps to hide the exchanges' latency) and with all its registers in
+ *     complex128; variant 6 is that shape with the other choice; variant 0 takes
+ *     one of these shapes by precision, length and number of paths (few paths
+ *     are spread over more threads); where a bound applies a variant repeats
+ *     another;
  *   2D and 3D lattices (4 variants): 0 uses, in complex64, the persistent
  *     TMA-pipelined row pass (lines of 128..1024 points) and the column pass
  *     with warp-synchronous two-stage transforms (columns of 128..512 points,

@@ -69,8 +69,11 @@ struct xsde_problem {
     void *d_tw[3] = {nullptr, nullptr, nullptr};
     void *d_tw1d[2] = {nullptr, nullptr};   // 1D: twiddles of the radix-4 and radix-2 plans
     void *d_tw2[3] = {nullptr, nullptr, nullptr};   // complex64 2D/3D: two-stage plan twiddles (warp column pass)
+    void *d_tw64 = nullptr;  // complex128 1D: FP64 twiddles of the adaptive integrator
     void *d_twp = nullptr;   // complex64 2D/3D: paired twiddles of the row dimension (TMA row pass)
     void *d_E[3] = {nullptr, nullptr, nullptr};
+    int E_x[3] = {kFxNone, kFxNone, kFxNone};    // complex128: exponents of d_E's limbs (fx.cuh) ...
+    int Ef_x[3] = {kFxNone, kFxNone, kFxNone};   // ... and of d_Ef's
     void *d_scratch = nullptr;
     size_t scratch_bytes = 0;
     int *d_status = nullptr;
@@ -241,9 +244,35 @@ void split_hi_lo(const std::complex<double> &z, float2 *hi, float2 *lo) {
     *hi = make_float2(hr, hm);
     *lo = make_float2((float)(z.real() - (double)hr), (float)(z.imag() - (double)hm));
 }
-void split_hi_lo(const std::complex<double> &z, double2 *hi, double2 *lo) {
-    *hi = make_double2(z.real(), z.imag());
-    *lo = make_double2(0.0, 0.0);
+// c 2^62 as two signed limbs (fx.cuh); |c| may pass 1 by the rounding of a modulus
+void fx_limbs(double c, int *hi, int *lo) {
+    const int64_t q = std::llround(std::ldexp(c, 62));
+    int64_t l = (int64_t)(int32_t)(uint32_t)(uint64_t)q;
+    if (l == INT32_MIN) ++l;   // the kernels negate the limbs
+    *lo = (int)l;
+    *hi = (int)((q - (int64_t)(int32_t)(uint32_t)(uint64_t)q) >> 32);
+}
+int4 fx_limbs(const std::complex<double> &z) {
+    int4 w;
+    fx_limbs(z.real(), &w.x, &w.y);
+    fx_limbs(z.imag(), &w.z, &w.w);
+    return w;
+}
+// Exponent e for a table of complex128 factors as limbs, f = limbs 2^e: the
+// largest modulus takes the limbs' whole range.  The limbs have one absolute
+// precision, so a table whose moduli differ by more than 4 (strong damping or
+// growth over the spectrum) keeps FP64 products: kFxNone.
+int fx_exponent(const std::vector<std::complex<double>> &h) {
+    double big = 0.0, small = HUGE_VAL;
+    for (const auto &z : h) {
+        const double a = std::abs(z);
+        if (!std::isfinite(a)) return kFxNone;
+        big = std::max(big, a);
+        small = std::min(small, a);
+    }
+    if (!(big > 0.0) || small * 4.0 < big) return kFxNone;
+    const int e = (int)std::ceil(std::log2(big) - 1e-9);
+    return e > -900 && e < 900 ? e : kFxNone;
 }
 
 template <typename V> int upload_raw(const std::vector<V> &tmp, void **dptr, cudaStream_t s) {
@@ -254,7 +283,9 @@ template <typename V> int upload_raw(const std::vector<V> &tmp, void **dptr, cud
     return XSDE_OK;
 }
 
-// twiddle table exp(-2 pi i m/n), m < n: FP64 (cos, sin); FP32 (hi, lo) split
+// twiddle table exp(-2 pi i m/n), m < n: complex128 Q62 limbs (FP64 values for
+// the adaptive integrator); FP32 (hi, lo) split
+void make_twiddle(const std::complex<double> &z, int4 *out) { *out = fx_limbs(z); }
 void make_twiddle(const std::complex<double> &z, double2 *out) { *out = make_double2(z.real(), z.imag()); }
 void make_twiddle(const std::complex<double> &z, float4 *out) {
     float2 hi, lo;
@@ -274,9 +305,10 @@ void make_twiddle_paired(const std::complex<double> &z, float4 *out) {
 // per-stage layout of fft.cuh: stage (Ns, R) holds w_n^(r k n/(Ns R)) at
 // [stage_table_offset(n, Ns) + (r-1) Ns + k]; n entries are allocated (the
 // table needs at most n - 1).  PAIRED (complex64): entries for fftp_*.
-template <typename R, int E = 8, bool PAIRED = false> int upload_twiddles(int n, void **dptr, cudaStream_t s) {
-    std::vector<tw_t<R>> tmp(n);
-    auto put = [&](const std::complex<double> &z, tw_t<R> *out) {
+template <typename R, int E = 8, bool PAIRED = false, typename TW = tw_t<R>>
+int upload_twiddles(int n, void **dptr, cudaStream_t s) {
+    std::vector<TW> tmp(n);
+    auto put = [&](const std::complex<double> &z, TW *out) {
         if constexpr (PAIRED) make_twiddle_paired(z, out);
         else make_twiddle(z, out);
     };
@@ -306,11 +338,27 @@ int upload_twiddles_2stage(int n, int E, void **dptr, cudaStream_t s) {
     return upload_raw(tmp, dptr, s);
 }
 
-// factor table as [hi[0..n), lo[0..n)]
-template <typename V> int upload(const std::vector<std::complex<double>> &h, void **dptr, cudaStream_t s) {
-    const size_t n = h.size();
-    std::vector<V> tmp(2 * n);
-    for (size_t i = 0; i < n; ++i) split_hi_lo(h[i], &tmp[i], &tmp[n + i]);
+// factor table [2 n]: complex64 hi [n], lo [n]; complex128 values [n], limbs [n]
+// (zero, and *fex = kFxNone, where fx_exponent gives none)
+void fill_factors(const std::vector<std::complex<double>> &h, float2 *out, int *fex) {
+    for (size_t i = 0; i < h.size(); ++i) split_hi_lo(h[i], &out[i], &out[h.size() + i]);
+    if (fex) *fex = kFxNone;
+}
+void fill_factors(const std::vector<std::complex<double>> &h, double2 *out, int *fex) {
+    static_assert(sizeof(int4) == sizeof(double2), "limbs take the place of lo");
+    const int e = fex ? fx_exponent(h) : kFxNone;
+    for (size_t i = 0; i < h.size(); ++i) {
+        out[i] = make_double2(h[i].real(), h[i].imag());
+        const int4 w = e == kFxNone ? make_int4(0, 0, 0, 0)
+                                    : fx_limbs(std::complex<double>(std::ldexp(h[i].real(), -e), std::ldexp(h[i].imag(), -e)));
+        std::memcpy(&out[h.size() + i], &w, sizeof w);
+    }
+    if (fex) *fex = e;
+}
+template <typename V>
+int upload(const std::vector<std::complex<double>> &h, void **dptr, cudaStream_t s, int *fex = nullptr) {
+    std::vector<V> tmp(2 * h.size());
+    fill_factors(h, tmp.data(), fex);
     return upload_raw(tmp, dptr, s);
 }
 
@@ -344,9 +392,9 @@ template <typename V> int ensure_tables(xsde_problem *p, double dt, cudaStream_t
         if (g.basis[0] != XSDE_BASIS_FOURIER) {
             std::vector<std::complex<double>> A, B;
             trig_pair_tables(g.basis[0], e, A, B);
-            if ((rc = upload<V>(A, &p->d_E[0], s)) != XSDE_OK) return rc;
+            if ((rc = upload<V>(A, &p->d_E[0], s, &p->E_x[0])) != XSDE_OK) return rc;
             if ((rc = upload<V>(B, &p->d_B, s)) != XSDE_OK) return rc;
-        } else if ((rc = upload<V>(e, &p->d_E[0], s)) != XSDE_OK) {
+        } else if ((rc = upload<V>(e, &p->d_E[0], s, &p->E_x[0])) != XSDE_OK) {
             return rc;
         }
     } else if (g.ndim == 2) {
@@ -372,8 +420,8 @@ template <typename V> int ensure_tables(xsde_problem *p, double dt, cudaStream_t
             e1 = A;
             if ((rc = upload<V>(B, &p->d_B1, s)) != XSDE_OK) return rc;
         }
-        if ((rc = upload<V>(e0, &p->d_E[0], s)) != XSDE_OK) return rc;
-        if ((rc = upload<V>(e1, &p->d_E[1], s)) != XSDE_OK) return rc;
+        if ((rc = upload<V>(e0, &p->d_E[0], s, &p->E_x[0])) != XSDE_OK) return rc;
+        if ((rc = upload<V>(e1, &p->d_E[1], s, &p->E_x[1])) != XSDE_OK) return rc;
         if (p->scheme == XSDE_SCHEME_SEMI_IMPLICIT) {
             // a whole step exp(L dt) between two semi-implicit stages (no pairing: Fourier lattices)
             std::vector<std::complex<double>> f0(g.n[0]), f1(g.n[1]);
@@ -385,8 +433,8 @@ template <typename V> int ensure_tables(xsde_problem *p, double dt, cudaStream_t
                 const double k = kval(g, 1, i);
                 f1[i] = std::exp(c2 * (k * k) * dt);
             }
-            if ((rc = upload<V>(f0, &p->d_Ef[0], s)) != XSDE_OK) return rc;
-            if ((rc = upload<V>(f1, &p->d_Ef[1], s)) != XSDE_OK) return rc;
+            if ((rc = upload<V>(f0, &p->d_Ef[0], s, &p->Ef_x[0])) != XSDE_OK) return rc;
+            if ((rc = upload<V>(f1, &p->d_Ef[1], s, &p->Ef_x[1])) != XSDE_OK) return rc;
         }
     } else if (g.ndim == 3) {
         // exp(L dt/2) = E0(k0) E1(k1) E2(k2); E0 carries exp(c0 dt/2)/(n0 n1 n2)
@@ -408,7 +456,7 @@ template <typename V> int ensure_tables(xsde_problem *p, double dt, cudaStream_t
                     e = A;
                     if ((rc = upload<V>(B, d == 0 ? &p->d_B : d == 1 ? &p->d_B1 : &p->d_B2, s)) != XSDE_OK) return rc;
                 }
-                if ((rc = upload<V>(e, h == 0 ? &p->d_E[d] : &p->d_Ef[d], s)) != XSDE_OK) return rc;
+                if ((rc = upload<V>(e, h == 0 ? &p->d_E[d] : &p->d_Ef[d], s, h == 0 ? &p->E_x[d] : &p->Ef_x[d])) != XSDE_OK) return rc;
             }
         }
     }
@@ -672,16 +720,19 @@ int run_3d(xsde_problem *p, void *psi, int64_t nsteps, int64_t npaths, uint64_t 
     qr.nmid = g.n[1];
     qr.tw1 = static_cast<const tw_t<R> *>(p->d_tw[2]);
     qr.E1 = static_cast<const V *>(p->d_E[2]);
+    qr.E1x = p->E_x[2];
     q1.npaths = npaths * g.n[0];              // columns along dimension 1, one slab per (path, i0)
     q1.n0 = g.n[1];
     q1.n1 = g.n[2];
     q1.tw0 = static_cast<const tw_t<R> *>(p->d_tw[1]);
     q1.E0 = static_cast<const V *>(p->d_E[1]);
+    q1.E0x = p->E_x[1];
     q0.npaths = npaths;                       // columns along dimension 0
     q0.n0 = g.n[0];
     q0.n1 = g.n[1] * g.n[2];
     q0.tw0 = static_cast<const tw_t<R> *>(p->d_tw[0]);
     q0.E0 = static_cast<const V *>(p->d_E[0]);
+    q0.E0x = p->E_x[0];
     q0.kinner = g.n[2];
     // cosine / sine dimensions: each pass pairs along its own dimension; the
     // spectral dimension-0 pass weighs the modes of dimensions 1 and 2
@@ -793,6 +844,7 @@ int run_si_2d(xsde_problem *p, Params2D<R> &q, int64_t nsteps, uint64_t step0, c
     auto row = [&](int op, const V *e1, uint64_t sg, int slot) -> cudaError_t {
         q.si_op = op;
         q.E1 = e1;
+        q.E1x = (e1 == E1f ? p->Ef_x : p->E_x)[1];
         q.sg = sg;
         q.sample_slot = slot;
         return timed(p, 4, s, [&] { return launch_row_pass<R>(ROW_SI, q, s); });
@@ -812,6 +864,7 @@ int run_si_2d(xsde_problem *p, Params2D<R> &q, int64_t nsteps, uint64_t step0, c
     }
     auto col = [&](const V *e0) -> cudaError_t {
         q.E0 = e0;
+        q.E0x = (e0 == E0f ? p->Ef_x : p->E_x)[0];
         q.sample_slot = -1;
         return timed(p, 7, s, [&] {
             if constexpr (std::is_same<R, float>::value)
@@ -871,6 +924,7 @@ int run_si_3d(xsde_problem *p, Params2D<R> &qr, Params2D<R> &q1, Params2D<R> &q0
     auto row = [&](int op, bool whole, uint64_t sg, int slot) -> cudaError_t {
         qr.si_op = op;
         qr.E1 = whole ? Ef[2] : Eh[2];
+        qr.E1x = (whole ? p->Ef_x : p->E_x)[2];
         qr.sg = sg;
         qr.sample_slot = slot;
         return timed(p, 4, s, [&] { return launch_row_pass<R>(ROW_SI, qr, s); });
@@ -878,6 +932,8 @@ int run_si_3d(xsde_problem *p, Params2D<R> &qr, Params2D<R> &q1, Params2D<R> &q0
     auto cols = [&](bool whole) -> cudaError_t {
         q1.E0 = whole ? Ef[1] : Eh[1];
         q0.E0 = whole ? Ef[0] : Eh[0];
+        q1.E0x = (whole ? p->Ef_x : p->E_x)[1];
+        q0.E0x = (whole ? p->Ef_x : p->E_x)[0];
         q1.sample_slot = q0.sample_slot = -1;
         cudaError_t e = timed(p, 7, s, [&] { return launch_col_pass<R>(COL_SINGLE, q1, s); });
         if (e != cudaSuccess) return e;
@@ -1014,8 +1070,11 @@ int run_integrate(xsde_problem *p, void *psi, double dt, int64_t nsteps, int64_t
         q.nsteps = nsteps;
         q.step0 = step0;
         q.Etab = static_cast<const V *>(p->d_E[0]);
+        q.Ex = p->E_x[0];
         const bool shape0 = p->scheme != XSDE_SCHEME_RK4IP || p->nonlocal || g.basis[0] != XSDE_BASIS_FOURIER;
-        const int elems = shape0 ? 8 : rk4ip_1d_elems(p->kernel_variant);
+        int variant = p->kernel_variant;
+        if (variant == 0 && !shape0) variant = rk4ip_1d_default(sizeof(R) == 8, g.n[0], npaths, p->num_sms);
+        const int elems = shape0 ? 8 : rk4ip_1d_elems(variant);
         q.tw = static_cast<const tw_t<R> *>(elems == 8 ? p->d_tw[0] : p->d_tw1d[elems == 4 ? 0 : 1]);
         q.lt = lt;
         q.sm = sm;
@@ -1024,7 +1083,7 @@ int run_integrate(xsde_problem *p, void *psi, double dt, int64_t nsteps, int64_t
         q.knl = p->nonlocal ? static_cast<const V *>(p->d_knl) : nullptr;
         q.basis = g.basis[0];
         q.Btab = static_cast<const V *>(p->d_B);
-        XSDE_CUDA(timed(p, 1, s, [&] { return launch_rk4ip_1d<R>(g.n[0], p->kernel_variant, q, s); }),
+        XSDE_CUDA(timed(p, 1, s, [&] { return launch_rk4ip_1d<R>(g.n[0], variant, q, s); }),
                   "rk4ip_1d launch");
         return XSDE_OK;
     }
@@ -1042,6 +1101,8 @@ int run_integrate(xsde_problem *p, void *psi, double dt, int64_t nsteps, int64_t
     q.tw1 = static_cast<const tw_t<R> *>(p->d_tw[1]);
     q.E0 = static_cast<const V *>(p->d_E[0]);
     q.E1 = static_cast<const V *>(p->d_E[1]);
+    q.E0x = p->E_x[0];
+    q.E1x = p->E_x[1];
     q.lt = lt;
     q.sm = sm;
     q.status = p->d_status;
@@ -1349,6 +1410,7 @@ void xsde_problem_destroy(xsde_problem *p) {
     cudaFree(p->d_tw1d[1]);
     for (int d = 0; d < 3; ++d) cudaFree(p->d_tw2[d]);
     cudaFree(p->d_twp);
+    cudaFree(p->d_tw64);
     cudaFree(p->d_knl);
     cudaFree(p->d_B);
     cudaFree(p->d_B1);
@@ -1639,12 +1701,11 @@ int xsde_adjoint(xsde_problem *p, const xsde_vector *psi0, const xsde_vector *ta
         q.nsteps = nsteps;
         q.K = K;
         q.Etab = static_cast<const V *>(p->d_E[0]);
-        // the problem's points-per-thread shape (the 2-point shape runs as 4);
-        // at the default variant, fewer paths than SMs (one CTA per path, each
-        // step a chain of dependent transforms) spread a path over 4 points per
-        // thread, twice the threads of the 8-point shape
-        int elems = rk4ip_1d_elems(p->kernel_variant) == 8 ? 8 : 4;
-        if (p->kernel_variant == 0 && npaths < p->num_sms) elems = 4;
+        q.Ex = p->E_x[0];
+        // 4 points a thread unless the problem's variant asks for an 8-point shape.
+        // Measured (1024 points, ms a 100-step gradient, 4 / 8 points): complex64
+        // 1 path 1.33 / 2.06, 304 paths 2.16 / 2.87; complex128 11.0 / 18.3, 12.6 / 22.0
+        const int elems = p->kernel_variant == 0 || rk4ip_1d_elems(p->kernel_variant) != 8 ? 4 : 8;
         q.tw = static_cast<const tw_t<R> *>(elems == 8 ? p->d_tw[0] : p->d_tw1d[0]);
         q.dx = grid_dx(g, 0);
         q.ckpt = static_cast<V *>(p->d_adj);
@@ -1704,7 +1765,17 @@ int xsde_integrate_adaptive(xsde_problem *p, xsde_vector *psi, const xsde_adapti
         q.psi = static_cast<V *>(psi->data);
         q.npaths = npaths;
         const int elems = ark45_1d_elems(n);
-        q.tw = static_cast<const tw_t<R> *>(elems == 8 ? p->d_tw[0] : p->d_tw1d[elems == 4 ? 0 : 1]);
+        if constexpr (std::is_same<R, double>::value) {
+            if (!p->d_tw64) {   // FP64 twiddles of this launch shape's plan: lattice only, filled once
+                rc = elems == 8   ? upload_twiddles<double, 8, false, double2>(n, &p->d_tw64, s)
+                     : elems == 4 ? upload_twiddles<double, 4, false, double2>(n, &p->d_tw64, s)
+                                  : upload_twiddles<double, 2, false, double2>(n, &p->d_tw64, s);
+                if (rc != XSDE_OK) return rc;
+            }
+            q.tw = static_cast<const double2 *>(p->d_tw64);
+        } else {
+            q.tw = static_cast<const tw_plain_t<R> *>(elems == 8 ? p->d_tw[0] : p->d_tw1d[elems == 4 ? 0 : 1]);
+        }
         q.kbuf = static_cast<V *>(p->d_scratch);
         q.c0_re = p->L.c0_re;
         q.c0_im = p->L.c0_im;
@@ -2253,6 +2324,7 @@ int static_integrate(xsde_problem *p, void *psi, double dt, int64_t nsteps, int6
     const std::complex<double> c0(p->L.c0_re, p->L.c0_im), c2(p->L.c2_re, p->L.c2_im);
     // tables into the host staging area, same layouts as the problem's own tables
     unsigned char *hdim[2] = {t_host_tables, t_host_tables + kStaticTwBytes + kStaticEBytes};
+    int fex[2];
     for (int d = 0; d < 2; ++d) {
         const int n = g.n[d];
         tw_t<R> *tw = reinterpret_cast<tw_t<R> *>(hdim[d]);
@@ -2270,13 +2342,14 @@ int static_integrate(xsde_problem *p, void *psi, double dt, int64_t nsteps, int6
             }
             ns *= rad;
         }
+        thread_local std::vector<std::complex<double>> f;   // grows to the longest dimension once
+        f.resize(n);
         for (int i = 0; i < n; ++i) {
             const double k = kval(g, d, i);
-            const std::complex<double> v =
-                d == 0 ? std::exp((c0 + c2 * (k * k)) * (0.5 * dt)) / ((double)g.n[0] * g.n[1])
-                       : std::exp(c2 * (k * k) * (0.5 * dt));
-            split_hi_lo(v, &e[i], &e[n + i]);
+            f[i] = d == 0 ? std::exp((c0 + c2 * (k * k)) * (0.5 * dt)) / ((double)g.n[0] * g.n[1])
+                          : std::exp(c2 * (k * k) * (0.5 * dt));
         }
+        fill_factors(f, e, &fex[d]);
     }
     XSDE_CUDA(cudaMemcpyAsync(sa.tables, t_host_tables, kStaticTableBytes, cudaMemcpyHostToDevice, s),
               "xsde_integrate_static_scratch: tables");
@@ -2304,6 +2377,8 @@ int static_integrate(xsde_problem *p, void *psi, double dt, int64_t nsteps, int6
     q.E0 = reinterpret_cast<const V *>(sa.tables + kStaticTwBytes);
     q.tw1 = reinterpret_cast<const tw_t<R> *>(sa.tables + kStaticTwBytes + kStaticEBytes);
     q.E1 = reinterpret_cast<const V *>(sa.tables + 2 * kStaticTwBytes + kStaticEBytes);
+    q.E0x = fex[0];
+    q.E1x = fex[1];
     q.lt = lt;
     q.sm = sm;
     q.status = p->d_status;

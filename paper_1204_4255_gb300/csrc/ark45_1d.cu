@@ -20,7 +20,10 @@
 // f5 and e in registers, the six stage derivatives live in a global workspace
 // that only the owning thread reads back (no synchronisation), and every
 // transform runs through shared memory as in rk4ip_1d.cu.  The propagator
-// factors exp(L(k) tau) are evaluated per step and node in FP64.
+// factors exp(L(k) tau) are evaluated per step and node in FP64.  The complex128
+// transforms stay on the FP64 pipe: explicit steps run at their stability bound,
+// where accept / reject follows the last bits of the error estimate, and a
+// fixed-point line (fx.cuh) would part from the FP64 step sequence sooner.
 #include "fft.cuh"
 #include "kernels.h"
 
@@ -76,12 +79,12 @@ __global__ void __launch_bounds__(N / E) ark45_1d_kernel(const AdaptiveParams<R>
     constexpr int T = N / E;
     constexpr int BUF = line_len<V, N>();
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    tw_t<R> *tws = reinterpret_cast<tw_t<R> *>(smem_raw);
+    tw_plain_t<R> *tws = reinterpret_cast<tw_plain_t<R> *>(smem_raw);
     V *buf = reinterpret_cast<V *>(tws + N);
     double *red = reinterpret_cast<double *>(buf + BUF);   // 64 doubles
     V *const sm1[1] = {buf};
     const SyncBlock sync{};
-    const TwiddleTable<tw_t<R>> tw{tws};
+    const TwiddleTable<tw_plain_t<R>> tw{tws};
     const LineLayout<V> L{};
     const int t = threadIdx.x;
     const int64_t path = blockIdx.x;
@@ -234,7 +237,7 @@ __global__ void __launch_bounds__(N / E) ark45_1d_kernel(const AdaptiveParams<R>
 
 template <typename R, int N> cudaError_t ark_launch(const AdaptiveParams<R> &p, cudaStream_t s) {
     constexpr int E = N >= 256 ? 8 : (N == 128 ? 4 : 2), T = N / E;
-    const size_t smem = (size_t)N * sizeof(tw_t<R>) + (size_t)line_len<cx<R>, N>() * sizeof(cx<R>) + 64 * sizeof(double);
+    const size_t smem = (size_t)N * sizeof(tw_plain_t<R>) + (size_t)line_len<cx<R>, N>() * sizeof(cx<R>) + 64 * sizeof(double);
     auto kern = ark45_1d_kernel<R, N, E>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -244,7 +247,9 @@ template <typename R, int N> cudaError_t ark_launch(const AdaptiveParams<R> &p, 
 
 }  // namespace
 
+#if !defined(XSDE_REAL_BITS) || XSDE_REAL_BITS == 32
 int ark45_1d_elems(int n) { return n >= 256 ? 8 : (n == 128 ? 4 : 2); }
+#endif
 
 template <typename R> cudaError_t launch_ark45_1d(int n, const AdaptiveParams<R> &p, cudaStream_t s) {
     switch (n) {
@@ -258,7 +263,12 @@ template <typename R> cudaError_t launch_ark45_1d(int n, const AdaptiveParams<R>
     }
 }
 
+// XSDE_REAL_BITS selects one precision per translation unit (parallel builds)
+#if !defined(XSDE_REAL_BITS) || XSDE_REAL_BITS == 32
 template cudaError_t launch_ark45_1d<float>(int, const AdaptiveParams<float> &, cudaStream_t);
+#endif
+#if !defined(XSDE_REAL_BITS) || XSDE_REAL_BITS == 64
 template cudaError_t launch_ark45_1d<double>(int, const AdaptiveParams<double> &, cudaStream_t);
+#endif
 
 }  // namespace xsde

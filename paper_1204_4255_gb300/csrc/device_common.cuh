@@ -77,8 +77,10 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint2 k) {
 
 // Standard normal pair from the Philox words of counter (point, path, step+1, 0).
 template <typename R> struct BoxMuller;
+// (FP64: a call, for the kernels' code size and registers; its ~75 FP64
+// instructions at 16 clocks each leave nothing to gain from inlining)
 template <> struct BoxMuller<double> {
-    __device__ __forceinline__ static double2 pair(uint32_t x0, uint32_t x1) {
+    __device__ __noinline__ static double2 pair(uint32_t x0, uint32_t x1) {
         const double s = 2.3283064365386963e-10;        // 2^-32
         double u0 = ((double)x0 + 0.5) * s, u1 = ((double)x1 + 0.5) * s;
         double r = sqrt(-2.0 * log(u0));

@@ -20,6 +20,7 @@
 #pragma once
 
 #include "device_common.cuh"
+#include "fx.cuh"
 
 namespace xsde {
 
@@ -103,7 +104,7 @@ template <int R, int S, typename V> __device__ __forceinline__ void dft(V *u) {
 }
 
 // ---------------------------------------------------------------------------
-// Twiddles.  FP64: (cos, sin).  FP32: (cos_hi, sin_hi, cos_lo, sin_lo), the
+// Twiddles.  complex128: Q62 limbs (fx.cuh).  FP32: (cos_hi, sin_hi, cos_lo, sin_lo), the
 // FP64 value split into a rounded pair and its rounded remainder, applied by
 // cmul_hilo so every twiddle acts with ~46-bit accuracy.  (FP32 twiddles alone
 // sit ~1e-8 below unit modulus on average at the angles the early stages use;
@@ -112,8 +113,12 @@ template <int R, int S, typename V> __device__ __forceinline__ void dft(V *u) {
 // ---------------------------------------------------------------------------
 template <typename R> struct tw_of;
 template <> struct tw_of<float> { using type = float4; };
-template <> struct tw_of<double> { using type = double2; };
+template <> struct tw_of<double> { using type = int4; };
 template <typename R> using tw_t = typename tw_of<R>::type;
+// (cos, sin) entries, for complex128 transforms on the FP64 pipe (ark45_1d.cu)
+template <typename R> struct tw_plain_of { using type = tw_t<R>; };
+template <> struct tw_plain_of<double> { using type = double2; };
+template <typename R> using tw_plain_t = typename tw_plain_of<R>::type;
 
 // u * w (S < 0) or u * conj(w) (S > 0)
 template <int S> __device__ __forceinline__ float2 twiddle_mul(float2 u, float4 w) {
@@ -218,6 +223,107 @@ __device__ __forceinline__ void fft(V (&v)[NV][E], int t, V *const (&sm)[NV], co
     static_assert((N & (N - 1)) == 0 && N >= E, "N must be a power of two, at least E");
     static_assert(N % E == 0, "E must divide N");
     fft_from<N, E, S, 1, NV>(v, t, sm, L, sync, tw);
+}
+
+// --- transforms of complex128 lines in fixed point (fx.cuh) -------------------
+// `g` is the line's FxLineGroup / FxColGroup; complex64 ignores it.
+
+// points combined at the stage boundary where a transform looks at its values
+// again: the first with 16 or more (0: below 256 points one scale serves)
+template <int E> __host__ __device__ constexpr int fx_middle(int N) {
+    int ns = 1;
+    while (ns < 16) ns *= stage_radix<E>(N / ns);
+    return N >= 256 ? ns : 0;
+}
+
+template <int N, int E, int S, int Ns, int NV, typename Layout, typename Sync, typename Tw, typename Group>
+__device__ __forceinline__ void fx_fft_from(longlong2 (&q)[NV][E], int (&ex)[NV], const int (&room)[NV], int t,
+                                            longlong2 *const (&sm)[NV], const Layout &L, const Sync &sync, const Tw &tw,
+                                            const Group &g) {
+    constexpr int R = stage_radix<E>(N / Ns);
+    fft_stage<N, E, R, Ns, S, NV>(q, t, tw);
+    if constexpr (Ns * R < N) {
+        if constexpr (Ns * R == fx_middle<E>(N)) fx_refit<N / (Ns * R), NV, E>(q, ex, room, g);
+        fft_exchange<N, E, R, Ns, NV>(q, t, sm, L, sync);
+        fx_fft_from<N, E, S, Ns * R, NV>(q, ex, room, t, sm, L, sync, tw, g);
+    }
+}
+
+// one transform: fft<> for either precision
+template <int N, int E, int S, int NV, typename Layout, typename Sync, typename Tw, typename Group>
+__device__ __forceinline__ void fft_line(float2 (&v)[NV][E], int t, float2 *const (&sm)[NV], const Layout &L,
+                                         const Sync &sync, const Tw &tw, const Group &) {
+    fft<N, E, S, NV>(v, t, sm, L, sync, tw);
+}
+template <int N, int E, int S, int NV, typename Layout, typename Sync, typename Tw, typename Group>
+__device__ __forceinline__ void fft_line(double2 (&v)[NV][E], int t, double2 *const (&sm)[NV], const Layout &L,
+                                         const Sync &sync, const Tw &tw, const Group &g) {
+    longlong2 q[NV][E], *qs[NV];
+    int ex[NV], room[NV];
+#pragma unroll
+    for (int i = 0; i < NV; ++i) qs[i] = reinterpret_cast<longlong2 *>(sm[i]);
+    fx_load<fx_middle<E>(N), NV, E>(v, q, ex, room, g);
+    fx_fft_from<N, E, S, 1, NV>(q, ex, room, t, qs, L, sync, tw, g);
+    fx_store<NV, E>(q, ex, v);
+}
+
+// element m of every vector times factor `at(m)` of the table F (double2 values
+// [n], then their limbs [n], which carry 2^fex)
+template <bool CONJ, int NV, int E, typename At>
+__device__ __forceinline__ void fx_factor(longlong2 (&q)[NV][E], int (&ex)[NV], const double2 *F, int n, int fex,
+                                          const At &at) {
+    const int4 *lim = reinterpret_cast<const int4 *>(F + n);
+#pragma unroll
+    for (int m = 0; m < E; ++m) {
+        const int4 w = __ldg(lim + at(m));
+#pragma unroll
+        for (int i = 0; i < NV; ++i) q[i][m] = twiddle_mul<CONJ ? +1 : -1>(q[i][m], w);
+    }
+#pragma unroll
+    for (int i = 0; i < NV; ++i)
+        if (ex[i] != kFxBad) ex[i] += fex;
+}
+template <bool CONJ, int NV, int E, typename At>
+__device__ __forceinline__ void fx_factor(double2 (&v)[NV][E], const double2 *F, const At &at) {
+#pragma unroll
+    for (int m = 0; m < E; ++m) {
+        const double2 w = __ldg(F + at(m));
+#pragma unroll
+        for (int i = 0; i < NV; ++i) v[i][m] = CONJ ? cmulconj(v[i][m], w) : cmul(v[i][m], w);
+    }
+}
+
+// forward transform, factors F (CONJ: their conjugates), and (BACK) the backward
+// transform, with one conversion in and one out where F has limbs (fex != kFxNone)
+template <int N, int E, bool BACK, bool CONJ, int NV, typename Layout, typename Sync, typename Tw, typename Group>
+__device__ __forceinline__ void fx_propagate(double2 (&v)[NV][E], int t, double2 *const (&sm)[NV], const Layout &L,
+                                             const Sync &sync, const Tw &tw, const Group &g, const double2 *F, int fex) {
+    constexpr int T = N / E, MID = fx_middle<E>(N);
+    auto at = [&](int m) { return t + m * T; };
+    longlong2 q[NV][E], *qs[NV];
+    int ex[NV], room[NV];
+#pragma unroll
+    for (int i = 0; i < NV; ++i) qs[i] = reinterpret_cast<longlong2 *>(sm[i]);
+    fx_load<MID, NV, E>(v, q, ex, room, g);
+    fx_fft_from<N, E, -1, 1, NV>(q, ex, room, t, qs, L, sync, tw, g);
+    if (fex != kFxNone) {
+        if constexpr (BACK) {
+            uint32_t mx[NV];
+            if constexpr (MID > 0) {
+                fx_largest<NV, E>(q, mx);
+                g.max(mx);
+            }
+            fx_fit<MID, NV, E>(q, ex, room, mx, g);
+        }
+        fx_factor<CONJ, NV, E>(q, ex, F, N, fex, at);
+    } else {
+        fx_store<NV, E>(q, ex, v);
+        fx_factor<CONJ, NV, E>(v, F, at);
+        if constexpr (BACK) fx_load<MID, NV, E>(v, q, ex, room, g);
+        else return;
+    }
+    if constexpr (BACK) fx_fft_from<N, E, +1, 1, NV>(q, ex, room, t, qs, L, sync, tw, g);
+    fx_store<NV, E>(q, ex, v);
 }
 
 // --- paired complex64 transforms ---------------------------------------------

@@ -63,7 +63,8 @@ template <typename R> struct Params1D {
     int64_t npaths;
     int64_t nsteps;
     uint64_t step0;        // global index of local step 0
-    const cx<R> *Etab;     // exp(L(k) dt/2)/N in FFT order, hi [N] then lo [N]
+    const cx<R> *Etab;     // exp(L(k) dt/2)/N in FFT order, hi [N] then lo [N] (complex128: limbs [N])
+    int Ex = kFxNone;      // exponent of Etab's limbs
     const tw_t<R> *tw;     // per-stage twiddles of the variant's radix plan [N] (FP32: hi, lo)
     LocalTerm<R> lt;
     Sampling sm;
@@ -85,6 +86,7 @@ int measure_fma_peaks(double *fp32_tflops, double *fp64_tflops);
 cudaError_t launch_wait_timeout(uint64_t wait_ns, int *status, cudaStream_t s);
 int rk4ip_1d_variants();
 int rk4ip_1d_elems(int variant);
+int rk4ip_1d_default(bool fp64, int n, int64_t npaths, int num_sms);
 template <typename R> cudaError_t launch_rk4ip_1d(int n, int variant, const Params1D<R> &p, cudaStream_t s);
 
 // --------------------------------------------------------------------------
@@ -140,8 +142,10 @@ template <typename R> struct Params2D {
     const tw_t<R> *tw0, *tw1; // twiddles per dimension
     // separable exp(L dt/2) = E0(k0) E1(k1), each hi [n] then lo [n]; E0 carries
     // exp(c0 dt/2)/(n0 n1) and is applied by the column pass, E1 by the row
-    // passes whose output feeds a column pass
+    // passes whose output feeds a column pass.  complex128 tables hold the values'
+    // Q62 limbs (fx.cuh) in place of lo; they carry 2^E0x and 2^E1x
     const cx<R> *E0, *E1;
+    int E0x = kFxNone, E1x = kFxNone;
     LocalTerm<R> lt;
     Sampling sm;
     int sample_slot;       // sample written by this pass (-1: none)
@@ -225,7 +229,8 @@ template <typename R> struct AdjParams {
     int64_t npaths;
     int64_t nsteps;
     int64_t K;             // checkpoint interval
-    const cx<R> *Etab;     // hi [N] then lo [N]
+    const cx<R> *Etab;     // hi [N] then lo [N] (complex128: limbs [N])
+    int Ex = kFxNone;      // exponent of Etab's limbs
     const tw_t<R> *tw;
     LocalTerm<R> lt;       // deterministic: noise off
     double dx;
@@ -248,7 +253,7 @@ enum { ST_STEP_LIMIT = 4 };   // a path used up its step attempts
 template <typename R> struct AdaptiveParams {
     cx<R> *psi;            // [npaths][N] real space, in/out
     int64_t npaths;
-    const tw_t<R> *tw;     // per-stage twiddles of the launch shape's radix plan
+    const tw_plain_t<R> *tw;   // per-stage twiddles of the launch shape's radix plan
     cx<R> *kbuf;           // [npaths][6][N] stage derivatives (workspace)
     LocalTerm<R> lt;       // the static potential (noise off)
     double c0_re, c0_im, c2_re, c2_im;   // L(k) = c0 + c2 k^2

@@ -87,6 +87,10 @@ __global__ void __launch_bounds__(PPC *(N / E), MINB) rk4ip_1d_kernel(const Para
     const SlotSync<T, PPC> sync{slot};
     const TwiddleTable<tw_t<R>> tw{tws};
     const LineLayout<V> L{};
+    using Sync = SlotSync<T, PPC>;
+    using Group = FxLineGroup<T, Sync>;
+    V *const bufs_end = reinterpret_cast<V *>(tws + N) + PPC * 2 * BUF;
+    const Group grp{reinterpret_cast<uint32_t *>(bufs_end) + slot * Group::kWords, t, sync};
 
     for (int i = threadIdx.x; i < N; i += blockDim.x) tws[i] = p.tw[i];
     __syncthreads();
@@ -111,7 +115,10 @@ __global__ void __launch_bounds__(PPC *(N / E), MINB) rk4ip_1d_kernel(const Para
     const bool vtime = p.lt.pot == PM_TABLE && p.lt.V_nt > 1;
 
     V x[2][E];
-    V Ek[E], El[E];   // exp(L dt/2)/N (Fourier) or A (TRIG), hi and lo; B is read through L1
+    // exp(L dt/2)/N (Fourier) or A (TRIG), hi and lo; B is read through L1.
+    // (complex128: both are read through L1, as limbs or as FP64 values)
+    constexpr bool FX = sizeof(R) == 8;
+    V Ek[E], El[E];
     R Vs[E];
 #pragma unroll
     for (int m = 0; m < E; ++m) {
@@ -119,8 +126,10 @@ __global__ void __launch_bounds__(PPC *(N / E), MINB) rk4ip_1d_kernel(const Para
         const int pj = point_of(j);
         x[0][m] = (active && XSDE_IN(lp * N + pj, p.npaths * N, p.status)) ? psi[pj] : mk<V>(R(0), R(0));
         if (negated(j)) x[0][m] = mk<V>(-x[0][m].x, -x[0][m].y);
-        Ek[m] = p.Etab[j];
-        El[m] = p.Etab[N + j];
+        if constexpr (!FX) {
+            Ek[m] = p.Etab[j];
+            El[m] = p.Etab[N + j];
+        }
         const int idx[3] = {pj, 0, 0};
         Vs[m] = vtime ? R(0) : potential(p.lt, 1, idx, pj, 0);
     }
@@ -145,7 +154,7 @@ __global__ void __launch_bounds__(PPC *(N / E), MINB) rk4ip_1d_kernel(const Para
             for (int m = 0; m < E; ++m)
 #pragma unroll
                 for (int iv = 0; iv < NV; ++iv)
-                    v[iv][m] = cadd(cmul_hilo(v[iv][m], Ek[m], El[m]),
+                    v[iv][m] = cadd(cmul_hilo(v[iv][m], FX ? __ldg(p.Etab + t + m * T) : Ek[m], El[m]),
                                     cmul_hilo(q[iv][m], __ldg(p.Btab + t + m * T), __ldg(p.Btab + N + t + m * T)));
         } else {
 #pragma unroll
@@ -153,6 +162,21 @@ __global__ void __launch_bounds__(PPC *(N / E), MINB) rk4ip_1d_kernel(const Para
 #pragma unroll
                 for (int iv = 0; iv < NV; ++iv) v[iv][m] = cmul_hilo(v[iv][m], Ek[m], El[m]);
         }
+    };
+    // D = F^-1 exp(L dt/2) F on NV vectors
+    auto propagate = [&](auto &v) {
+        constexpr int NV = sizeof(v) / sizeof(v[0]);
+        auto with = [&](V *const (&sm)[NV]) {
+            if constexpr (FX && !TRIG) {
+                fx_propagate<N, E, true, false, NV>(v, t, sm, L, sync, tw, grp, p.Etab, p.Ex);
+            } else {
+                fft_line<N, E, -1, NV>(v, t, sm, L, sync, tw, grp);
+                kmul(v);
+                fft_line<N, E, +1, NV>(v, t, sm, L, sync, tw, grp);
+            }
+        };
+        if constexpr (NV == 2) with(sm2);
+        else with(sm1);
     };
     const R gdt = p.lt.gdt;
     const R sixth = R(1) / R(6), third = R(1) / R(3), half = R(0.5);
@@ -163,10 +187,10 @@ __global__ void __launch_bounds__(PPC *(N / E), MINB) rk4ip_1d_kernel(const Para
         V y[1][E];
 #pragma unroll
         for (int m = 0; m < E; ++m) y[0][m] = mk<V>(cabs2(u[m]), R(0));
-        fft<N, E, -1, 1>(y, t, sm1, L, sync, tw);
+        fft_line<N, E, -1, 1>(y, t, sm1, L, sync, tw, grp);
 #pragma unroll
         for (int m = 0; m < E; ++m) y[0][m] = cmul(y[0][m], p.knl[t + m * T]);
-        fft<N, E, +1, 1>(y, t, sm1, L, sync, tw);
+        fft_line<N, E, +1, 1>(y, t, sm1, L, sync, tw, grp);
 #pragma unroll
         for (int m = 0; m < E; ++m) vn[m] = y[0][m].x;
     };
@@ -198,7 +222,7 @@ __global__ void __launch_bounds__(PPC *(N / E), MINB) rk4ip_1d_kernel(const Para
             V y[1][E];
 #pragma unroll
             for (int m = 0; m < E; ++m) y[0][m] = x[0][m];
-            fft<N, E, -1, 1>(y, t, sm1, L, sync, tw);
+            fft_line<N, E, -1, 1>(y, t, sm1, L, sync, tw, grp);
             if constexpr (TRIG) {
                 // cosine spectrum X_k from the pair (k, N-k); Parseval weight 2
                 // for every mode but k = 0; sine mode N-1-k sits at k
@@ -262,18 +286,14 @@ __global__ void __launch_bounds__(PPC *(N / E), MINB) rk4ip_1d_kernel(const Para
             V y[1][E];
 #pragma unroll
             for (int m = 0; m < E; ++m) y[0][m] = x[0][m];
-            fft<N, E, -1, 1>(y, t, sm1, L, sync, tw);
-            kmul(y);
-            fft<N, E, +1, 1>(y, t, sm1, L, sync, tw);       // a_I
+            propagate(y);       // a_I
 #pragma unroll
             for (int m = 0; m < E; ++m) {
                 V mid = y[0][m];
                 for (int it = 0; it < 3; ++it) mid = caxpy(y[0][m], half, apply_N(mid, pt[m], gdt));
                 y[0][m] = mk<V>(R(2) * mid.x - y[0][m].x, R(2) * mid.y - y[0][m].y);
             }
-            fft<N, E, -1, 1>(y, t, sm1, L, sync, tw);
-            kmul(y);
-            fft<N, E, +1, 1>(y, t, sm1, L, sync, tw);
+            propagate(y);
 #pragma unroll
             for (int m = 0; m < E; ++m) x[0][m] = y[0][m];
         } else {
@@ -315,9 +335,7 @@ __global__ void __launch_bounds__(PPC *(N / E), MINB) rk4ip_1d_kernel(const Para
                         }
                     }
                 }
-                fft<N, E, -1, 2>(x, t, sm2, L, sync, tw);
-                kmul(x);
-                fft<N, E, +1, 2>(x, t, sm2, L, sync, tw);
+                propagate(x);
             }
             // k4 = N(D(a_I + k3)); a <- D(acc) + k4/6
             if constexpr (NL) nonlocal(x[0], vn);
@@ -340,7 +358,8 @@ __global__ void __launch_bounds__(PPC *(N / E), MINB) rk4ip_1d_kernel(const Para
 template <typename R, int N, int E, int PPC, int SCHEME = 0, bool NL = false, bool TRIG = false, int MINB = 1>
 cudaError_t launch_ppc(const Params1D<R> &p, cudaStream_t s) {
     constexpr int T = N / E;
-    const size_t smem = (size_t)N * sizeof(tw_t<R>) + (size_t)PPC * 2 * line_len<cx<R>, N>() * sizeof(cx<R>);
+    const size_t smem = (size_t)N * sizeof(tw_t<R>) + (size_t)PPC * 2 * line_len<cx<R>, N>() * sizeof(cx<R>) +
+                        (sizeof(R) == 8 ? (size_t)PPC * FxLineGroup<T, SlotSync<T, PPC>>::kWords * 4 : 0);
     const bool noise = p.lt.noise != NM_NONE;
     auto kern = noise ? rk4ip_1d_kernel<R, N, E, PPC, true, SCHEME, NL, TRIG, MINB>
                       : rk4ip_1d_kernel<R, N, E, PPC, false, SCHEME, NL, TRIG, MINB>;
@@ -474,6 +493,19 @@ template <typename R> cudaError_t launch_rk4ip_1d(int n, int variant, const Para
 #if !defined(XSDE_PART) || XSDE_PART == 0
 int rk4ip_1d_variants() { return 7; }
 int rk4ip_1d_elems(int variant) { return variant == 4 ? 4 : variant == 5 ? 2 : 8; }
+// The shape that variant 0 stands for in complex128: few paths are spread over more
+// threads.  Measured (GB300, us a step; 8 points a thread capped at 128 registers /
+// uncapped / 4 points / 2 points):
+//    256 points,    1 path :  41 /  40 /  21 /  11;      4096: 136 / 171 / 126 / 133
+//   1024 points,    1 path :  63 /  61 /  30 /  40;      4096: 600 / 1006 / 841 / 1083
+int rk4ip_1d_default(bool fp64, int n, int64_t npaths, int num_sms) {
+    const int64_t pts = npaths * n;
+    if (fp64) {
+        if (n <= 256) return pts < (int64_t)4096 * num_sms ? 5 : 4;
+        return npaths <= num_sms ? 4 : 6;   // variant 6: capped in complex128
+    }
+    return 0;
+}
 #endif
 XSDE_1D_UNIT(float)
 #endif

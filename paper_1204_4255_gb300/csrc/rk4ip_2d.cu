@@ -57,7 +57,7 @@ template <int N1> struct RowCfg {
 
 // TRIG1: dimension 1 is a cosine or sine dimension (p.basis1), see below
 template <typename R, int N1, int MODE, bool TRIG1 = false>
-__global__ void __launch_bounds__(RowCfg<N1>::THREADS) row_pass_kernel(const Params2D<R> p) {
+__global__ void __launch_bounds__(RowCfg<N1>::THREADS, sizeof(R) == 8 ? 2 : 0) row_pass_kernel(const Params2D<R> p) {
     using V = cx<R>;
     using Cfg = RowCfg<N1>;
     constexpr int E = Cfg::E, T = Cfg::T, LINES = Cfg::LINES;
@@ -72,6 +72,8 @@ __global__ void __launch_bounds__(RowCfg<N1>::THREADS) row_pass_kernel(const Par
     const SyncBlock sync{};
     const TwiddleLdg<tw_t<R>> tw{p.tw1};
     const LineLayout<V> L{};
+    using Group = FxLineGroup<T, SyncBlock>;
+    const Group grp{reinterpret_cast<uint32_t *>(scratch + LINES * (T / 32 + 1) * 2) + line * Group::kWords, t, sync};
 
     const int64_t nrows = p.npaths * (int64_t)p.n0;
     const int64_t row = (int64_t)blockIdx.x * LINES + line;
@@ -107,8 +109,30 @@ __global__ void __launch_bounds__(RowCfg<N1>::THREADS) row_pass_kernel(const Par
     };
     auto store_real = [&](V *f, int sl, V v) { f[pt_of(sl)] = negated(sl) ? mk<V>(-v.x, -v.y) : v; };
 
-    // raw potential of point (line, t + m T) at global step gs
+    // raw potential of point (line, t + m T) at global step gs.  complex128: a
+    // harmonic trap is its line's part, once, plus three FP64 instructions a point
+    // (the FP64 pipe takes 16 clocks a warp instruction, conversions included)
+    R vline = R(0), xfirst = R(0), xstep = R(0), hlast = R(0);
+    if constexpr (sizeof(R) == 8) {
+        if (p.lt.pot == PM_HARMONIC) {
+            const R xa = p.lt.xmin[0] + R(la) * p.lt.dx[0];
+            vline = p.lt.hw2[0] * xa * xa;
+            if (p.ndim == 3) {
+                const R xb = p.lt.xmin[1] + R(lb) * p.lt.dx[1];
+                vline += p.lt.hw2[1] * xb * xb;
+            }
+            xstep = p.ndim == 3 ? p.lt.dx[2] : p.lt.dx[1];
+            hlast = p.ndim == 3 ? p.lt.hw2[2] : p.lt.hw2[1];
+            xfirst = (p.ndim == 3 ? p.lt.xmin[2] : p.lt.xmin[1]) + R(t) * xstep;
+        }
+    }
     auto pot = [&](int m, uint64_t gs) -> R {
+        if constexpr (sizeof(R) == 8 && !TRIG1) {
+            if (p.lt.pot == PM_HARMONIC) {
+                const R x = xfirst + R(m * T) * xstep;
+                return vline + hlast * x * x;
+            }
+        }
         const int ic = pt_of(t + m * T);
         const int idx2[3] = {la, ic, 0};
         const int idx3[3] = {la, lb, ic};
@@ -117,10 +141,14 @@ __global__ void __launch_bounds__(RowCfg<N1>::THREADS) row_pass_kernel(const Par
     // static potentials are evaluated once per element; tables with one row per
     // step are read for the step at hand
     const bool vtime = p.lt.pot == PM_TABLE && p.lt.V_nt > 1;
-    R Vst[E];
+    // (complex128: at each use, for the registers)
+    constexpr bool KEEP_V = sizeof(R) == 4;
+    R Vst[KEEP_V ? E : 1];
+    if constexpr (KEEP_V) {
 #pragma unroll
-    for (int m = 0; m < E; ++m) Vst[m] = vtime ? R(0) : pot(m, 0);
-    auto potv = [&](int m, uint64_t gs) -> R { return vtime ? pot(m, gs) : Vst[m]; };
+        for (int m = 0; m < E; ++m) Vst[m] = vtime ? R(0) : pot(m, 0);
+    }
+    auto potv = [&](int m, uint64_t gs) -> R { return !KEEP_V || vtime ? pot(m, gs) : Vst[m]; };
     auto pterm = [&](int m, uint64_t gs) -> PointTerm<R> {
         const int i1 = pt_of(t + m * T);
         PointTerm<R> pt = point_term(p.lt, potv(m, gs), (uint32_t)(i0 * N1 + i1), gp, (uint32_t)gs);
@@ -175,7 +203,7 @@ __global__ void __launch_bounds__(RowCfg<N1>::THREADS) row_pass_kernel(const Par
                 }
         };
         if (op == SI_ENTER) {
-            fft<N1, E, -1, 1>(y, t, sm1, L, sync, tw);
+            fft_line<N1, E, -1, 1>(y, t, sm1, L, sync, tw, grp);
             const R inv = R(1) / R(N1);
             if (active)
 #pragma unroll
@@ -187,7 +215,7 @@ __global__ void __launch_bounds__(RowCfg<N1>::THREADS) row_pass_kernel(const Par
                 V z[1][E];
 #pragma unroll
                 for (int m = 0; m < E; ++m) z[0][m] = y[0][m];
-                fft<N1, E, +1, 1>(z, t, sm1, L, sync, tw);
+                fft_line<N1, E, +1, 1>(z, t, sm1, L, sync, tw, grp);
                 sample_local(z[0], p.sg);
             }
             // back to the unnormalised F1 a the column pass expects (a power of two: exact)
@@ -196,7 +224,7 @@ __global__ void __launch_bounds__(RowCfg<N1>::THREADS) row_pass_kernel(const Par
             store_scaled(y[0]);
             return;
         }
-        fft<N1, E, +1, 1>(y, t, sm1, L, sync, tw);
+        fft_line<N1, E, +1, 1>(y, t, sm1, L, sync, tw, grp);
         if (op == SI_EXIT) {
             if (sample) sample_local(y[0], p.sg);
             if (active)
@@ -211,8 +239,15 @@ __global__ void __launch_bounds__(RowCfg<N1>::THREADS) row_pass_kernel(const Par
             for (int it = 0; it < 3; ++it) mid = caxpy(y[0][m], half, apply_N(mid, pt, gdt));
             y[0][m] = mk<V>(R(2) * mid.x - y[0][m].x, R(2) * mid.y - y[0][m].y);
         }
-        fft<N1, E, -1, 1>(y, t, sm1, L, sync, tw);
-        store_scaled(y[0]);
+        if constexpr (sizeof(R) == 8) {
+            fx_propagate<N1, E, false, false, 1>(y, t, sm1, L, sync, tw, grp, p.E1, p.E1x);
+            if (active)
+#pragma unroll
+                for (int m = 0; m < E; ++m) Arow[t + m * T] = y[0][m];
+        } else {
+            fft_line<N1, E, -1, 1>(y, t, sm1, L, sync, tw, grp);
+            store_scaled(y[0]);
+        }
         return;
     }
 
@@ -227,7 +262,7 @@ __global__ void __launch_bounds__(RowCfg<N1>::THREADS) row_pass_kernel(const Par
             V y[1][E];
 #pragma unroll
             for (int m = 0; m < E; ++m) y[0][m] = mk<V>(cabs2(u[m]), R(0));
-            fft<N1, E, -1, 1>(y, t, sm1, L, sync, tw);
+            fft_line<N1, E, -1, 1>(y, t, sm1, L, sync, tw, grp);
             if (active)
 #pragma unroll
                 for (int m = 0; m < E; ++m) Crow[t + m * T] = y[0][m];
@@ -237,7 +272,7 @@ __global__ void __launch_bounds__(RowCfg<N1>::THREADS) row_pass_kernel(const Par
             V y[1][E];
 #pragma unroll
             for (int m = 0; m < E; ++m) y[0][m] = Crow[t + m * T];
-            fft<N1, E, +1, 1>(y, t, sm1, L, sync, tw);
+            fft_line<N1, E, +1, 1>(y, t, sm1, L, sync, tw, grp);
 #pragma unroll
             for (int m = 0; m < E; ++m) v[m] = y[0][m].x;
         };
@@ -261,7 +296,7 @@ __global__ void __launch_bounds__(RowCfg<N1>::THREADS) row_pass_kernel(const Par
                 V y[1][E];
 #pragma unroll
                 for (int m = 0; m < E; ++m) y[0][m] = x[0][m];
-                fft<N1, E, -1, 1>(y, t, sm1, L, sync, tw);
+                fft_line<N1, E, -1, 1>(y, t, sm1, L, sync, tw, grp);
                 if (active)
 #pragma unroll
                     for (int m = 0; m < E; ++m) Brow[t + m * T] = y[0][m];
@@ -273,7 +308,7 @@ __global__ void __launch_bounds__(RowCfg<N1>::THREADS) row_pass_kernel(const Par
             V y[1][E];
 #pragma unroll
             for (int m = 0; m < E; ++m) y[0][m] = Arow[t + m * T];
-            fft<N1, E, +1, 1>(y, t, sm1, L, sync, tw);
+            fft_line<N1, E, +1, 1>(y, t, sm1, L, sync, tw, grp);
             density_out(y[0]);
             return;
         } else {
@@ -282,7 +317,7 @@ __global__ void __launch_bounds__(RowCfg<N1>::THREADS) row_pass_kernel(const Par
                 x[0][m] = Arow[t + m * T];
                 x[1][m] = Brow[t + m * T];
             }
-            fft<N1, E, +1, 2>(x, t, sm2, L, sync, tw);
+            fft_line<N1, E, +1, 2>(x, t, sm2, L, sync, tw, grp);
             if (op == NL_S2A) {
                 V u[E];
 #pragma unroll
@@ -330,7 +365,7 @@ __global__ void __launch_bounds__(RowCfg<N1>::THREADS) row_pass_kernel(const Par
             V y[1][E];
 #pragma unroll
             for (int m = 0; m < E; ++m) y[0][m] = x[0][m];
-            fft<N1, E, -1, 1>(y, t, sm1, L, sync, tw);
+            fft_line<N1, E, -1, 1>(y, t, sm1, L, sync, tw, grp);
             if constexpr (TRIG1) {
                 // the cosine spectrum X_k = (w_k V_k + conj(w_k) V_{N1-k}) / 2,
                 // w_k = exp(-i pi k / 2 N1) (for the sine basis, mode N1-k at k)
@@ -365,7 +400,7 @@ __global__ void __launch_bounds__(RowCfg<N1>::THREADS) row_pass_kernel(const Par
             x[0][m] = Arow[t + m * T];
             x[1][m] = Brow[t + m * T];
         }
-        fft<N1, E, +1, 2>(x, t, sm2, L, sync, tw);
+        fft_line<N1, E, +1, 2>(x, t, sm2, L, sync, tw, grp);
         if constexpr (MODE == ROW_STAGE2) {
 #pragma unroll
             for (int m = 0; m < E; ++m) {
@@ -392,7 +427,17 @@ __global__ void __launch_bounds__(RowCfg<N1>::THREADS) row_pass_kernel(const Par
             }
         }
     }
-    fft<N1, E, -1, 2>(x, t, sm2, L, sync, tw);
+    if constexpr (sizeof(R) == 8 && !TRIG1) {
+        fx_propagate<N1, E, false, false, 2>(x, t, sm2, L, sync, tw, grp, p.E1, p.E1x);
+        if (active)
+#pragma unroll
+            for (int m = 0; m < E; ++m) {
+                Arow[t + m * T] = x[0][m];
+                Brow[t + m * T] = x[1][m];
+            }
+        return;
+    }
+    fft_line<N1, E, -1, 2>(x, t, sm2, L, sync, tw, grp);
     // the dimension-1 factor of exp(L dt/2); the column pass applies the rest
     if constexpr (TRIG1) {
         V q[2][E];
@@ -440,11 +485,12 @@ template <typename R, int N0> struct ColCfg {
     // at least one full warp per CTA (the sample reductions use whole-warp shuffles)
     static constexpr int C = (C0 * T < 32) ? 32 / T : C0;
     static constexpr int THREADS = C * T;
+    static constexpr int MINB = sizeof(R) == 8 && THREADS <= 512 ? 512 / THREADS : 0;
     static_assert(THREADS % 32 == 0, "column tiles are whole warps");
 };
 
 template <typename R, int N0, int MODE, bool TRIG = false>
-__global__ void __launch_bounds__(ColCfg<R, N0>::THREADS) col_pass_kernel(const Params2D<R> p) {
+__global__ void __launch_bounds__(ColCfg<R, N0>::THREADS, ColCfg<R, N0>::MINB) col_pass_kernel(const Params2D<R> p) {
     using V = cx<R>;
     using Cfg = ColCfg<R, N0>;
     constexpr int C = Cfg::C, E = Cfg::E, T = Cfg::T;
@@ -458,6 +504,8 @@ __global__ void __launch_bounds__(ColCfg<R, N0>::THREADS) col_pass_kernel(const 
     const SyncBlock sync{};
     const TwiddleLdg<tw_t<R>> tw{p.tw0};
     const ColumnTile<C> L{c};
+    using Group = FxColGroup<C, T>;
+    const Group grp{reinterpret_cast<uint32_t *>(scratch + Cfg::THREADS / 32 + 1), (int)threadIdx.x};
 
     const int col = blockIdx.x * C + c;
     const int64_t path = blockIdx.y;
@@ -566,10 +614,10 @@ __global__ void __launch_bounds__(ColCfg<R, N0>::THREADS) col_pass_kernel(const 
         V y[1][E];
 #pragma unroll
         for (int m = 0; m < E; ++m) y[0][m] = p.C[base + (int64_t)(t + m * T) * n1];
-        fft<N0, E, -1, 1>(y, t, sm1, L, sync, tw);
+        fft_line<N0, E, -1, 1>(y, t, sm1, L, sync, tw, grp);
 #pragma unroll
         for (int m = 0; m < E; ++m) y[0][m] = cmul(y[0][m], __ldg(p.K2 + (int64_t)(t + m * T) * n1 + col));
-        fft<N0, E, +1, 1>(y, t, sm1, L, sync, tw);
+        fft_line<N0, E, +1, 1>(y, t, sm1, L, sync, tw, grp);
 #pragma unroll
         for (int m = 0; m < E; ++m) p.C[base + (int64_t)(t + m * T) * n1] = y[0][m];
         return;
@@ -577,13 +625,17 @@ __global__ void __launch_bounds__(ColCfg<R, N0>::THREADS) col_pass_kernel(const 
         V y[1][E];
 #pragma unroll
         for (int m = 0; m < E; ++m) y[0][m] = load(p.A, t + m * T);
-        fft<N0, E, -1, 1>(y, t, sm1, L, sync, tw);
+        if constexpr (sizeof(R) == 8) {
+            fx_propagate<N0, E, true, false, 1>(y, t, sm1, L, sync, tw, grp, p.E0, p.E0x);
+        } else {
+            fft_line<N0, E, -1, 1>(y, t, sm1, L, sync, tw, grp);
 #pragma unroll
-        for (int m = 0; m < E; ++m) {
-            const V eh = __ldg(p.E0 + t + m * T), el = __ldg(p.E0 + N0 + t + m * T);
-            y[0][m] = cmul_hilo(y[0][m], eh, el);
+            for (int m = 0; m < E; ++m) {
+                const V eh = __ldg(p.E0 + t + m * T), el = __ldg(p.E0 + N0 + t + m * T);
+                y[0][m] = cmul_hilo(y[0][m], eh, el);
+            }
+            fft_line<N0, E, +1, 1>(y, t, sm1, L, sync, tw, grp);
         }
-        fft<N0, E, +1, 1>(y, t, sm1, L, sync, tw);
 #pragma unroll
         for (int m = 0; m < E; ++m) store(p.A, t + m * T, y[0][m]);
         return;
@@ -591,7 +643,7 @@ __global__ void __launch_bounds__(ColCfg<R, N0>::THREADS) col_pass_kernel(const 
         V y[1][E];
 #pragma unroll
         for (int m = 0; m < E; ++m) y[0][m] = load(p.B, t + m * T);
-        fft<N0, E, MODE == COL_FFT_BWD ? +1 : -1, 1>(y, t, sm1, L, sync, tw);
+        fft_line<N0, E, MODE == COL_FFT_BWD ? +1 : -1, 1>(y, t, sm1, L, sync, tw, grp);
         if constexpr (MODE == COL_SPECTRAL) {
             V yq[1][E];
             if constexpr (TRIG) partners(y, yq);
@@ -623,7 +675,20 @@ __global__ void __launch_bounds__(ColCfg<R, N0>::THREADS) col_pass_kernel(const 
             x[0][m] = load(p.A, t + m * T);
             x[1][m] = load(p.B, t + m * T);
         }
-        fft<N0, E, -1, 2>(x, t, sm2, L, sync, tw);
+        // complex128: a pass that takes no sample stays in fixed point between
+        // the two transforms
+        if constexpr (sizeof(R) == 8 && !TRIG) {
+            if (!sample) {
+                fx_propagate<N0, E, true, false, 2>(x, t, sm2, L, sync, tw, grp, p.E0, p.E0x);
+#pragma unroll
+                for (int m = 0; m < E; ++m) {
+                    store(p.A, t + m * T, x[0][m]);
+                    store(p.B, t + m * T, x[1][m]);
+                }
+                return;
+            }
+        }
+        fft_line<N0, E, -1, 2>(x, t, sm2, L, sync, tw, grp);
         V xq[2][E];
         if constexpr (TRIG) partners(x, xq);
         if (sample) kinetic(x[0], xq[0]);
@@ -639,7 +704,7 @@ __global__ void __launch_bounds__(ColCfg<R, N0>::THREADS) col_pass_kernel(const 
                 x[1][m] = cmul_hilo(x[1][m], eh, el);
             }
         }
-        fft<N0, E, +1, 2>(x, t, sm2, L, sync, tw);
+        fft_line<N0, E, +1, 2>(x, t, sm2, L, sync, tw, grp);
 #pragma unroll
         for (int m = 0; m < E; ++m) {
             store(p.A, t + m * T, x[0][m]);
@@ -651,7 +716,8 @@ __global__ void __launch_bounds__(ColCfg<R, N0>::THREADS) col_pass_kernel(const 
 template <typename R, int N1, int MODE> cudaError_t row_launch(const Params2D<R> &p, cudaStream_t s) {
     using Cfg = RowCfg<N1>;
     const size_t smem = (size_t)Cfg::LINES * 2 * line_len<cx<R>, N1>() * sizeof(cx<R>) +
-                        (size_t)Cfg::LINES * (Cfg::T / 32 + 1) * 2 * sizeof(double);
+                        (size_t)Cfg::LINES * (Cfg::T / 32 + 1) * 2 * sizeof(double) +
+                        (sizeof(R) == 8 ? (size_t)Cfg::LINES * FxLineGroup<Cfg::T, SyncBlock>::kWords * 4 : 0);
     auto kern = row_pass_kernel<R, N1, MODE>;
     if constexpr (MODE == ROW_PROLOGUE || MODE == ROW_STAGE2 || MODE == ROW_STEADY || MODE == ROW_EPILOGUE ||
                   MODE == ROW_FFT_ONLY) {
@@ -667,6 +733,22 @@ template <typename R, int N1, int MODE> cudaError_t row_launch(const Params2D<R>
     return cudaGetLastError();
 }
 
+template <typename R, int N0, int MODE> cudaError_t col_launch(const Params2D<R> &p, cudaStream_t s) {
+    using Cfg = ColCfg<R, N0>;
+    const size_t smem = (size_t)2 * N0 * Cfg::C * sizeof(cx<R>) + (Cfg::THREADS / 32 + 1) * sizeof(double) +
+                        (sizeof(R) == 8 ? (size_t)FxColGroup<Cfg::C, Cfg::T>::kWords * 4 : 0);
+    auto kern = col_pass_kernel<R, N0, MODE>;
+    if constexpr (MODE != COL_FFT_BWD && MODE != COL_SINGLE && MODE != COL_CONV)
+        if (p.basis0) kern = col_pass_kernel<R, N0, MODE, true>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    dim3 grid((unsigned)(p.n1 / Cfg::C), (unsigned)p.npaths);
+    kern<<<grid, Cfg::THREADS, smem, s>>>(p);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
 template <typename R, int N1> cudaError_t row_mode(int mode, const Params2D<R> &p, cudaStream_t s) {
     switch (mode) {
         case ROW_PROLOGUE: return row_launch<R, N1, ROW_PROLOGUE>(p, s);
@@ -678,19 +760,6 @@ template <typename R, int N1> cudaError_t row_mode(int mode, const Params2D<R> &
         case ROW_NL: return row_launch<R, N1, ROW_NL>(p, s);
         default: return cudaErrorInvalidValue;
     }
-}
-
-template <typename R, int N0, int MODE> cudaError_t col_launch(const Params2D<R> &p, cudaStream_t s) {
-    using Cfg = ColCfg<R, N0>;
-    const size_t smem = (size_t)2 * N0 * Cfg::C * sizeof(cx<R>) + (Cfg::THREADS / 32 + 1) * sizeof(double);
-    auto kern = col_pass_kernel<R, N0, MODE>;
-    if constexpr (MODE != COL_FFT_BWD && MODE != COL_SINGLE && MODE != COL_CONV)
-        if (p.basis0) kern = col_pass_kernel<R, N0, MODE, true>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    dim3 grid((unsigned)(p.n1 / Cfg::C), (unsigned)p.npaths);
-    kern<<<grid, Cfg::THREADS, smem, s>>>(p);
-    return cudaGetLastError();
 }
 
 template <typename R, int N0> cudaError_t col_mode(int mode, const Params2D<R> &p, cudaStream_t s) {
@@ -705,9 +774,6 @@ template <typename R, int N0> cudaError_t col_mode(int mode, const Params2D<R> &
         default: return cudaErrorInvalidValue;
     }
 }
-
-}  // namespace
-
 
 template <typename R> cudaError_t launch_row_pass(int mode, const Params2D<R> &p, cudaStream_t s) {
     switch (p.n1) {
@@ -738,25 +804,37 @@ template <typename R> cudaError_t launch_col_pass(int mode, const Params2D<R> &p
     }
 }
 
-// XSDE_REAL_BITS selects one precision and XSDE_PART the row (0) or column (1)
-// passes per translation unit (parallel builds)
-#if !defined(XSDE_PART) || XSDE_PART == 0
-#define XSDE_2D_ROW(R) template cudaError_t launch_row_pass<R>(int, const Params2D<R> &, cudaStream_t);
+// Parallel builds: XSDE_REAL_BITS selects one precision and XSDE_PART (0..7) one
+// length, 16 << XSDE_PART, per translation unit; part 0 also holds the dispatch,
+// which sees the other lengths as extern instantiations.
+#define XSDE_2D_N(X, R, N)                                                          \
+    X template cudaError_t row_mode<R, N>(int, const Params2D<R> &, cudaStream_t);  \
+    X template cudaError_t col_mode<R, N>(int, const Params2D<R> &, cudaStream_t);
+#if !defined(XSDE_PART)
+#define XSDE_2D_LENGTHS(R)                                                                                    \
+    XSDE_2D_N(, R, 16) XSDE_2D_N(, R, 32) XSDE_2D_N(, R, 64) XSDE_2D_N(, R, 128) XSDE_2D_N(, R, 256)          \
+    XSDE_2D_N(, R, 512) XSDE_2D_N(, R, 1024) XSDE_2D_N(, R, 2048)
+#elif XSDE_PART == 0
+#define XSDE_2D_LENGTHS(R)                                                                                    \
+    XSDE_2D_N(, R, 16) XSDE_2D_N(extern, R, 32) XSDE_2D_N(extern, R, 64) XSDE_2D_N(extern, R, 128)            \
+    XSDE_2D_N(extern, R, 256) XSDE_2D_N(extern, R, 512) XSDE_2D_N(extern, R, 1024) XSDE_2D_N(extern, R, 2048)
 #else
-#define XSDE_2D_ROW(R)
+#define XSDE_2D_LENGTHS(R) XSDE_2D_N(, R, (16 << XSDE_PART))
 #endif
-#if !defined(XSDE_PART) || XSDE_PART == 1
-#define XSDE_2D_COL(R) template cudaError_t launch_col_pass<R>(int, const Params2D<R> &, cudaStream_t);
+#if !defined(XSDE_PART) || XSDE_PART == 0
+#define XSDE_2D_DISPATCH(R)                                                            \
+    template cudaError_t launch_row_pass<R>(int, const Params2D<R> &, cudaStream_t);   \
+    template cudaError_t launch_col_pass<R>(int, const Params2D<R> &, cudaStream_t);
 #else
-#define XSDE_2D_COL(R)
+#define XSDE_2D_DISPATCH(R)
 #endif
 #if !defined(XSDE_REAL_BITS) || XSDE_REAL_BITS == 32
-XSDE_2D_ROW(float)
-XSDE_2D_COL(float)
+XSDE_2D_LENGTHS(float)
+XSDE_2D_DISPATCH(float)
 #endif
 #if !defined(XSDE_REAL_BITS) || XSDE_REAL_BITS == 64
-XSDE_2D_ROW(double)
-XSDE_2D_COL(double)
+XSDE_2D_LENGTHS(double)
+XSDE_2D_DISPATCH(double)
 #endif
 
 }  // namespace xsde

@@ -22,27 +22,30 @@
 //    state.  Stage inputs of all steps are kept ([paths][nsteps][4][N]).
 //  - ADJ_SEQUENTIAL: one launch, one CTA per path, recomputing one segment at a
 //    time into a [paths][K][4][N] buffer (when the full buffer does not fit).
+#include <type_traits>
+
 #include "fft.cuh"
 #include "kernels.h"
 
 namespace xsde {
 namespace {
 
+// The adjoint of N at input u on the cotangent mu, and its V gradient
+// d = Re(conj(-i u) mu) = mu.x u.y - mu.y u.x (per unit dt).  With N = s w, s = dt V +
+// gdt |u|^2, w = -i u: dN = s (-i du) + 2 gdt Re(conj(u) du) w, so the adjoint is
+// i s mu + 2 gdt d u, and d is the gradient's own term: 10 multiply-adds for both,
+// where conj(A) mu + B conj(mu) took 18 (complex128 sits on the FP64 pipe here).
 template <typename R> struct AdjMath {
     using V = cx<R>;
-    // conj(A) mu + B conj(mu) at input u; dtV = dt (V + alpha xi), gdt = dt g
-    __device__ __forceinline__ static V adjN(V u, V mu, R dtV, R gdt) {
-        const R s = dtV + R(2) * gdt * cabs2(u);            // conj(A) = i s
-        const R bx = gdt * R(2) * u.x * u.y;                  // B = gdt (2 ux uy, -(ux^2 - uy^2))
-        const R by = -gdt * (u.x * u.x - u.y * u.y);
-        return mk<V>(-s * mu.y + bx * mu.x + by * mu.y, s * mu.x + by * mu.x - bx * mu.y);
+    __device__ __forceinline__ static V adjN(V u, V mu, R dtV, R gdt, R &d) {
+        d = mu.x * u.y - mu.y * u.x;
+        const R s = dtV + gdt * cabs2(u), k = R(2) * gdt * d;
+        return mk<V>(k * u.x - s * mu.y, k * u.y + s * mu.x);
     }
-    // Re(conj(mu) (-i dt u)) / dt
-    __device__ __forceinline__ static R dv(V mu, V u) { return mu.x * u.y - mu.y * u.x; }
 };
 
 template <typename R, int N, int E>
-__global__ void __launch_bounds__(N / E) rk4ip_adjoint_kernel(const AdjParams<R> p) {
+__global__ void __launch_bounds__(N / E, sizeof(R) == 8 && E == 4 ? 512 / (N / E) : 1) rk4ip_adjoint_kernel(const AdjParams<R> p) {
     using V = cx<R>;
     using M = AdjMath<R>;
     constexpr int T = N / E;
@@ -58,15 +61,17 @@ __global__ void __launch_bounds__(N / E) rk4ip_adjoint_kernel(const AdjParams<R>
     const LineLayout<V> L{};
     const int t = threadIdx.x;
     const int64_t path = blockIdx.x;
+    using Group = FxLineGroup<T, SyncBlock>;
+    const Group grp{reinterpret_cast<uint32_t *>(red + 2 * ((T + 31) / 32)), t, sync};
     if (!XSDE_IN(path, p.npaths, p.status)) return;   // whole CTA: one path each
     const int64_t nck = (p.nsteps + p.K - 1) / p.K;    // checkpoints held by p.ckpt
 
     for (int i = t; i < N; i += blockDim.x) tws[i] = p.tw[i];
     __syncthreads();
 
-    V Ek[E], El[E];
+    V Ek[E], El[E];   // (complex128 reads the table through L1)
 #pragma unroll
-    for (int m = 0; m < E; ++m) {
+    for (int m = 0; m < E && sizeof(R) == 4; ++m) {
         Ek[m] = p.Etab[t + m * T];
         El[m] = p.Etab[N + t + m * T];
     }
@@ -83,19 +88,19 @@ __global__ void __launch_bounds__(N / E) rk4ip_adjoint_kernel(const AdjParams<R>
         return mk<V>(s * u.y, -s * u.x);
     };
     // D (S = -1 then +1 with E) or its adjoint (conj(E)) on both vectors
-    auto Dpair = [&](V (&x)[2][E], bool adjoint) {
-        fft<N, E, -1, 2>(x, t, sm2, L, sync, tw);
+    auto Dpair = [&](V (&x)[2][E], auto adjoint) {
+        constexpr bool CONJ = decltype(adjoint)::value;
+        if constexpr (sizeof(R) == 8) {
+            fx_propagate<N, E, true, CONJ, 2>(x, t, sm2, L, sync, tw, grp, p.Etab, p.Ex);
+        } else {
+            fft<N, E, -1, 2>(x, t, sm2, L, sync, tw);
 #pragma unroll
-        for (int m = 0; m < E; ++m) {
-            if (adjoint) {
-                x[0][m] = cmulconj_hilo(x[0][m], Ek[m], El[m]);
-                x[1][m] = cmulconj_hilo(x[1][m], Ek[m], El[m]);
-            } else {
-                x[0][m] = cmul_hilo(x[0][m], Ek[m], El[m]);
-                x[1][m] = cmul_hilo(x[1][m], Ek[m], El[m]);
-            }
+            for (int m = 0; m < E; ++m)
+#pragma unroll
+                for (int iv = 0; iv < 2; ++iv)
+                    x[iv][m] = CONJ ? cmulconj_hilo(x[iv][m], Ek[m], El[m]) : cmul_hilo(x[iv][m], Ek[m], El[m]);
+            fft<N, E, +1, 2>(x, t, sm2, L, sync, tw);
         }
-        fft<N, E, +1, 2>(x, t, sm2, L, sync, tw);
     };
     const size_t stride = (size_t)p.npaths * N;              // one field of all paths
     const bool full = p.phase != ADJ_SEQUENTIAL;
@@ -111,22 +116,27 @@ __global__ void __launch_bounds__(N / E) rk4ip_adjoint_kernel(const AdjParams<R>
             if (store) interm[(slot * 4 + 0) * N + t + m * T] = x[0][m];
             x[1][m] = nl(x[0][m], dtv[m]);
         }
-        Dpair(x, false);
+        // one copy of the transform pair (rolled): two would not stay in the
+        // instruction cache, and one CTA has few warps to hide its misses
+#pragma unroll 1
+        for (int h = 0; h < 2; ++h) {
+            if (h == 1)
 #pragma unroll
-        for (int m = 0; m < E; ++m) {
-            const V aI = x[0][m], k1 = x[1][m];
-            const V w2 = caxpy(aI, half, k1);
-            const V k2 = nl(w2, dtv[m]);
-            const V w3 = caxpy(aI, half, k2);
-            const V k3 = nl(w3, dtv[m]);
-            if (store) {
-                interm[(slot * 4 + 1) * N + t + m * T] = w2;
-                interm[(slot * 4 + 2) * N + t + m * T] = w3;
-            }
-            x[0][m] = cadd(aI, k3);
-            x[1][m] = caxpy(caxpy(caxpy(aI, sixth, k1), third, k2), third, k3);
+                for (int m = 0; m < E; ++m) {
+                    const V aI = x[0][m], k1 = x[1][m];
+                    const V w2 = caxpy(aI, half, k1);
+                    const V k2 = nl(w2, dtv[m]);
+                    const V w3 = caxpy(aI, half, k2);
+                    const V k3 = nl(w3, dtv[m]);
+                    if (store) {
+                        interm[(slot * 4 + 1) * N + t + m * T] = w2;
+                        interm[(slot * 4 + 2) * N + t + m * T] = w3;
+                    }
+                    x[0][m] = cadd(aI, k3);
+                    x[1][m] = caxpy(caxpy(caxpy(aI, sixth, k1), third, k2), third, k3);
+                }
+            Dpair(x, std::false_type{});
         }
-        Dpair(x, false);
 #pragma unroll
         for (int m = 0; m < E; ++m) {
             if (store) interm[(slot * 4 + 3) * N + t + m * T] = x[0][m];
@@ -235,30 +245,33 @@ __global__ void __launch_bounds__(N / E) rk4ip_adjoint_kernel(const AdjParams<R>
                 const V Du1 = interm[(slot * 4 + 3) * N + t + m * T];
                 const V l4 = cscale(lam[m], sixth);
                 y[0][m] = lam[m];
-                y[1][m] = M::adjN(Du1, l4, dtv[m], gdt);
-                gv[m] = M::dv(l4, Du1);
+                y[1][m] = M::adjN(Du1, l4, dtv[m], gdt, gv[m]);
             }
-            Dpair(y, true);
+#pragma unroll 1
+            for (int h = 0; h < 2; ++h) {
+                if (h == 1)
 #pragma unroll
-            for (int m = 0; m < E; ++m) {
-                const V w2 = (sizeof(R) == 8) ? w2s[m] : interm[(slot * 4 + 1) * N + t + m * T];
-                const V w3 = (sizeof(R) == 8) ? w3s[m] : interm[(slot * 4 + 2) * N + t + m * T];
-                const V la = y[0][m], lu = y[1][m];
-                const V lk3 = caxpy(lu, third, la);
-                const V lw3 = M::adjN(w3, lk3, dtv[m], gdt);
-                gv[m] += M::dv(lk3, w3);
-                const V lk2 = caxpy(cscale(la, third), half, lw3);
-                const V lw2 = M::adjN(w2, lk2, dtv[m], gdt);
-                gv[m] += M::dv(lk2, w2);
-                y[0][m] = caxpy(cscale(la, sixth), half, lw2);        // lambda_k1
-                y[1][m] = cadd(cadd(cadd(la, lu), lw3), lw2);          // lambda_aI
+                    for (int m = 0; m < E; ++m) {
+                        const V w2 = (sizeof(R) == 8) ? w2s[m] : interm[(slot * 4 + 1) * N + t + m * T];
+                        const V w3 = (sizeof(R) == 8) ? w3s[m] : interm[(slot * 4 + 2) * N + t + m * T];
+                        const V la = y[0][m], lu = y[1][m];
+                        R d3, d2;
+                        const V lk3 = caxpy(lu, third, la);
+                        const V lw3 = M::adjN(w3, lk3, dtv[m], gdt, d3);
+                        const V lk2 = caxpy(cscale(la, third), half, lw3);
+                        const V lw2 = M::adjN(w2, lk2, dtv[m], gdt, d2);
+                        gv[m] += d3 + d2;
+                        y[0][m] = caxpy(cscale(la, sixth), half, lw2);        // lambda_k1
+                        y[1][m] = cadd(cadd(cadd(la, lu), lw3), lw2);          // lambda_aI
+                    }
+                Dpair(y, std::true_type{});
             }
-            Dpair(y, true);
 #pragma unroll
             for (int m = 0; m < E; ++m) {
                 const V a = interm[(slot * 4 + 0) * N + t + m * T];
-                lam[m] = cadd(M::adjN(a, y[0][m], dtv[m], gdt), y[1][m]);
-                gv[m] += M::dv(y[0][m], a);
+                R d1;
+                lam[m] = cadd(M::adjN(a, y[0][m], dtv[m], gdt, d1), y[1][m]);
+                gv[m] += d1;
                 atomicAdd(p.dLdV + n * N + t + m * T, (double)(gv[m] * dt));
             }
         }
@@ -272,7 +285,8 @@ __global__ void __launch_bounds__(N / E) rk4ip_adjoint_kernel(const AdjParams<R>
 template <typename R, int N, int E> cudaError_t adj_launch(const AdjParams<R> &p, cudaStream_t s) {
     constexpr int T = N / E;
     const size_t smem = (size_t)N * sizeof(tw_t<R>) + (size_t)2 * line_len<cx<R>, N>() * sizeof(cx<R>) +
-                        (size_t)2 * ((T + 31) / 32) * sizeof(double);
+                        (size_t)2 * ((T + 31) / 32) * sizeof(double) +
+                        (sizeof(R) == 8 ? (size_t)FxLineGroup<T, SyncBlock>::kWords * 4 : 0);
     auto kern = rk4ip_adjoint_kernel<R, N, E>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -283,11 +297,11 @@ template <typename R, int N, int E> cudaError_t adj_launch(const AdjParams<R> &p
     return cudaGetLastError();
 }
 
+}  // namespace
+
 template <typename R, int N> cudaError_t adj_launch_e(int elems, const AdjParams<R> &p, cudaStream_t s) {
     return elems == 4 ? adj_launch<R, N, 4>(p, s) : adj_launch<R, N, 8>(p, s);
 }
-
-}  // namespace
 
 // elems: points per thread, 8 (radix-8 plan) or 4 (radix-4 plan; p.tw must
 // hold that plan's table)
@@ -301,12 +315,29 @@ template <typename R> cudaError_t launch_adjoint_1d(int n, int elems, const AdjP
     }
 }
 
-// XSDE_REAL_BITS selects one precision per translation unit (parallel builds)
+// Parallel builds: XSDE_REAL_BITS selects one precision and XSDE_PART (4..7) one
+// length, 16 << XSDE_PART, per translation unit; part 4 also holds the dispatch.
+#define XSDE_ADJ_N(X, R, N) X template cudaError_t adj_launch_e<R, N>(int, const AdjParams<R> &, cudaStream_t);
+#if !defined(XSDE_PART)
+#define XSDE_ADJ_UNIT(R) XSDE_ADJ_N(, R, 256) XSDE_ADJ_N(, R, 512) XSDE_ADJ_N(, R, 1024) XSDE_ADJ_N(, R, 2048)
+#elif XSDE_PART == 4
+#define XSDE_ADJ_UNIT(R) \
+    XSDE_ADJ_N(, R, 256) XSDE_ADJ_N(extern, R, 512) XSDE_ADJ_N(extern, R, 1024) XSDE_ADJ_N(extern, R, 2048)
+#else
+#define XSDE_ADJ_UNIT(R) XSDE_ADJ_N(, R, (16 << XSDE_PART))
+#endif
+#if !defined(XSDE_PART) || XSDE_PART == 4
+#define XSDE_ADJ_DISPATCH(R) template cudaError_t launch_adjoint_1d<R>(int, int, const AdjParams<R> &, cudaStream_t);
+#else
+#define XSDE_ADJ_DISPATCH(R)
+#endif
 #if !defined(XSDE_REAL_BITS) || XSDE_REAL_BITS == 32
-template cudaError_t launch_adjoint_1d<float>(int, int, const AdjParams<float> &, cudaStream_t);
+XSDE_ADJ_UNIT(float)
+XSDE_ADJ_DISPATCH(float)
 #endif
 #if !defined(XSDE_REAL_BITS) || XSDE_REAL_BITS == 64
-template cudaError_t launch_adjoint_1d<double>(int, int, const AdjParams<double> &, cudaStream_t);
+XSDE_ADJ_UNIT(double)
+XSDE_ADJ_DISPATCH(double)
 #endif
 
 }  // namespace xsde
