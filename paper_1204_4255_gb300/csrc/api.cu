@@ -76,6 +76,8 @@ struct xsde_problem {
     int Ef_x[3] = {kFxNone, kFxNone, kFxNone};   // ... and of d_Ef's
     void *d_scratch = nullptr;
     size_t scratch_bytes = 0;
+    void *d_noise = nullptr;  // a 2D / 3D step's normals between its passes (noise_buffer)
+    size_t noise_bytes = 0;
     int *d_status = nullptr;
     int num_sms = 1;
     int kernel_variant = 0;   // see xsde_set_kernel_variant
@@ -615,6 +617,34 @@ int ensure_scratch(xsde_problem *p, size_t need, cudaStream_t s) {
     return XSDE_OK;
 }
 
+// The buffer of a noisy 2D / 3D RK4IP step's scaled normals (Params2D::Z), grown and
+// never shrunk; nullptr (every pass draws for itself) for other problems, where it
+// cannot be had, or where the stream is being captured and it would have to grow.
+void *noise_buffer(xsde_problem *p, int64_t npaths, cudaStream_t s) {
+    if (p->noise.kind == XSDE_NOISE_NONE || p->scheme != XSDE_SCHEME_RK4IP || p->grid.ndim < 2) return nullptr;
+    const size_t real = elem_bytes(p->dtype) / 2;
+    const size_t need = (size_t)npaths * p->grid.npts * (p->noise.kind == XSDE_NOISE_WIENER_COMPLEX ? 2 * real : real);
+    if (p->noise_bytes >= need) return p->d_noise;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    if (p->d_noise) {
+        if (cudaStreamSynchronize(s) != cudaSuccess) return nullptr;   // the launches report it
+        cudaFree(p->d_noise);
+        p->d_noise = nullptr;
+        p->noise_bytes = 0;
+    }
+    if (cudaMalloc(&p->d_noise, need) != cudaSuccess) {
+        cudaGetLastError();
+        p->d_noise = nullptr;
+        return nullptr;
+    }
+    p->noise_bytes = need;
+    return p->d_noise;
+}
+
 template <typename R>
 int run_si_3d(xsde_problem *p, Params2D<R> &qr, Params2D<R> &q1, Params2D<R> &q0, int64_t nsteps, int64_t npaths,
               uint64_t step0, cudaStream_t s);
@@ -713,6 +743,7 @@ int run_3d(xsde_problem *p, void *psi, int64_t nsteps, int64_t npaths, uint64_t 
     base.sample_slot = -1;
     base.sg = 0;
     base.ndim = 3;
+    base.Z = static_cast<R *>(noise_buffer(p, npaths, s));
     Params2D<R> qr = base, q1 = base, q0 = base;
     qr.npaths = npaths;                       // rows: lines along dimension 2
     qr.n0 = g.n[0] * g.n[1];
@@ -1103,6 +1134,7 @@ int run_integrate(xsde_problem *p, void *psi, double dt, int64_t nsteps, int64_t
     q.E1 = static_cast<const V *>(p->d_E[1]);
     q.E0x = p->E_x[0];
     q.E1x = p->E_x[1];
+    q.Z = static_cast<R *>(noise_buffer(p, npaths, s));
     q.lt = lt;
     q.sm = sm;
     q.status = p->d_status;
@@ -1417,6 +1449,7 @@ void xsde_problem_destroy(xsde_problem *p) {
     cudaFree(p->d_B2);
     for (int d = 0; d < 3; ++d) cudaFree(p->d_Ef[d]);
     cudaFree(p->d_scratch);
+    cudaFree(p->d_noise);
     cudaFree(p->d_adj);
     cudaFree(p->d_status);
     cudaFree(p->d_plain);
@@ -2073,6 +2106,7 @@ int prepare_member(xsde_problem *p, double dt, int64_t npaths, cudaStream_t s) {
     int rc = p->dtype == XSDE_C64 ? ensure_tables<cx<float>>(p, dt, s) : ensure_tables<cx<double>>(p, dt, s);
     if (rc == XSDE_OK && p->grid.ndim >= 2)
         rc = ensure_scratch(p, (size_t)scratch_fields(p) * npaths * p->grid.npts * elem_bytes(p->dtype), s);
+    if (rc == XSDE_OK) noise_buffer(p, npaths, s);
     return rc;
 }
 
@@ -2080,7 +2114,7 @@ int prepare_member(xsde_problem *p, double dt, int64_t npaths, cudaStream_t s) {
 std::vector<uintptr_t> member_signature(const xsde_batch_member &m) {
     const xsde_problem *p = m.prob;
     std::vector<uintptr_t> v = {(uintptr_t)p->generation, (uintptr_t)m.psi->data, (uintptr_t)p->d_scratch,
-                                (uintptr_t)m.psi->npaths, (uintptr_t)m.path_offset};
+                                (uintptr_t)p->d_noise, (uintptr_t)m.psi->npaths, (uintptr_t)m.path_offset};
     for (int d = 0; d < 3; ++d) {
         v.push_back((uintptr_t)p->d_tw[d]);
         v.push_back((uintptr_t)p->d_E[d]);

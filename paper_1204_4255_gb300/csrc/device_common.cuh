@@ -66,44 +66,59 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint2 k) {
 #pragma unroll
     for (int round = 0; round < 10; ++round) {
         const uint32_t m0 = 0xD2511F53u, m1 = 0xCD9E8D57u;
-        uint32_t hi0 = __umulhi(m0, c.x), lo0 = m0 * c.x;
-        uint32_t hi1 = __umulhi(m1, c.z), lo1 = m1 * c.z;
-        c = make_uint4(hi1 ^ c.y ^ k.x, lo1, hi0 ^ c.w ^ k.y, lo0);
+        const uint64_t p0 = (uint64_t)m0 * c.x, p1 = (uint64_t)m1 * c.z;   // one wide multiply each
+        c = make_uint4((uint32_t)(p1 >> 32) ^ c.y ^ k.x, (uint32_t)p1, (uint32_t)(p0 >> 32) ^ c.w ^ k.y, (uint32_t)p0);
         k.x += 0x9E3779B9u;
         k.y += 0xBB67AE85u;
     }
     return c;
 }
 
-// Standard normal pair from the Philox words of counter (point, path, step+1, 0).
+// Standard normal pair from the Philox words of counter (point, path, step+1, 0);
+// first() is the pair's z0 alone (real noise takes no more).
 template <typename R> struct BoxMuller;
 // (FP64: a call, for the kernels' code size and registers; its ~75 FP64
 // instructions at 16 clocks each leave nothing to gain from inlining)
 template <> struct BoxMuller<double> {
+    __device__ __forceinline__ static double uniform(uint32_t x) { return ((double)x + 0.5) * 2.3283064365386963e-10; }
     __device__ __noinline__ static double2 pair(uint32_t x0, uint32_t x1) {
-        const double s = 2.3283064365386963e-10;        // 2^-32
-        double u0 = ((double)x0 + 0.5) * s, u1 = ((double)x1 + 0.5) * s;
-        double r = sqrt(-2.0 * log(u0));
+        const double r = sqrt(-2.0 * log(uniform(x0)));
         double sn, cs;
-        sincospi(2.0 * u1, &sn, &cs);
+        sincospi(2.0 * uniform(x1), &sn, &cs);
         return make_double2(r * cs, r * sn);
+    }
+    __device__ __noinline__ static double first(uint32_t x0, uint32_t x1) {
+        return sqrt(-2.0 * log(uniform(x0))) * cospi(2.0 * uniform(x1));
     }
 };
 template <> struct BoxMuller<float> {
+    __device__ __forceinline__ static float uniform(uint32_t x) {
+        return fmaf(__uint2float_rn(x), 2.3283064365386963e-10f, 1.1641532182693481e-10f);   // 2^-32, 2^-33
+    }
+    // sqrt(-2 ln u), u in [2^-33, 1]: one Newton step s + (x - s^2) / (2 s) on
+    // s = x rsqrt(x), which leaves the last rounding (the square root's call has a
+    // branch that keeps a thread's draws from overlapping)
+    __device__ __forceinline__ static float radius(float u) {
+        const float x = -2.0f * logf(u), i = rsqrtf(fmaxf(x, 1e-30f)), s = x * i;
+        return fmaf(fmaf(-s, s, x), 0.5f * i, s);
+    }
     __device__ __forceinline__ static float2 pair(uint32_t x0, uint32_t x1) {
-        const float s = 2.3283064365386963e-10f, h = 1.1641532182693481e-10f;  // 2^-32, 2^-33
-        float u0 = fmaf(__uint2float_rn(x0), s, h), u1 = fmaf(__uint2float_rn(x1), s, h);
-        float r = sqrtf(-2.0f * logf(u0));
+        const float r = radius(uniform(x0));
         float sn, cs;
-        sincospif(2.0f * u1, &sn, &cs);
+        sincospif(2.0f * uniform(x1), &sn, &cs);
         return make_float2(r * cs, r * sn);
+    }
+    __device__ __forceinline__ static float first(uint32_t x0, uint32_t x1) {
+        return radius(uniform(x0)) * cospif(2.0f * uniform(x1));
     }
 };
 
-template <typename R>
+// (BOTH false: z1 is not formed)
+template <typename R, bool BOTH = true>
 __device__ __forceinline__ cx<R> wiener_pair(uint2 key, uint32_t point, uint32_t path, uint32_t step) {
-    uint4 x = philox4x32_10(make_uint4(point, path, step + 1u, 0u), key);
-    return BoxMuller<R>::pair(x.x, x.y);
+    const uint4 x = philox4x32_10(make_uint4(point, path, step + 1u, 0u), key);
+    if constexpr (BOTH) return BoxMuller<R>::pair(x.x, x.y);
+    else return mk<cx<R>>(BoxMuller<R>::first(x.x, x.y), R(0));
 }
 
 }  // namespace xsde

@@ -189,6 +189,11 @@ template <typename R> struct Params2D {
     const cx<R> *K2 = nullptr;
     int nl_op = 0;
     int nl_last = 0;
+    // the step's scaled normals (load_noise), written by the pass that first draws
+    // them (ROW_PROLOGUE, the second half of ROW_STEADY, NL_PROLOGUE) and read by the
+    // others: a draw costs ~200 instructions and a step's passes take it three or
+    // four times; nullptr: every pass draws
+    R *Z = nullptr;
 };
 template <typename R> cudaError_t launch_row_pass(int mode, const Params2D<R> &p, cudaStream_t s);
 template <typename R> cudaError_t launch_col_pass(int mode, const Params2D<R> &p, cudaStream_t s);
@@ -322,32 +327,89 @@ template <typename R> struct PointTerm {
     cx<R> na;
 };
 
+// The scaled normals of one step, point and path: amplitude * sqrt(dt/dV) (z0, z1),
+// z1 with complex noise only.
+//
+// With substeps S the step's Wiener increment is the sum of those of S
+// steps S times shorter (fine global steps S n .. S n + S - 1): the same
+// Brownian path as a run with dt/S, normalised back to N(0, 1).
+template <typename R>
+static __device__ __noinline__ cx<R> fine_normals(uint2 key, uint32_t j, uint32_t gpath, uint32_t gstep, int substeps) {
+    cx<R> z = mk<cx<R>>(R(0), R(0));
+    for (int i = 0; i < substeps; ++i) {
+        const cx<R> w = wiener_pair<R>(key, j, gpath, gstep * (uint32_t)substeps + (uint32_t)i);
+        z.x += w.x;
+        z.y += w.y;
+    }
+    return cscale(z, R(1) / sqrt(R(substeps)));
+}
+template <typename R, bool BOTH>
+__device__ __forceinline__ cx<R> scaled_normals(const LocalTerm<R> &lt, uint32_t j, uint32_t gpath, uint32_t gstep) {
+    cx<R> z;
+    if (lt.substeps == 1) {
+        z = wiener_pair<R, BOTH>(lt.key, j, gpath, gstep);
+    } else {
+        z = fine_normals<R>(lt.key, j, gpath, gstep, lt.substeps);
+        if (!BOTH) z.y = R(0);
+    }
+    return cscale(z, lt.nscale);
+}
+// those of a thread's E points (point(m)): the usual case without a branch between
+// the points, whose draws then overlap
+template <typename R, int E, typename Point>
+__device__ __forceinline__ void draw_points(const LocalTerm<R> &lt, uint32_t gpath, uint32_t gstep, const Point &point,
+                                            cx<R> (&xi)[E]) {
+    if (lt.substeps == 1 && lt.noise == NM_ADD_COMPLEX) {
+#pragma unroll
+        for (int m = 0; m < E; ++m) xi[m] = cscale(wiener_pair<R, true>(lt.key, point(m), gpath, gstep), lt.nscale);
+    } else if (lt.substeps == 1) {
+#pragma unroll
+        for (int m = 0; m < E; ++m) xi[m] = cscale(wiener_pair<R, false>(lt.key, point(m), gpath, gstep), lt.nscale);
+    } else {
+#pragma unroll
+        for (int m = 0; m < E; ++m) {
+            xi[m] = cscale(fine_normals<R>(lt.key, point(m), gpath, gstep, lt.substeps), lt.nscale);
+            if (lt.noise != NM_ADD_COMPLEX) xi[m].y = R(0);
+        }
+    }
+}
+// the point term of raw potential Vraw with the scaled normals xi, the noise kind at run time
+template <typename R> __device__ __forceinline__ PointTerm<R> noisy_term(const LocalTerm<R> &lt, R Vraw, cx<R> xi) {
+    const bool mul = lt.noise == NM_MUL_REAL;
+    PointTerm<R> pt;
+    pt.dtV = lt.dt * Vraw + (mul ? xi.x : R(0));
+    pt.na = mul ? mk<cx<R>>(R(0), R(0)) : xi;
+    return pt;
+}
+// for a noise kind known at compile time
+template <int NOISE, typename R>
+__device__ __forceinline__ PointTerm<R> point_term(const LocalTerm<R> &lt, R Vraw, cx<R> xi) {
+    PointTerm<R> pt;
+    pt.dtV = lt.dt * Vraw + (NOISE == NM_MUL_REAL ? xi.x : R(0));
+    pt.na = NOISE == NM_ADD_REAL || NOISE == NM_ADD_COMPLEX ? xi : mk<cx<R>>(R(0), R(0));
+    return pt;
+}
+// at run time
+template <typename R>
+__device__ __forceinline__ cx<R> step_noise(const LocalTerm<R> &lt, uint32_t j, uint32_t gpath, uint32_t gstep) {
+    if (lt.noise == NM_NONE) return mk<cx<R>>(R(0), R(0));
+    return lt.noise == NM_ADD_COMPLEX ? scaled_normals<R, true>(lt, j, gpath, gstep)
+                                      : scaled_normals<R, false>(lt, j, gpath, gstep);
+}
 template <typename R>
 __device__ __forceinline__ PointTerm<R> point_term(const LocalTerm<R> &lt, R Vraw, uint32_t j, uint32_t gpath,
                                                    uint32_t gstep) {
-    PointTerm<R> pt;
-    pt.dtV = lt.dt * Vraw;
-    pt.na = mk<cx<R>>(R(0), R(0));
-    if (lt.noise != NM_NONE) {
-        // With substeps S the step's Wiener increment is the sum of those of S
-        // steps S times shorter (fine global steps S n .. S n + S - 1): the same
-        // Brownian path as a run with dt/S, normalised back to N(0, 1).
-        cx<R> z = wiener_pair<R>(lt.key, j, gpath, gstep * (uint32_t)lt.substeps);
-        if (lt.substeps > 1) {
-            for (int i = 1; i < lt.substeps; ++i) {
-                const cx<R> w = wiener_pair<R>(lt.key, j, gpath, gstep * (uint32_t)lt.substeps + (uint32_t)i);
-                z.x += w.x;
-                z.y += w.y;
-            }
-            const R r = R(1) / sqrt(R(lt.substeps));
-            z.x *= r;
-            z.y *= r;
-        }
-        if (lt.noise == NM_MUL_REAL) pt.dtV += lt.nscale * z.x;
-        else if (lt.noise == NM_ADD_REAL) pt.na = mk<cx<R>>(lt.nscale * z.x, R(0));
-        else pt.na = mk<cx<R>>(lt.nscale * z.x, lt.nscale * z.y);
-    }
-    return pt;
+    return noisy_term(lt, Vraw, step_noise<R>(lt, j, gpath, gstep));
+}
+
+// The scaled normals of a 2D / 3D step, kept in memory between its passes:
+// [npaths][npts] values (complex noise: pairs).
+template <typename R> __device__ __forceinline__ cx<R> load_noise(const R *Z, int noise, int64_t i) {
+    return noise == NM_ADD_COMPLEX ? reinterpret_cast<const cx<R> *>(Z)[i] : mk<cx<R>>(Z[i], R(0));
+}
+template <typename R> __device__ __forceinline__ void store_noise(R *Z, int noise, int64_t i, cx<R> xi) {
+    if (noise == NM_ADD_COMPLEX) reinterpret_cast<cx<R> *>(Z)[i] = xi;
+    else Z[i] = xi.x;
 }
 
 // N(u) = dt * (-i (V + alpha xi + g|u|^2) u + sigma xi_a)

@@ -196,10 +196,12 @@ __global__ void __launch_bounds__(PPC *(N / E), MINB) rk4ip_1d_kernel(const Para
     };
     R vn[E];
 
+    int64_t next = p.sm.every > 0 ? 0 : -1, slot_s = 0;   // the next sample's step and index
     for (int64_t n = 0;; ++n) {
         // ---- sampling group (XMDS2 Sec. 2.5 moments over paths) ----------
-        if (p.sm.every > 0 && n % p.sm.every == 0) {
-            const int64_t s = n / p.sm.every;
+        if (n == next) {
+            const int64_t s = slot_s++;
+            next += p.sm.every;
             const uint64_t gs = p.step0 + n;
             double acc[3] = {0.0, 0.0, 0.0};   // norm, local energy, kinetic energy
             if constexpr (NL) nonlocal(x[0], vn);
@@ -267,6 +269,9 @@ __global__ void __launch_bounds__(PPC *(N / E), MINB) rk4ip_1d_kernel(const Para
         const uint64_t sg = p.step0 + n;
         PointTerm<R> pt[E];
         if constexpr (NL) nonlocal(x[0], vn);
+        V xi[NOISE ? E : 1];
+        if constexpr (NOISE)
+            draw_points<R, E>(p.lt, gp, (uint32_t)sg, [&](int m) { return (uint32_t)point_of(t + m * T); }, xi);
 #pragma unroll
         for (int m = 0; m < E; ++m) {
             const int j = t + m * T;
@@ -274,7 +279,7 @@ __global__ void __launch_bounds__(PPC *(N / E), MINB) rk4ip_1d_kernel(const Para
             R v = Vs[m];
             if (vtime) v = XSDE_IN((int64_t)sg * N + pj, p.lt.V_nt * N, p.status) ? p.lt.V[(int64_t)sg * N + pj] : R(0);
             if constexpr (NOISE) {
-                pt[m] = point_term(p.lt, v, (uint32_t)pj, gp, (uint32_t)sg);
+                pt[m] = noisy_term(p.lt, v, xi[m]);
                 if (negated(j)) pt[m].na = mk<V>(-pt[m].na.x, -pt[m].na.y);
             } else {
                 pt[m].dtV = p.lt.dt * v;
@@ -493,18 +498,26 @@ template <typename R> cudaError_t launch_rk4ip_1d(int n, int variant, const Para
 #if !defined(XSDE_PART) || XSDE_PART == 0
 int rk4ip_1d_variants() { return 7; }
 int rk4ip_1d_elems(int variant) { return variant == 4 ? 4 : variant == 5 ? 2 : 8; }
-// The shape that variant 0 stands for in complex128: few paths are spread over more
-// threads.  Measured (GB300, us a step; 8 points a thread capped at 128 registers /
-// uncapped / 4 points / 2 points):
-//    256 points,    1 path :  41 /  40 /  21 /  11;      4096: 136 / 171 / 126 / 133
-//   1024 points,    1 path :  63 /  61 /  30 /  40;      4096: 600 / 1006 / 841 / 1083
+// The shape that variant 0 stands for: few paths are spread over more threads
+// (4 or 2 points each), ensembles keep 8 points a thread.  Measured (GB300, us a
+// step; 8 points capped at 128 registers / uncapped / 4 points / 2 points):
+//   complex64    32 points,  152 paths: 3.28 / 3.02 / 1.57 / 1.14;  4096: 3.30 / 3.01 / 2.34 / 3.05
+//               128 points,  304 paths: 2.75 / 2.79 / 1.56 / 2.23;  4096: 7.66 / 8.08 / 7.31 / 18.1
+//               256 points,  304 paths: 2.69 / 2.73 / 2.01 / 3.32;  1216: 4.27 / 4.07 / 5.06 / 10.6
+//              1024 points,  152 paths: 4.76 / 4.29 / 4.13 / 7.60;   304: 7.24 / 6.35 / 6.87 / 15.2
+//   complex128  256 points,    1 path :  41 /  40 /  21 /  11;      4096: 136 / 171 / 126 / 133
+//              1024 points,    1 path :  63 /  61 /  30 /  40;      4096: 600 / 1006 / 841 / 1083
 int rk4ip_1d_default(bool fp64, int n, int64_t npaths, int num_sms) {
     const int64_t pts = npaths * n;
     if (fp64) {
         if (n <= 256) return pts < (int64_t)4096 * num_sms ? 5 : 4;
         return npaths <= num_sms ? 4 : 6;   // variant 6: capped in complex128
     }
-    return 0;
+    if (n <= 32 && pts <= (int64_t)512 * num_sms) return 5;
+    if (n <= 128) return 4;
+    if (n <= 256) return npaths <= 2 * (int64_t)num_sms ? 4 : 0;
+    if (n <= 1024 && npaths <= num_sms) return 4;
+    return npaths <= 2 * (int64_t)num_sms ? 6 : 0;   // variant 6: uncapped in complex64
 }
 #endif
 XSDE_1D_UNIT(float)

@@ -149,9 +149,20 @@ __global__ void __launch_bounds__(RowCfg<N1>::THREADS, sizeof(R) == 8 ? 2 : 0) r
         for (int m = 0; m < E; ++m) Vst[m] = vtime ? R(0) : pot(m, 0);
     }
     auto potv = [&](int m, uint64_t gs) -> R { return !KEEP_V || vtime ? pot(m, gs) : Vst[m]; };
-    auto pterm = [&](int m, uint64_t gs) -> PointTerm<R> {
+    // first: this pass is the first to use the step's noise, and keeps it
+    auto pterm = [&](int m, uint64_t gs, bool first = false) -> PointTerm<R> {
         const int i1 = pt_of(t + m * T);
-        PointTerm<R> pt = point_term(p.lt, potv(m, gs), (uint32_t)(i0 * N1 + i1), gp, (uint32_t)gs);
+        V xi = mk<V>(R(0), R(0));
+        if (p.lt.noise != NM_NONE) {
+            const int64_t iz = rrow * N1 + i1;
+            if (p.Z && !first) {
+                xi = load_noise(p.Z, p.lt.noise, iz);
+            } else {
+                xi = step_noise<R>(p.lt, (uint32_t)(i0 * N1 + i1), gp, (uint32_t)gs);
+                if (p.Z && active) store_noise(p.Z, p.lt.noise, iz, xi);
+            }
+        }
+        PointTerm<R> pt = noisy_term(p.lt, potv(m, gs), xi);
         if (negated(t + m * T)) pt.na = mk<V>(-pt.na.x, -pt.na.y);
         return pt;
     };
@@ -277,8 +288,8 @@ __global__ void __launch_bounds__(RowCfg<N1>::THREADS, sizeof(R) == 8 ? 2 : 0) r
             for (int m = 0; m < E; ++m) v[m] = y[0][m].x;
         };
         // the point term of step gs with V_nl added to the potential
-        auto ptv = [&](int m, uint64_t gs, R vnl) -> PointTerm<R> {
-            PointTerm<R> pt = pterm(m, gs);
+        auto ptv = [&](int m, uint64_t gs, R vnl, bool first = false) -> PointTerm<R> {
+            PointTerm<R> pt = pterm(m, gs, first);
             pt.dtV += p.lt.dt * vnl;
             return pt;
         };
@@ -303,7 +314,7 @@ __global__ void __launch_bounds__(RowCfg<N1>::THREADS, sizeof(R) == 8 ? 2 : 0) r
                 return;
             }
 #pragma unroll
-            for (int m = 0; m < E; ++m) x[1][m] = apply_N(x[0][m], ptv(m, p.sg, v[m]), gdt);
+            for (int m = 0; m < E; ++m) x[1][m] = apply_N(x[0][m], ptv(m, p.sg, v[m], true), gdt);
         } else if (op == NL_SDA) {
             V y[1][E];
 #pragma unroll
@@ -392,7 +403,7 @@ __global__ void __launch_bounds__(RowCfg<N1>::THREADS, sizeof(R) == 8 ? 2 : 0) r
             return;
         } else {
 #pragma unroll
-            for (int m = 0; m < E; ++m) x[1][m] = apply_N(x[0][m], pterm(m, p.sg), gdt);
+            for (int m = 0; m < E; ++m) x[1][m] = apply_N(x[0][m], pterm(m, p.sg, true), gdt);
         }
     } else {
 #pragma unroll
@@ -423,7 +434,7 @@ __global__ void __launch_bounds__(RowCfg<N1>::THREADS, sizeof(R) == 8 ? 2 : 0) r
             } else {
                 if (sample) sample_local(x[0], p.sg + 1);
 #pragma unroll
-                for (int m = 0; m < E; ++m) x[1][m] = apply_N(x[0][m], pterm(m, p.sg + 1), gdt);
+                for (int m = 0; m < E; ++m) x[1][m] = apply_N(x[0][m], pterm(m, p.sg + 1, true), gdt);
             }
         }
     }

@@ -195,9 +195,22 @@ __global__ void __launch_bounds__(RowTma<N1>::THREADS, 1) row_pass_tma_kernel(co
 #pragma unroll
         for (int m = 0; m < E; ++m) Vst[m] = vtime ? 0.0f : pot(m, 0);
         auto potv = [&](int m, uint64_t gs) -> float { return vtime ? pot(m, gs) : Vst[m]; };
+        // the noise of step sg comes from p.Z (kept by the pass that drew it), read
+        // ahead of the transforms; ROW_STEADY draws and keeps that of step sg + 1
+        V xi[NOISE ? E : 1];
+        auto draw = [&](uint64_t gs) {
+            if constexpr (NOISE)
+                draw_points<float, E>(p.lt, gp, (uint32_t)gs, [&](int m) { return (uint32_t)(i0 * N1 + t + m * T); }, xi);
+        };
+        if constexpr (NOISE) {
+            if (p.Z)
+#pragma unroll
+                for (int m = 0; m < E; ++m) xi[m] = load_noise(p.Z, p.lt.noise, row * N1 + t + m * T);
+            else draw(p.sg);
+        }
         auto pterm = [&](int m, uint64_t gs) -> PointTerm<float> {
             if constexpr (NOISE) {
-                return point_term(p.lt, potv(m, gs), (uint32_t)(i0 * N1 + t + m * T), gp, (uint32_t)gs);
+                return noisy_term(p.lt, potv(m, gs), xi[m]);
             } else {
                 PointTerm<float> pt;
                 pt.dtV = p.lt.dt * potv(m, gs);
@@ -252,6 +265,12 @@ __global__ void __launch_bounds__(RowTma<N1>::THREADS, 1) row_pass_tma_kernel(co
                     }
                     if (!isfinite(acc[0])) atomicOr(p.status, ST_NONFINITE);
                 }
+            }
+            if constexpr (NOISE) {
+                draw(p.sg + 1);
+                if (p.Z)
+#pragma unroll
+                    for (int m = 0; m < E; ++m) store_noise(p.Z, p.lt.noise, row * N1 + t + m * T, xi[m]);
             }
 #pragma unroll
             for (int m = 0; m < E; ++m) x[1][m] = apply_N(x[0][m], pterm(m, p.sg + 1), gdt);
