@@ -560,7 +560,7 @@ bool encode_field_map_warp(CUtensorMap *m, void *base, int64_t rows, int64_t col
 
 // The persistent TMA row pass applies to lines of n1 points when the line
 // count fills whole work items.
-bool tma_rows_ok(int n1, int64_t lines) { return tma_row_supported(n1) && lines % (4096 / n1) == 0; }
+bool tma_rows_ok(int n1, int64_t lines) { return tma_row_supported(n1) && lines % tma_row_lines(n1) == 0; }
 
 // Which complex64 pass runs the hot modes (kernel variant, lattice, alignment):
 // PASS_WARP the warp-synchronous column pass of rk4ip_2d_warp.cu, PASS_TMA the
@@ -810,7 +810,7 @@ int run_3d(xsde_problem *p, void *psi, int64_t nsteps, int64_t npaths, uint64_t 
         qr.sample_slot = slot;
         return timed(p, 2 + mode, s, [&] {
             if constexpr (std::is_same<R, float>::value) {
-                if (rk == PASS_TMA && (mode == ROW_STAGE2 || mode == ROW_STEADY))
+                if (rk == PASS_TMA && mode <= ROW_EPILOGUE)
                     return launch_row_pass_tma(mode, qr, p->num_sms, s);
             }
             return launch_row_pass<R>(mode, qr, s);
@@ -856,6 +856,17 @@ int run_3d(xsde_problem *p, void *psi, int64_t nsteps, int64_t npaths, uint64_t 
     return XSDE_OK;
 }
 
+// A row pass of the semi-implicit schedule, through the TMA row pass where it has
+// the sub-operation
+template <typename R>
+cudaError_t launch_si_row(bool tma, int op, const Params2D<R> &q, int num_sms, cudaStream_t s) {
+    if constexpr (std::is_same<R, float>::value) {
+        const int mode = op == SI_START ? ROW_SI_START : op == SI_STEP ? ROW_SI_STEP : op == SI_EXIT ? ROW_SI_EXIT : -1;
+        if (tma && mode >= 0) return launch_row_pass_tma(mode, q, num_sms, s);
+    }
+    return launch_row_pass<R>(ROW_SI, q, s);
+}
+
 // The semi-implicit step on a 2D lattice (XMDS2 Sec. 2.5's semi-implicit
 // method in the interaction picture of Sec. 2.6).  One field, A, row-transformed
 // between passes (SiOp): a step is one row pass (the three midpoint iterations
@@ -872,16 +883,21 @@ int run_si_2d(xsde_problem *p, Params2D<R> &q, int64_t nsteps, uint64_t step0, c
     const V *E0f = static_cast<const V *>(p->d_Ef[0]), *E1f = static_cast<const V *>(p->d_Ef[1]);
     const int S = q.sm.every;
     auto is_sample = [&](int64_t k) { return S > 0 && k % S == 0; };
+    // complex64 lines of 128..1024 points take the TMA row pass, columns of
+    // 128..512 points the warp (or TMA) column pass, on the one field
+    bool tma_rows = false;
+    if constexpr (std::is_same<R, float>::value) {
+        tma_rows = (uintptr_t)q.A % 16 == 0 && p->d_twp && tma_rows_ok(q.n1, q.npaths * q.n0);
+        q.tw1p = static_cast<const tw_t<R> *>(p->d_twp);
+    }
     auto row = [&](int op, const V *e1, uint64_t sg, int slot) -> cudaError_t {
         q.si_op = op;
         q.E1 = e1;
         q.E1x = (e1 == E1f ? p->Ef_x : p->E_x)[1];
         q.sg = sg;
         q.sample_slot = slot;
-        return timed(p, 4, s, [&] { return launch_row_pass<R>(ROW_SI, q, s); });
+        return timed(p, 4, s, [&] { return launch_si_row<R>(tma_rows, op, q, p->num_sms, s); });
     };
-    // complex64 columns of 128..512 points take the warp (or TMA) column pass
-    // on the one field
     int ck = PASS_GENERIC;
     CUtensorMap mapA, mapA2;
     if constexpr (std::is_same<R, float>::value) {
@@ -915,8 +931,15 @@ int run_si_2d(xsde_problem *p, Params2D<R> &q, int64_t nsteps, uint64_t step0, c
         k.spec_scale = (double)q.n1 * (double)q.n1;
         return timed(p, 8, s, [&] { return launch_col_pass<R>(COL_SPECTRAL, k, s); });
     };
-    XSDE_CUDA(row(SI_ENTER, E1h, step0, -1), "row pass");   // state: F1 a_0 / n1
-    bool at_a = true;                                        // state holds a_k (not D a_k)
+    // straight into step 0 where its state is not sampled: F1 D a_0 / n1
+    const bool start = tma_rows && nsteps > 0 && !is_sample(0);
+    if (start) {
+        XSDE_CUDA(row(SI_START, E1h, step0, -1), "row pass");
+        XSDE_CUDA(col(E0h), "col pass");
+    } else {
+        XSDE_CUDA(row(SI_ENTER, E1h, step0, -1), "row pass");   // state: F1 a_0 / n1
+    }
+    bool at_a = !start;                                      // state holds a_k (not D a_k)
     for (int64_t k = 0; k <= nsteps; ++k) {
         const int slot = is_sample(k) ? (int)(k / S) : -1;
         if (k == nsteps) {
@@ -952,13 +975,41 @@ int run_si_3d(xsde_problem *p, Params2D<R> &qr, Params2D<R> &q1, Params2D<R> &q0
     }
     const int S = qr.sm.every;
     auto is_sample = [&](int64_t k) { return S > 0 && k % S == 0; };
+    // complex64: the TMA rows and warp columns of run_si_2d, where they apply
+    bool tma_rows = false;
+    int ck1 = PASS_GENERIC, ck0 = PASS_GENERIC;
+    CUtensorMap map1, map0, unused;
+    if constexpr (std::is_same<R, float>::value) {
+        if ((uintptr_t)qr.A % 16 == 0) {
+            const xsde_grid &g = p->grid;
+            tma_rows = p->d_twp && tma_rows_ok(qr.n1, qr.npaths * qr.n0);
+            qr.tw1p = static_cast<const tw_t<R> *>(p->d_twp);
+            if (warp_col_supported(q1.n0, q1.n1) && p->d_tw2[1])
+                ck1 = col_maps(PASS_WARP, &map1, &unused, q1.A, q1.A, npaths * g.n[0] * g.n[1], g.n[2], g.n[1]);
+            if (warp_col_supported(q0.n0, q0.n1) && p->d_tw2[0])
+                ck0 = col_maps(PASS_WARP, &map0, &unused, q0.A, q0.A, npaths * g.n[0], (int64_t)g.n[1] * g.n[2], g.n[0]);
+            q1.tw0w = static_cast<const tw_t<R> *>(p->d_tw2[1]);
+            q0.tw0w = static_cast<const tw_t<R> *>(p->d_tw2[0]);
+        }
+    }
+    auto single = [&](Params2D<R> &q, int ck, const CUtensorMap &map) -> cudaError_t {
+        return timed(p, 7, s, [&] {
+            if constexpr (std::is_same<R, float>::value)
+                if (ck == PASS_WARP) {
+                    Params2D<float> t = q;
+                    t.single_field = 1;
+                    return launch_col_pass_warp(t, map, map, p->num_sms, s);
+                }
+            return launch_col_pass<R>(COL_SINGLE, q, s);
+        });
+    };
     auto row = [&](int op, bool whole, uint64_t sg, int slot) -> cudaError_t {
         qr.si_op = op;
         qr.E1 = whole ? Ef[2] : Eh[2];
         qr.E1x = (whole ? p->Ef_x : p->E_x)[2];
         qr.sg = sg;
         qr.sample_slot = slot;
-        return timed(p, 4, s, [&] { return launch_row_pass<R>(ROW_SI, qr, s); });
+        return timed(p, 4, s, [&] { return launch_si_row<R>(tma_rows, op, qr, p->num_sms, s); });
     };
     auto cols = [&](bool whole) -> cudaError_t {
         q1.E0 = whole ? Ef[1] : Eh[1];
@@ -966,9 +1017,8 @@ int run_si_3d(xsde_problem *p, Params2D<R> &qr, Params2D<R> &q1, Params2D<R> &q0
         q1.E0x = (whole ? p->Ef_x : p->E_x)[1];
         q0.E0x = (whole ? p->Ef_x : p->E_x)[0];
         q1.sample_slot = q0.sample_slot = -1;
-        cudaError_t e = timed(p, 7, s, [&] { return launch_col_pass<R>(COL_SINGLE, q1, s); });
-        if (e != cudaSuccess) return e;
-        return timed(p, 7, s, [&] { return launch_col_pass<R>(COL_SINGLE, q0, s); });
+        cudaError_t e = single(q1, ck1, map1);
+        return e == cudaSuccess ? single(q0, ck0, map0) : e;
     };
     auto kinetic = [&](int slot) -> cudaError_t {
         const size_t bytes = (size_t)npaths * p->grid.npts * sizeof(V);
@@ -981,8 +1031,14 @@ int run_si_3d(xsde_problem *p, Params2D<R> &qr, Params2D<R> &q1, Params2D<R> &q0
         k.spec_scale = (double)qr.n1 * (double)qr.n1;
         return timed(p, 8, s, [&] { return launch_col_pass<R>(COL_SPECTRAL, k, s); });
     };
-    XSDE_CUDA(row(SI_ENTER, false, step0, -1), "row pass");
-    bool at_a = true;
+    const bool start = tma_rows && nsteps > 0 && !is_sample(0);   // as run_si_2d
+    if (start) {
+        XSDE_CUDA(row(SI_START, false, step0, -1), "row pass");
+        XSDE_CUDA(cols(false), "col pass");
+    } else {
+        XSDE_CUDA(row(SI_ENTER, false, step0, -1), "row pass");
+    }
+    bool at_a = !start;
     for (int64_t k = 0; k <= nsteps; ++k) {
         const int slot = is_sample(k) ? (int)(k / S) : -1;
         if (k == nsteps) {
@@ -1171,7 +1227,7 @@ int run_integrate(xsde_problem *p, void *psi, double dt, int64_t nsteps, int64_t
         q.sample_slot = slot;
         return timed(p, 2 + mode, s, [&] {
             if constexpr (std::is_same<R, float>::value) {
-                if (rk == PASS_TMA && (mode == ROW_STAGE2 || mode == ROW_STEADY))
+                if (rk == PASS_TMA && mode <= ROW_EPILOGUE)
                     return launch_row_pass_tma(mode, q, p->num_sms, s);
             }
             return launch_row_pass<R>(mode, q, s);

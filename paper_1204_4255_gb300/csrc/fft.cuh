@@ -19,6 +19,8 @@
 // basis of Sec. 2.1, written for sm_103a register files and shared memory.
 #pragma once
 
+#include <type_traits>
+
 #include "device_common.cuh"
 #include "fx.cuh"
 
@@ -167,6 +169,30 @@ template <typename Layout> struct odd_swap_first {
     static constexpr bool value = false;
 };
 
+// Both index patterns are sums of a thread's own part and a compile-time part in
+// other bits, and layouts map such a sum to join(map of the one, the other): one
+// XOR, or an immediate offset, per access.
+template <typename Layout, int NV, typename V> __device__ __forceinline__ void slot_put(V *const (&sm)[NV], int slot, const V (&v)[NV]) {
+    if constexpr (Layout::kPair) {
+        static_assert(NV == 2, "pair slots hold two vectors");
+        reinterpret_cast<float4 *>(sm[0])[slot] = make_float4(v[0].x, v[0].y, v[1].x, v[1].y);
+    } else {
+#pragma unroll
+        for (int iv = 0; iv < NV; ++iv) sm[iv][slot] = v[iv];
+    }
+}
+template <typename Layout, int NV, typename V> __device__ __forceinline__ void slot_get(V *const (&sm)[NV], int slot, V (&v)[NV]) {
+    if constexpr (Layout::kPair) {
+        static_assert(NV == 2, "pair slots hold two vectors");
+        const float4 u = reinterpret_cast<const float4 *>(sm[0])[slot];
+        v[0] = make_float2(u.x, u.y);
+        v[1] = make_float2(u.z, u.w);
+    } else {
+#pragma unroll
+        for (int iv = 0; iv < NV; ++iv) v[iv] = sm[iv][slot];
+    }
+}
+
 template <int N, int E, int R, int Ns, int NV, typename V, typename Layout, typename Sync>
 __device__ __forceinline__ void fft_exchange(V (&v)[NV][E], int t, V *const (&sm)[NV], const Layout &L,
                                              const Sync &sync) {
@@ -180,26 +206,23 @@ __device__ __forceinline__ void fft_exchange(V (&v)[NV][E], int t, V *const (&sm
     for (int q = 0; q < B; ++q) {
         const int j = t + q * T;
         const int k = j & (Ns - 1);
-        const int base = (j - k) * R + k;
+        const int base = (j - k) * R + k, lb = L(base);
 #pragma unroll
         for (int r = 0; r < R; ++r) {
-            if constexpr (swap) {
-                const int slot = L(base + (odd ? (r ^ 1) : r));
+            V u[NV];
 #pragma unroll
-                for (int iv = 0; iv < NV; ++iv) sm[iv][slot] = odd ? v[iv][q + (r ^ 1) * B] : v[iv][q + r * B];
-            } else {
-                const int slot = L(base + r * Ns);
-#pragma unroll
-                for (int iv = 0; iv < NV; ++iv) sm[iv][slot] = v[iv][q + r * B];
-            }
+            for (int iv = 0; iv < NV; ++iv) u[iv] = swap && odd ? v[iv][q + (r ^ 1) * B] : v[iv][q + r * B];
+            slot_put<Layout, NV>(sm, swap ? L(base + (odd ? (r ^ 1) : r)) : L.join(lb, r * Ns), u);
         }
     }
     sync();
+    const int lt = L(t);
 #pragma unroll
     for (int m = 0; m < E; ++m) {
-        const int slot = L(t + m * T);
+        V u[NV];
+        slot_get<Layout, NV>(sm, L.join(lt, m * T), u);
 #pragma unroll
-        for (int iv = 0; iv < NV; ++iv) v[iv][m] = sm[iv][slot];
+        for (int iv = 0; iv < NV; ++iv) v[iv][m] = u[iv];
     }
     sync();
 }
@@ -406,23 +429,26 @@ template <int N, int E, int R, int Ns, int NV, typename V, typename Layout, type
 __device__ __forceinline__ void fft_exchange_back(V (&v)[NV][E], int t, V *const (&sm)[NV], const Layout &L,
                                                   const Sync &sync) {
     constexpr int B = E / R, T = N / E;
+    const int lt = L(t);
 #pragma unroll
     for (int m = 0; m < E; ++m) {
-        const int slot = L(t + m * T);
+        V u[NV];
 #pragma unroll
-        for (int iv = 0; iv < NV; ++iv) sm[iv][slot] = v[iv][m];
+        for (int iv = 0; iv < NV; ++iv) u[iv] = v[iv][m];
+        slot_put<Layout, NV>(sm, L.join(lt, m * T), u);
     }
     sync();
 #pragma unroll
     for (int q = 0; q < B; ++q) {
         const int j = t + q * T;
         const int k = j & (Ns - 1);
-        const int base = (j - k) * R + k;
+        const int lb = L((j - k) * R + k);
 #pragma unroll
         for (int r = 0; r < R; ++r) {
-            const int slot = L(base + r * Ns);
+            V u[NV];
+            slot_get<Layout, NV>(sm, L.join(lb, r * Ns), u);
 #pragma unroll
-            for (int iv = 0; iv < NV; ++iv) v[iv][q + r * B] = sm[iv][slot];
+            for (int iv = 0; iv < NV; ++iv) v[iv][q + r * B] = u[iv];
         }
     }
     sync();
@@ -463,24 +489,53 @@ __device__ __forceinline__ void fftp_bwd(float2 (&v)[NV][E], int t, float2 *cons
 // --- index maps and barriers ------------------------------------------------
 
 // Exchange buffer of one line.  8-byte elements (complex64): rows of 16 slots
-// (128 bytes) whose low four index bits are XOR-ed with (5 x row) mod 16; a
-// wavefront count of every exchange of the radix-2/4/8 plans (16..2048 points,
-// 8/4/2 elements per thread) puts it within 0.2 % of conflict-free, where one
-// pad slot every 8 was 48 % above.  A slot stays in its row, so the buffer
-// holds N slots.  16-byte elements (complex128): one pad slot every 8, already
-// conflict-free for these patterns.
+// (128 bytes) whose low four index bits are XOR-ed with a linear (bitwise XOR)
+// function of the row, so that join() is an XOR with a constant and an immediate
+// offset.  The function comes from a search: conflict-free for every exchange of
+// the radix-2/4/8 plans of 64..2048 points but the 8-element 64-point one (one pad
+// slot every 8 is 48 % above conflict-free, (5 x row) mod 16 12 %).  A slot stays
+// in its row, so the buffer holds N slots.  16-byte elements (complex128): one pad
+// slot every 8, conflict-free for these patterns.
+template <int BIT> __host__ __device__ constexpr int bit_of(int h) { return (h >> BIT) & 1; }
 template <typename V> struct LineLayout {
+    static constexpr bool kPair = false;
+    __host__ __device__ static constexpr int swz(int h) {
+        return (15 * bit_of<0>(h)) ^ (10 * bit_of<1>(h)) ^ (12 * bit_of<2>(h)) ^ (15 * bit_of<3>(h)) ^ (2 * bit_of<4>(h)) ^
+               (13 * bit_of<5>(h)) ^ (2 * bit_of<6>(h));
+    }
     __device__ __forceinline__ int operator()(int i) const {
-        if constexpr (sizeof(V) == 8) return i ^ (((i >> 4) * 5) & 15);
+        if constexpr (sizeof(V) == 8) return i ^ swz(i >> 4);
         else return i + (i >> 3);
     }
+    // the slot of a + c from that of a, for c in bits that a has clear
+    __device__ __forceinline__ int join(int la, int c) const {
+        if constexpr (sizeof(V) == 8) return (la ^ ((c & 15) ^ swz(c >> 4))) + (c & ~15);
+        else return la + c + (c >> 3);
+    }
 };
+// Two complex64 vectors of one line in one buffer of N 16-byte slots (the first
+// vector's buffer, with room for both): half the shared-memory instructions of two
+// buffers.  Rows of 8 slots, the low three index bits XOR-ed as above:
+// conflict-free for the plans of 64..2048 points.
+struct PairLine {
+    static constexpr bool kPair = true;
+    __host__ __device__ static constexpr int swz(int h) {
+        return (7 * bit_of<0>(h)) ^ (5 * bit_of<1>(h)) ^ (6 * bit_of<2>(h)) ^ (3 * bit_of<4>(h)) ^ (6 * bit_of<5>(h)) ^
+               (5 * bit_of<6>(h));
+    }
+    __device__ __forceinline__ int operator()(int i) const { return i ^ swz(i >> 3); }
+    __device__ __forceinline__ int join(int la, int c) const { return (la ^ ((c & 7) ^ swz(c >> 3))) + (c & ~7); }
+};
+// the layout of the NV-vector exchanges of a line
+template <typename V, int NV> using ExchangeLayout = std::conditional_t<sizeof(V) == 8 && NV == 2, PairLine, LineLayout<V>>;
 template <typename V, int N> __host__ __device__ constexpr int line_len() { return sizeof(V) == 8 ? N : N + N / 8; }
 
 // tile of C lines interleaved element by element (slot = i*C + c)
 template <int C> struct ColumnTile {
+    static constexpr bool kPair = false;
     int c;
     __device__ __forceinline__ int operator()(int i) const { return i * C + c; }
+    __device__ __forceinline__ int join(int la, int a) const { return la + a * C; }
 };
 // 8 complex64 columns: a row is 64 B, so two rows an even distance apart share
 // banks, and a half-warp (two threads per column) writing lines R apart conflicts

@@ -186,33 +186,43 @@ __device__ __forceinline__ float2 tw_bwd(float2 x, float4 w) {
     return cmulconj_hilo(x, make_float2(w.x, w.y), make_float2(w.z, w.w));
 }
 
-// Physical row of logical index i during a column exchange: the low three bits
-// are XOR-ed with the three bits above log2(E).  With swizzled tile rows (two
-// or four columns per warp) both the stage-1 writes and the stage-2 reads then
-// spread a column's lanes evenly over the eight 16-byte bank groups.
-template <int E> __device__ __forceinline__ int xslot(int i) { return i ^ ((i >> ilog2c(E)) & 7); }
+// Rows of a column's exchange: the physical row of logical index i is i with the
+// low three bits XOR-ed by the three bits above log2(E).  With swizzled tile rows
+// (two or four columns per warp) both the stage-1 writes and the stage-2 reads then
+// spread a column's lanes evenly over the eight 16-byte bank groups.  Written i = E t
+// + r and read i = t + P m, the row is a lane's own part, one of eight XORs and a
+// constant: `xw(x, r)` and `xr(x, m)` below address (low-bits XOR x, high part).
+template <int N, int E> struct ColumnSlots {
+    static constexpr int P = N / E;
+    // written: row E t + (r ^ (t & 7)) = (E t + (t & 7)) ^ (r & 7) + (r & ~7)
+    __host__ __device__ static constexpr int write_low(int r) { return r & 7; }
+    __host__ __device__ static constexpr int write_high(int r) { return r & ~7; }
+    // read: row (t + P m) ^ c, c = (P m >> log2 E) & 7 (t < P <= E)
+    __host__ __device__ static constexpr int read_low(int m) { return ((P * m) >> ilog2c(E)) & 7; }
+    __host__ __device__ static constexpr int read_high(int m) { return P * m; }
+};
 
 // Twiddle table of the two-stage plan: entry (r - 1) E + j holds w_N^(r j)
 // for r in [1, P), j in [0, E) as (c, s, c eps, s eps) (tw_fwd / tw_bwd).
 template <int N, int E> __host__ __device__ constexpr int warp_fft_table_size() { return (N / E - 1) * E; }
 
 // The forward transform of the line held by this lane's group of P lanes.
-// `xat(i)` is the address of the exchange slot of logical index i (the
-// caller's layout spreads both exchange patterns over the banks); the caller
+// `xw(r)` and `xr(m)` are the addresses of the exchange slots this lane writes
+// (logical index E t + r) and reads (t + P m), see ColumnSlots; the caller
 // has synchronised the warp since the slots were last read.  Ends with a
 // __syncwarp() before the result is in registers, so the slots may be
 // rewritten by the caller.
-template <int N, int E, typename XAt, typename Tw>
-__device__ __forceinline__ void warp_fft(float2 (&x)[E], int t, const XAt &xat, const Tw &tw) {
+template <int N, int E, typename XW, typename XR, typename Tw>
+__device__ __forceinline__ void warp_fft(float2 (&x)[E], int t, const XW &xw, const XR &xr, const Tw &tw) {
     constexpr int P = N / E;
     static_assert(P == 8 || P == 16, "two-stage plan: 8 or 16 lanes per line");
     static_assert(E >= P && E % P == 0, "two-stage plan: E >= P");
     dft_fwd<E>(x);
 #pragma unroll
-    for (int r = 0; r < E; ++r) *xat(E * t + r) = x[r];
+    for (int r = 0; r < E; ++r) *xw(r) = x[r];
     __syncwarp();
 #pragma unroll
-    for (int m = 0; m < E; ++m) x[m] = *xat(t + P * m);
+    for (int m = 0; m < E; ++m) x[m] = *xr(m);
     __syncwarp();
 #pragma unroll
     for (int q = 0; q < E / P; ++q) {
@@ -230,8 +240,8 @@ __device__ __forceinline__ void warp_fft(float2 (&x)[E], int t, const XAt &xat, 
 // N times the inverse of warp_fft<N, E>: stage 2 undone (DFT_P inverted, then
 // the twiddles), the exchange undone, then DFT_E inverted.  Same
 // synchronisation contract as warp_fft.
-template <int N, int E, typename XAt, typename Tw>
-__device__ __forceinline__ void warp_ifft(float2 (&x)[E], int t, const XAt &xat, const Tw &tw) {
+template <int N, int E, typename XW, typename XR, typename Tw>
+__device__ __forceinline__ void warp_ifft(float2 (&x)[E], int t, const XW &xw, const XR &xr, const Tw &tw) {
     constexpr int P = N / E;
     static_assert(P == 8 || P == 16, "two-stage plan: 8 or 16 lanes per line");
 #pragma unroll
@@ -246,10 +256,10 @@ __device__ __forceinline__ void warp_ifft(float2 (&x)[E], int t, const XAt &xat,
         for (int r = 1; r < P; ++r) x[q + (E / P) * r] = tw_bwd(u[r], tw((r - 1) * E + j));
     }
 #pragma unroll
-    for (int m = 0; m < E; ++m) *xat(t + P * m) = x[m];
+    for (int m = 0; m < E; ++m) *xr(m) = x[m];
     __syncwarp();
 #pragma unroll
-    for (int r = 0; r < E; ++r) x[r] = *xat(E * t + r);
+    for (int r = 0; r < E; ++r) x[r] = *xw(r);
     __syncwarp();
     dft_bwd<E>(x);
 }

@@ -100,7 +100,11 @@ enum RowMode {
     ROW_EPILOGUE = 3,   // as STEADY but writes a' in real space to A only
     ROW_FFT_ONLY = 4,   // A (real) -> B = F1 A (for the spectral part of the energy)
     ROW_SI = 5,         // semi-implicit scheme on A alone; sub-operation p.si_op (SiOp)
-    ROW_NL = 6          // RK4IP with a non-local pair potential; sub-operation p.nl_op (NlOp)
+    ROW_NL = 6,         // RK4IP with a non-local pair potential; sub-operation p.nl_op (NlOp)
+    // complex64 TMA row pass: the semi-implicit scheme on A alone
+    ROW_SI_START = 7,   // A (real a) -> E1 F1 a (SI_ENTER and SI_MUL at once)
+    ROW_SI_STEP = 8,    // SI_STEP
+    ROW_SI_EXIT = 9     // SI_EXIT
 };
 // RK4IP steps with a non-local potential V_nl[u] = Re F^-1[khat F |u|^2] on 2D
 // lattices evaluate every N(u) with the V_nl of its own argument, so each
@@ -123,7 +127,8 @@ enum SiOp {
     SI_ENTER = 0,       // A (real a) -> F1 a / n1
     SI_MUL = 1,         // A *= n1 E1 (sampling: the local terms of F1^-1 A first)
     SI_STEP = 2,        // A = F1 a_I / n1 -> a_I; m <- a_I + N(m)/2 three times; A = E1 F1 (2m - a_I) / n1
-    SI_EXIT = 3         // A -> real F1^-1 A (sampling: its local terms)
+    SI_EXIT = 3,        // A -> real F1^-1 A (sampling: its local terms)
+    SI_START = 4        // A (real a) -> E1 F1 a: SI_ENTER and SI_MUL at once (TMA row pass only)
 };
 enum ColMode {
     COL_PROPAGATE = 0,  // A, B -> F0^-1 E0 F0 (A, B)
@@ -207,7 +212,8 @@ constexpr int COL_TMA_C = 8;   // columns per column-pass tile
 bool tma_row_supported(int n1);   // row-pass line length
 bool tma_col_supported(int n0);   // column length
 size_t col_tma_box_rows(int n0);
-cudaError_t launch_row_pass_tma(int mode, const Params2D<float> &p, int grid, cudaStream_t s);
+cudaError_t launch_row_pass_tma(int mode, const Params2D<float> &p, int num_sms, cudaStream_t s);
+int64_t tma_row_lines(int n1);    // the lines of a pass are a multiple of it
 cudaError_t launch_col_pass_tma(const Params2D<float> &p, const CUtensorMap &mapA, const CUtensorMap &mapB, int grid,
                                 cudaStream_t s);
 
@@ -437,6 +443,27 @@ __device__ __forceinline__ R potential(const LocalTerm<R> &lt, int ndim, const i
     }
     return R(0);
 }
+
+// x as FP64 on the integer pipes (a conversion takes the FP64 pipe 16 clocks);
+// denormals become zero
+__device__ __forceinline__ double widen(float x) {
+    const uint32_t b = __float_as_uint(x), e = (b >> 23) & 0xffu;
+    uint32_t hi = ((b & 0x7fffffffu) >> 3) + 0x38000000u;
+    hi = e == 0u ? 0u : e == 255u ? hi | 0x7ff00000u : hi;
+    return __hiloint2double((int)(hi | (b & 0x80000000u)), (int)(e == 0u ? 0u : b << 29));
+}
+__device__ __forceinline__ double widen(double x) { return x; }
+// FP64 sums of a sample's local terms: three FP64 instructions a point
+struct MomentSums {
+    double norm, pot, quart;
+    template <typename R> __device__ __forceinline__ void add(R m2, R v) {
+        const double d = widen(m2);
+        norm += d;
+        pot = fma(widen(v), d, pot);
+        quart = fma(d, d, quart);
+    }
+    __device__ __forceinline__ double energy(double g) const { return pot + 0.5 * g * quart; }
+};
 
 __device__ __forceinline__ double warp_sum(double x) {
 #pragma unroll

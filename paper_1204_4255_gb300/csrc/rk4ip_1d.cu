@@ -166,13 +166,14 @@ __global__ void __launch_bounds__(PPC *(N / E), MINB) rk4ip_1d_kernel(const Para
     // D = F^-1 exp(L dt/2) F on NV vectors
     auto propagate = [&](auto &v) {
         constexpr int NV = sizeof(v) / sizeof(v[0]);
+        const ExchangeLayout<V, NV> X{};
         auto with = [&](V *const (&sm)[NV]) {
             if constexpr (FX && !TRIG) {
-                fx_propagate<N, E, true, false, NV>(v, t, sm, L, sync, tw, grp, p.Etab, p.Ex);
+                fx_propagate<N, E, true, false, NV>(v, t, sm, X, sync, tw, grp, p.Etab, p.Ex);
             } else {
-                fft_line<N, E, -1, NV>(v, t, sm, L, sync, tw, grp);
+                fft_line<N, E, -1, NV>(v, t, sm, X, sync, tw, grp);
                 kmul(v);
-                fft_line<N, E, +1, NV>(v, t, sm, L, sync, tw, grp);
+                fft_line<N, E, +1, NV>(v, t, sm, X, sync, tw, grp);
             }
         };
         if constexpr (NV == 2) with(sm2);

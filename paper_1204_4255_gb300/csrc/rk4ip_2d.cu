@@ -72,6 +72,7 @@ __global__ void __launch_bounds__(RowCfg<N1>::THREADS, sizeof(R) == 8 ? 2 : 0) r
     const SyncBlock sync{};
     const TwiddleLdg<tw_t<R>> tw{p.tw1};
     const LineLayout<V> L{};
+    const ExchangeLayout<V, 2> L2{};
     using Group = FxLineGroup<T, SyncBlock>;
     const Group grp{reinterpret_cast<uint32_t *>(scratch + LINES * (T / 32 + 1) * 2) + line * Group::kWords, t, sync};
 
@@ -328,7 +329,7 @@ __global__ void __launch_bounds__(RowCfg<N1>::THREADS, sizeof(R) == 8 ? 2 : 0) r
                 x[0][m] = Arow[t + m * T];
                 x[1][m] = Brow[t + m * T];
             }
-            fft_line<N1, E, +1, 2>(x, t, sm2, L, sync, tw, grp);
+            fft_line<N1, E, +1, 2>(x, t, sm2, L2, sync, tw, grp);
             if (op == NL_S2A) {
                 V u[E];
 #pragma unroll
@@ -411,7 +412,7 @@ __global__ void __launch_bounds__(RowCfg<N1>::THREADS, sizeof(R) == 8 ? 2 : 0) r
             x[0][m] = Arow[t + m * T];
             x[1][m] = Brow[t + m * T];
         }
-        fft_line<N1, E, +1, 2>(x, t, sm2, L, sync, tw, grp);
+        fft_line<N1, E, +1, 2>(x, t, sm2, L2, sync, tw, grp);
         if constexpr (MODE == ROW_STAGE2) {
 #pragma unroll
             for (int m = 0; m < E; ++m) {
@@ -439,7 +440,7 @@ __global__ void __launch_bounds__(RowCfg<N1>::THREADS, sizeof(R) == 8 ? 2 : 0) r
         }
     }
     if constexpr (sizeof(R) == 8 && !TRIG1) {
-        fx_propagate<N1, E, false, false, 2>(x, t, sm2, L, sync, tw, grp, p.E1, p.E1x);
+        fx_propagate<N1, E, false, false, 2>(x, t, sm2, L2, sync, tw, grp, p.E1, p.E1x);
         if (active)
 #pragma unroll
             for (int m = 0; m < E; ++m) {
@@ -448,7 +449,7 @@ __global__ void __launch_bounds__(RowCfg<N1>::THREADS, sizeof(R) == 8 ? 2 : 0) r
             }
         return;
     }
-    fft_line<N1, E, -1, 2>(x, t, sm2, L, sync, tw, grp);
+    fft_line<N1, E, -1, 2>(x, t, sm2, L2, sync, tw, grp);
     // the dimension-1 factor of exp(L dt/2); the column pass applies the rest
     if constexpr (TRIG1) {
         V q[2][E];

@@ -2,16 +2,16 @@
 //
 // Same arithmetic as rk4ip_2d.cu (XMDS2 Sec. 2.6: exp(L dt/2) in Fourier space,
 // the real-space RK4 stages in between; Sec. 2.2: separable transforms), laid
-// out for sm_103a: one CTA per SM walks a list of 64 KB work items; three
-// shared-memory stages hold the item being transformed and the next two, which
-// the tensor-memory-access unit is already copying in (cp.async.bulk, completion
-// on an mbarrier with a byte count).  Each FFT runs in place in the staged tile
-// and the result leaves through a bulk store, so the SM never waits on a global
-// load while it computes and no register holds data in flight.
-//   row item    : ROWS consecutive lines of A and of B (2 x 32 KB, 1D bulk copies)
+// out for sm_103a: persistent CTAs walk a list of work items; shared-memory stages
+// hold the item being transformed and the next ones, which the
+// tensor-memory-access unit is already copying in (cp.async.bulk, completion
+// on an mbarrier with a byte count), so that no register holds data in flight.
+//   row item    : ROWS lines of A and of B (1D bulk copies, 2 x 8 KB, four CTAs an SM);
+//                 each FFT runs in place in the staged lines, the result leaves
+//                 from registers
 //   column item : an 8-column x n0-row tile of A or of B (32 KB, 2D tensor copies);
 //                 two CTAs per SM, so one CTA's exchanges overlap the other's arithmetic
-// Row exchanges use an XOR swizzle within each line (conflict-free for n1 = 512);
+// Row exchanges swizzle within each line (fft.cuh);
 // column tiles are naturally conflict-free (a half-warp touches two whole 64-byte rows).
 #include <type_traits>
 
@@ -24,13 +24,11 @@ namespace {
 
 using V = float2;
 using TW = float4;
-constexpr int NST = 3;                        // shared-memory stages
+constexpr int NST = 3;                        // shared-memory stages (column pass)
+constexpr int kRowStages = 2;                 // (row pass)
+// fields that a row mode works on
+__host__ __device__ constexpr int row_fields(int mode) { return mode >= ROW_SI_START && mode <= ROW_SI_EXIT ? 1 : 2; }
 constexpr uint64_t kWaitNs = 2000000000ull;    // give up on a copy after 2 s
-
-// slot of element i of a line during row exchanges
-struct SwizzledLine {
-    __device__ __forceinline__ int operator()(int i) const { return i ^ ((i >> 4) & 7) ^ (((i >> 6) & 1) << 3); }
-};
 
 template <int T>
 __device__ __forceinline__ void line_sum2(double (&v)[2], int t, int line, double *scratch) {
@@ -72,24 +70,40 @@ __device__ void give_up(int *status, uint64_t *bars, const uint32_t *parity_next
 // ---------------------------------------------------------------------------
 // Row pass
 // ---------------------------------------------------------------------------
-template <int N1> struct RowTma {
+// FIELDS: those of a work item, A and B or A alone (the semi-implicit modes).  Work
+// items are small and several CTAs share an SM, each with one item in work and one
+// on its way.  What bounds the pass is shared memory (L1/TEX 73 % busy, ~250 bytes a
+// point of a copy engine's writes, exchanges and tables) next to issue (57 %) and
+// DRAM (41 %); small CTAs wait for less at each barrier, spread a small field over
+// the SMs, and leave through the registers.  64 x 512^2: 165 -> 144 us a pass against
+// one CTA an SM with 64 KB items and bulk stores; one 512^2: 14.6 -> 10.1 us; five
+// CTAs (96 registers, tables read through L1) 174 us.
+template <int N1, int FIELDS> struct RowTma {
     static constexpr int E = 8;
     static constexpr int T = N1 / E;
-    static constexpr int ROWS = 4096 / N1;               // 2 x ROWS x N1 x 8 B = 64 KB per item
-    static constexpr int THREADS = ROWS * T;              // 512
-    static constexpr size_t ITEM = (size_t)2 * ROWS * N1 * sizeof(V);
+    static constexpr int THREADS = FIELDS == 2 && N1 <= 512 ? 128 : 256;
+    static constexpr int ROWS = THREADS / T;
+    static constexpr int CTAS_PER_SM = (FIELDS == 2 ? 512 : 768) / THREADS;
+    static constexpr size_t ITEM = (size_t)FIELDS * ROWS * N1 * sizeof(V);
     static constexpr size_t SCRATCH = (size_t)ROWS * (T / 32 + 1) * 2 * sizeof(double);
-    static constexpr size_t SMEM = NST * ITEM + (size_t)N1 * sizeof(TW) + (size_t)2 * N1 * sizeof(V) + SCRATCH +
-                                   NST * sizeof(uint64_t);
+    static constexpr size_t SMEM = kRowStages * ITEM + (size_t)N1 * sizeof(TW) + (size_t)2 * N1 * sizeof(V) + SCRATCH +
+                                   kRowStages * sizeof(uint64_t);
+    static_assert(CTAS_PER_SM * (SMEM + 1024) <= 233472, "shared memory per SM");
 };
 
-// SAMPLE: this pass writes a sample (ROW_STEADY only); NOISE: the problem has
-// Wiener noise.  Both are template flags so the common pass carries neither the
-// sampling code nor the generator.
+// SAMPLE: this pass writes a sample; NOISE: the problem has Wiener noise.  Both
+// are template flags so the common pass carries neither the sampling code nor the
+// generator.
 template <int N1, int MODE, bool SAMPLE, bool NOISE>
-__global__ void __launch_bounds__(RowTma<N1>::THREADS, 1) row_pass_tma_kernel(const Params2D<float> p) {
-    using Cfg = RowTma<N1>;
-    constexpr int E = Cfg::E, T = Cfg::T, ROWS = Cfg::ROWS;
+__global__ void __launch_bounds__(RowTma<N1, row_fields(MODE)>::THREADS, RowTma<N1, row_fields(MODE)>::CTAS_PER_SM)
+    row_pass_tma_kernel(const Params2D<float> p) {
+    constexpr int F = row_fields(MODE);
+    using Cfg = RowTma<N1, F>;
+    constexpr int E = Cfg::E, T = Cfg::T, ROWS = Cfg::ROWS, NST = kRowStages;
+    constexpr bool IN_B = MODE == ROW_STAGE2 || MODE == ROW_STEADY || MODE == ROW_EPILOGUE;   // reads B too
+    constexpr bool OUT_B = F == 2 && MODE != ROW_EPILOGUE;                                    // writes B too
+    constexpr bool REAL_IN = MODE == ROW_PROLOGUE || MODE == ROW_SI_START;
+    constexpr bool REAL_OUT = MODE == ROW_EPILOGUE || MODE == ROW_SI_EXIT;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     V *bufs = reinterpret_cast<V *>(smem_raw);
     TW *tw_s = reinterpret_cast<TW *>(smem_raw + NST * Cfg::ITEM);
@@ -101,12 +115,13 @@ __global__ void __launch_bounds__(RowTma<N1>::THREADS, 1) row_pass_tma_kernel(co
     const int line = tid / T, t = tid - line * T;
     const int64_t nitems = p.npaths * (int64_t)p.n0 / ROWS;
     const int64_t mine = nitems > blockIdx.x ? (nitems - 1 - blockIdx.x) / gridDim.x + 1 : 0;
-    const size_t vec_bytes = (size_t)ROWS * N1 * sizeof(V);
+    constexpr uint32_t line_bytes = (uint32_t)(N1 * sizeof(V)), vec_bytes = ROWS * line_bytes;
 
     // the paired twiddles as (c, s) and (c eps, s eps) halves in tw_s's N1 entries
     float2 *tw_hi = reinterpret_cast<float2 *>(tw_s), *tw_lo = tw_hi + N1;
     stage_paired(tw_hi, tw_lo, p.tw1p, N1, tid, blockDim.x);
-    for (int i = tid; i < 2 * N1; i += blockDim.x) e1_s[i] = p.E1[i];
+    if constexpr (!REAL_OUT)
+        for (int i = tid; i < 2 * N1; i += blockDim.x) e1_s[i] = p.E1[i];
     if (tid == 0) {
         for (int s = 0; s < NST; ++s) mbar_init(bars + s, 1);
         fence_barrier_init();
@@ -119,25 +134,32 @@ __global__ void __launch_bounds__(RowTma<N1>::THREADS, 1) row_pass_tma_kernel(co
     auto issue_load = [&](int64_t k) {   // item k of this CTA into stage k % NST
         const int s = (int)(k % NST);
         const int64_t row0 = (blockIdx.x + k * gridDim.x) * ROWS;
-        V *dst = bufs + (size_t)s * 2 * ROWS * N1;
+        V *dst = bufs + (size_t)s * F * ROWS * N1;
         // (bounds-checking build: a copy past the fields is skipped, the stage
         // completes without bytes)
         if (!XSDE_IN(row0 + ROWS - 1, p.npaths * (int64_t)p.n0, p.status)) {
             mbar_arrive(bars + s);
             return;
         }
-        mbar_arrive_expect_tx(bars + s, (uint32_t)(2 * vec_bytes));
-        bulk_load(dst, p.A + row0 * N1, (uint32_t)vec_bytes, bars + s);
-        bulk_load(dst + ROWS * N1, p.B + row0 * N1, (uint32_t)vec_bytes, bars + s);
+        mbar_arrive_expect_tx(bars + s, IN_B ? 2 * vec_bytes : vec_bytes);
+        if constexpr (F == 1) {
+            bulk_load(dst, p.A + row0 * N1, vec_bytes, bars + s);
+        } else {
+#pragma unroll
+            for (int r = 0; r < ROWS; ++r) {
+                bulk_load(dst + 2 * r * N1, p.A + (row0 + r) * N1, line_bytes, bars + s);
+                if constexpr (IN_B) bulk_load(dst + (2 * r + 1) * N1, p.B + (row0 + r) * N1, line_bytes, bars + s);
+            }
+        }
     };
     if (tid == 0)
-        for (int64_t k = 0; k < NST - 1 && k < mine; ++k) issue_load(k);
+        for (int64_t k = 0; k < NST && k < mine; ++k) issue_load(k);
 
     const float gdt = p.lt.gdt;
     const float sixth = 1.0f / 6.0f, third = 1.0f / 3.0f, half = 0.5f;
     const bool vtime = p.lt.pot == PM_TABLE && p.lt.V_nt > 1;
     const PairedTwiddles tw{tw_hi, tw_lo};
-    const SwizzledLine L{};
+    const ExchangeLayout<V, F> L{};
     // a line's exchanges involve only its own T threads: one warp, or a named
     // barrier per line (ids 1..ROWS), so the lines of an item drift apart and
     // one line's arithmetic overlaps another's exchanges
@@ -150,9 +172,13 @@ __global__ void __launch_bounds__(RowTma<N1>::THREADS, 1) row_pass_tma_kernel(co
         // every thread waits for the stage; the CTA gives up together if any timed out
         const bool landed = mbar_wait(bars + s, (uint32_t)((k / NST) & 1), kWaitNs);
         if (!__syncthreads_and(landed)) {
-            uint32_t par[NST];
-            for (int q = 0; q < NST; ++q) par[q] = (uint32_t)(((k + (q - s + NST) % NST) / NST) & 1);
-            give_up(p.status, bars, par);
+            if (tid == 0) {
+                atomicOr(p.status, ST_TIMEOUT);
+                // the items loaded and not yet waited for
+                for (int64_t q = k; q < k + NST && q < mine; ++q)
+                    mbar_wait(bars + q % NST, (uint32_t)((q / NST) & 1), kWaitNs);
+            }
+            __syncthreads();
             return;
         }
         const int64_t row0 = (blockIdx.x + k * gridDim.x) * ROWS;
@@ -160,9 +186,12 @@ __global__ void __launch_bounds__(RowTma<N1>::THREADS, 1) row_pass_tma_kernel(co
         const int64_t path = row / p.n0;
         const int i0 = (int)(row - path * p.n0);
         const uint32_t gp = (uint32_t)(p.lt.path_offset + path);
-        V *lineA = bufs + (size_t)s * 2 * ROWS * N1 + line * N1;
-        V *lineB = lineA + ROWS * N1;
-        V *const sm2[2] = {lineA, lineB};
+        // a line's A and B lie side by side: its exchanges use both as one buffer
+        V *lineA = bufs + (size_t)s * F * ROWS * N1 + line * F * N1;
+        V *lineB = F == 2 ? lineA + N1 : lineA;
+        V *sm[F];
+        sm[0] = lineA;
+        if constexpr (F == 2) sm[1] = lineB;
 
         // 3D lattices: line i0 of a path is the point pair (i0 / nmid, i0 % nmid)
         const int la = p.ndim == 3 ? i0 / p.nmid : i0;
@@ -196,17 +225,29 @@ __global__ void __launch_bounds__(RowTma<N1>::THREADS, 1) row_pass_tma_kernel(co
         for (int m = 0; m < E; ++m) Vst[m] = vtime ? 0.0f : pot(m, 0);
         auto potv = [&](int m, uint64_t gs) -> float { return vtime ? pot(m, gs) : Vst[m]; };
         // the noise of step sg comes from p.Z (kept by the pass that drew it), read
-        // ahead of the transforms; ROW_STEADY draws and keeps that of step sg + 1
+        // ahead of the transforms; ROW_STEADY draws and keeps that of step sg + 1,
+        // ROW_PROLOGUE that of step sg
         V xi[NOISE ? E : 1];
         auto draw = [&](uint64_t gs) {
             if constexpr (NOISE)
                 draw_points<float, E>(p.lt, gp, (uint32_t)gs, [&](int m) { return (uint32_t)(i0 * N1 + t + m * T); }, xi);
         };
-        if constexpr (NOISE) {
-            if (p.Z)
+        auto keep = [&]() {
+            if constexpr (NOISE)
+                if (p.Z)
 #pragma unroll
-                for (int m = 0; m < E; ++m) xi[m] = load_noise(p.Z, p.lt.noise, row * N1 + t + m * T);
-            else draw(p.sg);
+                    for (int m = 0; m < E; ++m) store_noise(p.Z, p.lt.noise, row * N1 + t + m * T, xi[m]);
+        };
+        if constexpr (NOISE) {
+            if constexpr (IN_B) {
+                if (p.Z)
+#pragma unroll
+                    for (int m = 0; m < E; ++m) xi[m] = load_noise(p.Z, p.lt.noise, row * N1 + t + m * T);
+                else draw(p.sg);
+            } else if constexpr (MODE == ROW_PROLOGUE || MODE == ROW_SI_STEP) {
+                draw(p.sg);
+                if constexpr (MODE == ROW_PROLOGUE) keep();
+            }
         }
         auto pterm = [&](int m, uint64_t gs) -> PointTerm<float> {
             if constexpr (NOISE) {
@@ -219,14 +260,44 @@ __global__ void __launch_bounds__(RowTma<N1>::THREADS, 1) row_pass_tma_kernel(co
             }
         };
 
-        V x[2][E];
+        V x[F][E];
 #pragma unroll
         for (int m = 0; m < E; ++m) {
             x[0][m] = lineA[t + m * T];
-            x[1][m] = lineB[t + m * T];
+            if constexpr (IN_B) x[1][m] = lineB[t + m * T];
         }
         sync();   // the line's natural-order reads complete before swizzled exchanges
-        fftp_bwd<N1, E, 2>(x, t, sm2, L, sync, tw);
+        if constexpr (!REAL_IN) {
+            fftp_bwd<N1, E, F>(x, t, sm, L, sync, tw);
+        }
+        // local terms of the sample of the real-space field x[0] at global step gs
+        auto sample_local = [&](uint64_t gs) {
+            MomentSums acc{};
+#pragma unroll
+            for (int m = 0; m < E; ++m) {
+                const float m2 = cabs2(x[0][m]);
+                acc.add(m2, potv(m, gs));
+                if ((p.sm.which & (MOM_MOD2 | MOM_MOD4)) && p.sm.per_point &&
+                    XSDE_IN((int64_t)p.sample_slot * p.lt.npts + (int64_t)i0 * N1 + t + m * T,
+                            p.sm.nsamp * p.lt.npts, p.status)) {
+                    double *pp = p.sm.per_point + 2 * ((int64_t)p.sample_slot * p.lt.npts + (int64_t)i0 * N1 + t + m * T);
+                    const double d = (double)m2;
+                    atomicAdd(pp, d * p.sm.inv_paths);
+                    atomicAdd(pp + 1, d * d * p.sm.inv_paths);
+                }
+            }
+            double sum[2] = {acc.norm, acc.energy(p.sm.g)};
+            line_sum2<T>(sum, t, line, scratch);
+            if (t == 0) {
+                if ((p.sm.which & (MOM_NORM | MOM_ENERGY)) && p.sm.per_path &&
+                    XSDE_IN((int64_t)p.sample_slot * p.npaths + path, p.sm.nsamp * p.npaths, p.status)) {
+                    double *pq = p.sm.per_path + 2 * ((int64_t)p.sample_slot * p.npaths + path);
+                    atomicAdd(pq, sum[0] * p.sm.dV);
+                    atomicAdd(pq + 1, sum[1] * p.sm.dV);
+                }
+                if (!isfinite(sum[0])) atomicOr(p.status, ST_NONFINITE);
+            }
+        };
         if constexpr (MODE == ROW_STAGE2) {
 #pragma unroll
             for (int m = 0; m < E; ++m) {
@@ -237,71 +308,61 @@ __global__ void __launch_bounds__(RowTma<N1>::THREADS, 1) row_pass_tma_kernel(co
                 x[0][m] = cadd(aI, k3);
                 x[1][m] = caxpy(caxpy(caxpy(aI, sixth, k1), third, k2), third, k3);
             }
-        } else {
+        } else if constexpr (MODE == ROW_SI_STEP) {
 #pragma unroll
-            for (int m = 0; m < E; ++m) x[0][m] = caxpy(x[1][m], sixth, apply_N(x[0][m], pterm(m, p.sg), gdt));
-            if constexpr (SAMPLE) {
-                double acc[2] = {0.0, 0.0};
+            for (int m = 0; m < E; ++m) {
+                const PointTerm<float> pt = pterm(m, p.sg);
+                const V aI = x[0][m];
+                V mid = aI;
+#pragma unroll
+                for (int it = 0; it < 3; ++it) mid = caxpy(aI, half, apply_N(mid, pt, gdt));
+                x[0][m] = make_float2(2.0f * mid.x - aI.x, 2.0f * mid.y - aI.y);
+            }
+        } else {
+            if constexpr (IN_B) {
+#pragma unroll
+                for (int m = 0; m < E; ++m) x[0][m] = caxpy(x[1][m], sixth, apply_N(x[0][m], pterm(m, p.sg), gdt));
+            }
+            if constexpr (SAMPLE) sample_local(MODE == ROW_STEADY ? p.sg + 1 : p.sg);
+            if constexpr (MODE == ROW_STEADY) {
+                draw(p.sg + 1);
+                keep();
+            }
+            if constexpr (OUT_B) {
+#pragma unroll
+                for (int m = 0; m < E; ++m)
+                    x[1][m] = apply_N(x[0][m], pterm(m, MODE == ROW_STEADY ? p.sg + 1 : p.sg), gdt);
+            }
+        }
+        // results leave from the registers (a warp writes 256 contiguous bytes), past
+        // shared memory, which is the busiest unit of this pass
+        V *outA = p.A + row * N1, *outB = p.B + row * N1;
+        const bool inside = XSDE_IN(row0 + ROWS - 1, p.npaths * (int64_t)p.n0, p.status);
+        if constexpr (REAL_OUT) {
+            if (inside)
+#pragma unroll
+                for (int m = 0; m < E; ++m) outA[t + m * T] = x[0][m];
+        } else {
+            fftp_fwd<N1, E, F>(x, t, sm, L, sync, tw);
+            // the dimension-1 factor of exp(L dt/2) (hi/lo: a factor whose FP32
+            // rounding misses its modulus by ~6e-8 would scale the populated modes
+            // by that at every step)
+            if (inside)
 #pragma unroll
                 for (int m = 0; m < E; ++m) {
-                    const double m2 = (double)cabs2(x[0][m]);
-                    acc[0] += m2;
-                    acc[1] += (double)potv(m, p.sg + 1) * m2 + 0.5 * p.sm.g * m2 * m2;
-                    if ((p.sm.which & (MOM_MOD2 | MOM_MOD4)) && p.sm.per_point &&
-                        XSDE_IN((int64_t)p.sample_slot * p.lt.npts + (int64_t)i0 * N1 + t + m * T,
-                                p.sm.nsamp * p.lt.npts, p.status)) {
-                        double *pp = p.sm.per_point + 2 * ((int64_t)p.sample_slot * p.lt.npts + (int64_t)i0 * N1 + t + m * T);
-                        atomicAdd(pp, m2 * p.sm.inv_paths);
-                        atomicAdd(pp + 1, m2 * m2 * p.sm.inv_paths);
-                    }
+                    const int j = t + m * T;
+                    const V eh = e1_s[j], el = e1_s[N1 + j];
+                    outA[j] = cmul_hilo(x[0][m], eh, el);
+                    if constexpr (F == 2) outB[j] = cmul_hilo(x[1][m], eh, el);
                 }
-                line_sum2<T>(acc, t, line, scratch);
-                if (t == 0) {
-                    if ((p.sm.which & (MOM_NORM | MOM_ENERGY)) && p.sm.per_path &&
-                        XSDE_IN((int64_t)p.sample_slot * p.npaths + path, p.sm.nsamp * p.npaths, p.status)) {
-                        double *pq = p.sm.per_path + 2 * ((int64_t)p.sample_slot * p.npaths + path);
-                        atomicAdd(pq, acc[0] * p.sm.dV);
-                        atomicAdd(pq + 1, acc[1] * p.sm.dV);
-                    }
-                    if (!isfinite(acc[0])) atomicOr(p.status, ST_NONFINITE);
-                }
-            }
-            if constexpr (NOISE) {
-                draw(p.sg + 1);
-                if (p.Z)
-#pragma unroll
-                    for (int m = 0; m < E; ++m) store_noise(p.Z, p.lt.noise, row * N1 + t + m * T, xi[m]);
-            }
-#pragma unroll
-            for (int m = 0; m < E; ++m) x[1][m] = apply_N(x[0][m], pterm(m, p.sg + 1), gdt);
         }
-        fftp_fwd<N1, E, 2>(x, t, sm2, L, sync, tw);
-        // the dimension-1 factor of exp(L dt/2) (hi/lo: a factor whose FP32
-        // rounding misses its modulus by ~6e-8 would scale the populated modes
-        // by that at every step); results back in natural order
-#pragma unroll
-        for (int m = 0; m < E; ++m) {
-            const int j = t + m * T;
-            const V eh = e1_s[j], el = e1_s[N1 + j];
-            lineA[j] = cmul_hilo(x[0][m], eh, el);
-            lineB[j] = cmul_hilo(x[1][m], eh, el);
-        }
-        fence_proxy_async();
-        __syncthreads();
-        if (tid == 0) {
-            V *src = bufs + (size_t)s * 2 * ROWS * N1;
-            if (XSDE_IN(row0 + ROWS - 1, p.npaths * (int64_t)p.n0, p.status)) {
-                bulk_store(p.A + row0 * N1, src, (uint32_t)vec_bytes);
-                bulk_store(p.B + row0 * N1, src + ROWS * N1, (uint32_t)vec_bytes);
-            }
-            bulk_commit();
-            if (k + NST - 1 < mine) {
-                bulk_wait_read<1>();     // the stage of item k-1 has been read out
-                issue_load(k + NST - 1);
-            }
+        // the stage goes back to the copy engine (async proxy)
+        if (k + NST < mine) {
+            fence_proxy_async();
+            __syncthreads();
+            if (tid == 0) issue_load(k + NST);
         }
     }
-    if (tid == 0) bulk_wait<0>();
 }
 
 // ---------------------------------------------------------------------------
@@ -522,13 +583,13 @@ cudaError_t launch_dependent(K kern, int grid, int threads, size_t smem, cudaStr
 }
 
 template <int N1, int MODE, bool SAMPLE, bool NOISE>
-cudaError_t row_tma_launch(const Params2D<float> &p, int grid, cudaStream_t s) {
-    using Cfg = RowTma<N1>;
+cudaError_t row_tma_launch(const Params2D<float> &p, int num_sms, cudaStream_t s) {
+    using Cfg = RowTma<N1, row_fields(MODE)>;
     auto kern = row_pass_tma_kernel<N1, MODE, SAMPLE, NOISE>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::SMEM);
     if (e != cudaSuccess) return e;
-    const int64_t items = p.npaths * (int64_t)p.n0 / Cfg::ROWS;
-    const int g = (int)(items < grid ? items : grid);
+    const int64_t items = p.npaths * (int64_t)p.n0 / Cfg::ROWS, want = (int64_t)num_sms * Cfg::CTAS_PER_SM;
+    const int g = (int)(items < want ? items : want);
     return launch_dependent(kern, g, Cfg::THREADS, Cfg::SMEM, s, p);
 }
 
@@ -550,28 +611,49 @@ cudaError_t col_tma_launch(const Params2D<float> &p, const CUtensorMap &a, const
 bool tma_row_supported(int n1) { return n1 == 128 || n1 == 256 || n1 == 512 || n1 == 1024; }
 bool tma_col_supported(int n0) { return n0 == 128 || n0 == 256 || n0 == 512; }
 
-template <int N1> cudaError_t row_tma_dispatch(int mode, const Params2D<float> &p, int grid, cudaStream_t s) {
+template <int N1> cudaError_t row_tma_dispatch(int mode, const Params2D<float> &p, int num_sms, cudaStream_t s) {
     const bool noise = p.lt.noise != NM_NONE, sample = p.sample_slot >= 0;
-    if (mode == ROW_STAGE2)
-        return noise ? row_tma_launch<N1, ROW_STAGE2, false, true>(p, grid, s)
-                     : row_tma_launch<N1, ROW_STAGE2, false, false>(p, grid, s);
-    if (sample)
-        return noise ? row_tma_launch<N1, ROW_STEADY, true, true>(p, grid, s)
-                     : row_tma_launch<N1, ROW_STEADY, true, false>(p, grid, s);
-    return noise ? row_tma_launch<N1, ROW_STEADY, false, true>(p, grid, s)
-                 : row_tma_launch<N1, ROW_STEADY, false, false>(p, grid, s);
-}
-
-cudaError_t launch_row_pass_tma(int mode, const Params2D<float> &p, int grid, cudaStream_t s) {
-    if (mode != ROW_STAGE2 && mode != ROW_STEADY) return cudaErrorInvalidValue;
-    switch (p.n1) {
-        case 128: return row_tma_dispatch<128>(mode, p, grid, s);
-        case 256: return row_tma_dispatch<256>(mode, p, grid, s);
-        case 512: return row_tma_dispatch<512>(mode, p, grid, s);
-        case 1024: return row_tma_dispatch<1024>(mode, p, grid, s);
+    // (mode, samples, uses noise): the instantiated combinations
+    switch (mode) {
+        case ROW_STAGE2:
+            return noise ? row_tma_launch<N1, ROW_STAGE2, false, true>(p, num_sms, s)
+                         : row_tma_launch<N1, ROW_STAGE2, false, false>(p, num_sms, s);
+        case ROW_STEADY:
+            if (sample)
+                return noise ? row_tma_launch<N1, ROW_STEADY, true, true>(p, num_sms, s)
+                             : row_tma_launch<N1, ROW_STEADY, true, false>(p, num_sms, s);
+            return noise ? row_tma_launch<N1, ROW_STEADY, false, true>(p, num_sms, s)
+                         : row_tma_launch<N1, ROW_STEADY, false, false>(p, num_sms, s);
+        case ROW_PROLOGUE:
+            if (sample)
+                return noise ? row_tma_launch<N1, ROW_PROLOGUE, true, true>(p, num_sms, s)
+                             : row_tma_launch<N1, ROW_PROLOGUE, true, false>(p, num_sms, s);
+            return noise ? row_tma_launch<N1, ROW_PROLOGUE, false, true>(p, num_sms, s)
+                         : row_tma_launch<N1, ROW_PROLOGUE, false, false>(p, num_sms, s);
+        case ROW_EPILOGUE:
+            return noise ? row_tma_launch<N1, ROW_EPILOGUE, false, true>(p, num_sms, s)
+                         : row_tma_launch<N1, ROW_EPILOGUE, false, false>(p, num_sms, s);
+        case ROW_SI_START: return row_tma_launch<N1, ROW_SI_START, false, false>(p, num_sms, s);
+        case ROW_SI_STEP:
+            return noise ? row_tma_launch<N1, ROW_SI_STEP, false, true>(p, num_sms, s)
+                         : row_tma_launch<N1, ROW_SI_STEP, false, false>(p, num_sms, s);
+        case ROW_SI_EXIT:
+            return sample ? row_tma_launch<N1, ROW_SI_EXIT, true, false>(p, num_sms, s)
+                          : row_tma_launch<N1, ROW_SI_EXIT, false, false>(p, num_sms, s);
         default: return cudaErrorInvalidValue;
     }
 }
+
+cudaError_t launch_row_pass_tma(int mode, const Params2D<float> &p, int num_sms, cudaStream_t s) {
+    switch (p.n1) {
+        case 128: return row_tma_dispatch<128>(mode, p, num_sms, s);
+        case 256: return row_tma_dispatch<256>(mode, p, num_sms, s);
+        case 512: return row_tma_dispatch<512>(mode, p, num_sms, s);
+        case 1024: return row_tma_dispatch<1024>(mode, p, num_sms, s);
+        default: return cudaErrorInvalidValue;
+    }
+}
+int64_t tma_row_lines(int n1) { return 256 / (n1 / 8); }   // the larger of the two work items
 
 cudaError_t launch_col_pass_tma(const Params2D<float> &p, const CUtensorMap &a, const CUtensorMap &b, int grid,
                                 cudaStream_t s) {

@@ -43,23 +43,28 @@ __device__ __forceinline__ bool wait_or_abort(uint64_t *bar, uint32_t parity, co
 // ---------------------------------------------------------------------------
 // Column pass
 // ---------------------------------------------------------------------------
-template <int N0> struct ColW {
+template <int N0, bool SPREAD> struct ColW {
     static constexpr int E = N0 >= 256 ? N0 / 16 : 16;        // points per lane: 32 / 16 / 16
     static constexpr int P = N0 / E;                           // lanes per column: 16 / 16 / 8
     static constexpr int C = WARP_COL_C;                       // tile columns (64-byte rows)
     static constexpr int CPW = 32 / P;                         // columns per warp
-    static constexpr int NW = C / CPW;                         // warps per CTA: 4 / 4 / 2
-    static constexpr int THREADS = NW * 32;
-    static constexpr int NST = N0 == 512 ? 2 : 3;              // shared-memory stages (3 at 512: no faster)
+    static constexpr int NW = C / CPW;                         // warps per tile: 4 / 4 / 2
+    // A CTA is GROUPS independent groups of NW warps, each with its own stages, that
+    // share one copy of the tables (the room for them is what held an SM to 8 warps
+    // at 512 points): 12 warps at 167 registers, 16 at 128 for the shorter columns.
+    // 64 x 512^2: 136 -> 120 us; 16 warps with one stage each 163 us.  SPREAD: one
+    // group, for fields of few tiles.
+    static constexpr int GROUPS = SPREAD ? 1 : N0 == 512 ? 3 : N0 == 256 ? 4 : 8;
+    static constexpr int THREADS = GROUPS * NW * 32;
+    static constexpr int NST = N0 == 512 ? 2 : 3;        // shared-memory stages of a group
     static constexpr int BOXR = N0 < 256 ? N0 : 256;           // tensor-copy box rows
     static constexpr size_t TILE = (size_t)N0 * C * sizeof(V); // 32 / 16 / 8 KB
     static constexpr int NTW = warp_fft_table_size<N0, E>();
     // (512 points: a compact (c, s) copy of the twiddles for the forward, NTW float2)
     static constexpr size_t TWF = N0 > 256 ? NTW * sizeof(float2) : 0;
-    static constexpr size_t SMEM = 1024 + NST * TILE + NTW * sizeof(TW) + 2 * N0 * sizeof(V) + TWF +
-                                   NST * (sizeof(uint64_t) + sizeof(long long) + sizeof(int)) + 16;
-    static constexpr int CTAS_PER_SM = N0 == 512 ? 2 : N0 == 256 ? 3 : 6;
-    static_assert(CTAS_PER_SM * (SMEM + 1024) <= 233472, "shared memory per SM");
+    static constexpr size_t SMEM = 1024 + GROUPS * NST * TILE + NTW * sizeof(TW) + 2 * N0 * sizeof(V) + TWF +
+                                   GROUPS * (NST * (sizeof(uint64_t) + sizeof(long long) + sizeof(int)) + 16);
+    static_assert(SMEM + 1024 <= 233472, "shared memory per SM");
 };
 
 // The stage ring has no producer warp: thread 0 fills the first stages, and
@@ -67,31 +72,39 @@ template <int N0> struct ColW {
 // refills its stage with the tile NST items later.  A bulk store's completion
 // is tracked per thread, so that warp also waits until its store has read the
 // stage before the load reuses it.
-template <int N0>
-__global__ void __launch_bounds__(ColW<N0>::THREADS, ColW<N0>::CTAS_PER_SM)
+template <int N0, bool SPREAD>
+__global__ void __launch_bounds__(ColW<N0, SPREAD>::THREADS, 1)
     col_pass_warp_kernel(const Params2D<float> p, const __grid_constant__ CUtensorMap mapA,
                          const __grid_constant__ CUtensorMap mapB) {
-    using Cfg = ColW<N0>;
+    using Cfg = ColW<N0, SPREAD>;
     constexpr int E = Cfg::E, P = Cfg::P, C = Cfg::C, CPW = Cfg::CPW, NW = Cfg::NW, NST = Cfg::NST,
                   BOXR = Cfg::BOXR;
     extern __shared__ unsigned char smem_raw[];
     // tiles start on a 1024-byte boundary (the swizzle pattern repeats every 512)
     unsigned char *base = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
-    unsigned char *tiles = base;
-    TW *tw_s = reinterpret_cast<TW *>(base + NST * Cfg::TILE);
+    constexpr int GROUPS = Cfg::GROUPS, GT = NW * 32;   // groups, threads of one
+    const int group = threadIdx.x / GT;
+    unsigned char *tiles = base + (size_t)group * NST * Cfg::TILE;
+    TW *tw_s = reinterpret_cast<TW *>(base + (size_t)GROUPS * NST * Cfg::TILE);
     V *e0_s = reinterpret_cast<V *>(tw_s + Cfg::NTW);
     float2 *twf_s = reinterpret_cast<float2 *>(e0_s + 2 * N0);          // e0_s: hi[N0] | lo[N0]
     uint64_t *full = reinterpret_cast<uint64_t *>(reinterpret_cast<unsigned char *>(twf_s) + Cfg::TWF);
-    volatile long long *issued = reinterpret_cast<volatile long long *>(full + NST);   // last item loaded per stage
-    int *done = reinterpret_cast<int *>(const_cast<long long *>(issued) + NST);         // warps finished per stage
-    volatile int *abort_flag = done + NST;
+    volatile long long *issued = reinterpret_cast<volatile long long *>(full + GROUPS * NST);   // last item loaded per stage
+    int *done = reinterpret_cast<int *>(const_cast<long long *>(issued) + GROUPS * NST);         // warps finished per stage
+    volatile int *abort_flag = done + GROUPS * NST + group;
+    full += group * NST;
+    issued += group * NST;
+    done += group * NST;
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    // (within the group)
+    const int tid = threadIdx.x - group * GT, warp = tid >> 5, lane = tid & 31;
+    // tiles go to the SMs in turn before they go to another group of the same SM
+    const int64_t vblock = blockIdx.x + (int64_t)group * gridDim.x, vgrid = (int64_t)gridDim.x * GROUPS;
     const int tiles_per_path = p.n1 / C;
     // two fields (A, B) per tile, or A alone for the semi-implicit scheme
     const int nvec = p.single_field ? 1 : 2;
     const int64_t nitems = p.npaths * (int64_t)tiles_per_path * nvec;
-    const int64_t mine = nitems > blockIdx.x ? (nitems - 1 - blockIdx.x) / gridDim.x + 1 : 0;
+    const int64_t mine = nitems > vblock ? (nitems - 1 - vblock) / vgrid + 1 : 0;
 
     // columns of 128 and 256 points (shared-memory-bound at 16 points a lane)
     // stage the paired twiddles as split (c, s) / (c eps, s eps) arrays, so the
@@ -101,15 +114,15 @@ __global__ void __launch_bounds__(ColW<N0>::THREADS, ColW<N0>::CTAS_PER_SM)
     constexpr bool SPLIT = N0 <= 256;
     float2 *tw_hi = reinterpret_cast<float2 *>(tw_s), *tw_lo = tw_hi + Cfg::NTW;
     if constexpr (SPLIT) {
-        stage_paired(tw_hi, tw_lo, p.tw0w, Cfg::NTW, tid, blockDim.x);
+        stage_paired(tw_hi, tw_lo, p.tw0w, Cfg::NTW, threadIdx.x, blockDim.x);
     } else {
-        for (int i = tid; i < Cfg::NTW; i += blockDim.x) {
+        for (int i = threadIdx.x; i < Cfg::NTW; i += blockDim.x) {
             const TW w = p.tw0w[i];
             tw_s[i] = w;
             twf_s[i] = make_float2(w.x, w.y);
         }
     }
-    for (int i = tid; i < 2 * N0; i += blockDim.x) e0_s[i] = p.E0[i];
+    for (int i = threadIdx.x; i < 2 * N0; i += blockDim.x) e0_s[i] = p.E0[i];
     if (tid == 0) {
         for (int s = 0; s < NST; ++s) {
             mbar_init(full + s, 1);
@@ -126,7 +139,7 @@ __global__ void __launch_bounds__(ColW<N0>::THREADS, ColW<N0>::CTAS_PER_SM)
 
     // item -> (vector, path, column tile)
     auto decode = [&](int64_t k, int &vec, int64_t &path, int &tile) {
-        const uint32_t it = (uint32_t)(blockIdx.x + k * gridDim.x);
+        const uint32_t it = (uint32_t)(vblock + k * vgrid);
         vec = nvec == 2 ? (int)(it & 1) : 0;
         const uint32_t rest = nvec == 2 ? it >> 1 : it;
         const uint32_t pth = rest / (uint32_t)tiles_per_path;
@@ -209,16 +222,25 @@ __global__ void __launch_bounds__(ColW<N0>::THREADS, ColW<N0>::CTAS_PER_SM)
         decode(k, vec, path, tile);
         unsigned char *tb = tiles + (size_t)s * Cfg::TILE;
         // element (row, c) of the tile as the 64-byte swizzle lays it out: in
-        // 64-byte rows, 16-byte chunk (c / 2) ^ ((row / 2) % 4)
-        auto at = [&](int row) -> V * {
-            return reinterpret_cast<V *>(tb + 64 * row + ((((c >> 1) ^ ((row >> 1) & 3))) << 4) + ((c & 1) << 3));
+        // 64-byte rows, 16-byte chunk (c / 2) ^ ((row / 2) % 4); its offset is XOR-linear
+        // in the row, row_off, so an access is the lane's own offset, an XOR and a constant
+        auto row_off = [](int row) -> int { return (row << 6) ^ (((row >> 1) & 3) << 4); };
+        const int co = ((c >> 1) << 4) | ((c & 1) << 3);
+        const int rt = row_off(t) ^ co, wt = row_off(t & 7) ^ co;
+        unsigned char *const tbw = tb + 64 * E * t;
+        using Slots = ColumnSlots<N0, E>;
+        auto nat = [&](int m) -> V * { return reinterpret_cast<V *>(tb + rt + 64 * P * m); };   // row t + P m
+        auto xw = [&](int r) -> V * {
+            return reinterpret_cast<V *>(tbw + (wt ^ row_off(Slots::write_low(r))) + 64 * Slots::write_high(r));
         };
-        auto xat = [&](int i) -> V * { return at(xslot<E>(i)); };
+        auto xr = [&](int m) -> V * {
+            return reinterpret_cast<V *>(tb + (rt ^ row_off(Slots::read_low(m))) + 64 * Slots::read_high(m));
+        };
         V x[E];
 #pragma unroll
-        for (int m = 0; m < E; ++m) x[m] = *at(t + P * m);
+        for (int m = 0; m < E; ++m) x[m] = *nat(m);
         __syncwarp();
-        warp_fft<N0, E>(x, t, xat, twf);
+        warp_fft<N0, E>(x, t, xw, xr, twf);
         if (sample && vec == 0) {
             // kinetic energy of a_n: sum_k Re(i L(k)) |F psi|^2 dV/(n0 n1); the
             // dimension-1 factor of exp(L dt/2) already applied is divided out
@@ -244,9 +266,9 @@ __global__ void __launch_bounds__(ColW<N0>::THREADS, ColW<N0>::CTAS_PER_SM)
             const int j = t + P * m;
             x[m] = cmul_hilo(x[m], e0_s[j], e0_s[N0 + j]);
         }
-        warp_ifft<N0, E>(x, t, xat, tw);
+        warp_ifft<N0, E>(x, t, xw, xr, tw);
 #pragma unroll
-        for (int m = 0; m < E; ++m) *at(t + P * m) = x[m];
+        for (int m = 0; m < E; ++m) *nat(m) = x[m];
         // the tile goes out through the tensor-memory-access unit (async proxy)
         fence_proxy_async();
         __syncwarp();
@@ -286,17 +308,23 @@ cudaError_t launch_dependent(K kern, int grid, int threads, size_t smem, cudaStr
     return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
+template <int N0, bool SPREAD>
+cudaError_t col_warp_launch_as(const Params2D<float> &p, int64_t items, const CUtensorMap &a, const CUtensorMap &b,
+                               int num_sms, cudaStream_t s) {
+    using Cfg = ColW<N0, SPREAD>;
+    auto kern = col_pass_warp_kernel<N0, SPREAD>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::SMEM);
+    if (e != cudaSuccess) return e;
+    const int64_t want = SPREAD ? items : num_sms;
+    return launch_dependent(kern, (int)(items < want ? items : want), Cfg::THREADS, Cfg::SMEM, s, p, a, b);
+}
+// few tiles are spread over the SMs, one group to a CTA
 template <int N0>
 cudaError_t col_warp_launch(const Params2D<float> &p, const CUtensorMap &a, const CUtensorMap &b, int num_sms,
                             cudaStream_t s) {
-    using Cfg = ColW<N0>;
-    auto kern = col_pass_warp_kernel<N0>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::SMEM);
-    if (e != cudaSuccess) return e;
-    const int64_t items = p.npaths * (int64_t)(p.n1 / Cfg::C) * (p.single_field ? 1 : 2);
-    const int64_t want = (int64_t)num_sms * Cfg::CTAS_PER_SM;
-    const int g = (int)(items < want ? items : want);
-    return launch_dependent(kern, g, Cfg::THREADS, Cfg::SMEM, s, p, a, b);
+    const int64_t items = p.npaths * (int64_t)(p.n1 / WARP_COL_C) * (p.single_field ? 1 : 2);
+    return items <= 2 * (int64_t)num_sms ? col_warp_launch_as<N0, true>(p, items, a, b, num_sms, s)
+                                         : col_warp_launch_as<N0, false>(p, items, a, b, num_sms, s);
 }
 
 }  // namespace

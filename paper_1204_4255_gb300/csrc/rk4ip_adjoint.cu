@@ -58,7 +58,7 @@ __global__ void __launch_bounds__(N / E, sizeof(R) == 8 && E == 4 ? 512 / (N / E
     V *const sm2[2] = {bufA, bufB};
     const SyncBlock sync{};
     const TwiddleTable<tw_t<R>> tw{tws};
-    const LineLayout<V> L{};
+    const ExchangeLayout<V, 2> L{};
     const int t = threadIdx.x;
     const int64_t path = blockIdx.x;
     using Group = FxLineGroup<T, SyncBlock>;
