@@ -304,6 +304,8 @@ void make_twiddle_paired(const std::complex<double> &z, float4 *out) {
     *out = make_float4(c, sn, (float)(c * eps), (float)(sn * eps));
 }
 
+void make_twiddle64(const std::complex<double> &z, float4 *out) { make_twiddle(z, out); }
+
 // per-stage layout of fft.cuh: stage (Ns, R) holds w_n^(r k n/(Ns R)) at
 // [stage_table_offset(n, Ns) + (r-1) Ns + k]; n entries are allocated (the
 // table needs at most n - 1).  PAIRED (complex64): entries for fftp_*.
@@ -336,7 +338,9 @@ int upload_twiddles_2stage(int n, int E, void **dptr, cudaStream_t s) {
     std::vector<float4> tmp((size_t)(n / E - 1) * E);
     for (int r = 1; r < n / E; ++r)
         for (int j = 0; j < E; ++j)
-            make_twiddle_paired(std::polar(1.0, -2.0 * M_PI * (double)((long)r * j) / n), &tmp[(size_t)(r - 1) * E + j]);
+            // (64 points: compensated, see rk4ip_2d_warp.cu)
+            (n == 64 ? make_twiddle64 : make_twiddle_paired)(std::polar(1.0, -2.0 * M_PI * (double)((long)r * j) / n),
+                                                             &tmp[(size_t)(r - 1) * E + j]);
     return upload_raw(tmp, dptr, s);
 }
 
@@ -560,7 +564,9 @@ bool encode_field_map_warp(CUtensorMap *m, void *base, int64_t rows, int64_t col
 
 // The persistent TMA row pass applies to lines of n1 points when the line
 // count fills whole work items.
-bool tma_rows_ok(int n1, int64_t lines) { return tma_row_supported(n1) && lines % tma_row_lines(n1) == 0; }
+bool tma_rows_ok(int n1, int64_t lines, int fields) {
+    return tma_row_supported(n1) && lines % tma_row_lines(n1, fields) == 0;
+}
 
 // Which complex64 pass runs the hot modes (kernel variant, lattice, alignment):
 // PASS_WARP the warp-synchronous column pass of rk4ip_2d_warp.cu, PASS_TMA the
@@ -572,12 +578,18 @@ enum { PASS_GENERIC = 0, PASS_TMA = 1, PASS_WARP = 2 };
 int row_pass_kind(const xsde_problem *p, int n1, int64_t lines) {
     const int v = p->kernel_variant;
     if (v == 1 || p->grid.basis[p->grid.ndim - 1] != XSDE_BASIS_FOURIER) return PASS_GENERIC;
-    return tma_rows_ok(n1, lines) ? PASS_TMA : PASS_GENERIC;
+    return tma_rows_ok(n1, lines, 2) ? PASS_TMA : PASS_GENERIC;
 }
-int col_pass_kind(const xsde_problem *p, int n0, int64_t n1, int basis0) {
+// slabs: fields of n0 x n1 per field of the call.  Cosine / sine columns hold their
+// partners' values too: the warp pass is the faster one at 128 and 256 points
+// with tiles for every SM (16 x 256 x 512: 90 against 99 us a step for the TMA
+// pass, 32 x 128 x 512 89 against 105; one path 27 against 23 to 26, 512 points equal,
+// 64 points 89 against 80 generic); in 3D the alternative is the generic pass.
+int col_pass_kind(const xsde_problem *p, int n0, int64_t n1, int64_t slabs, int basis0) {
     const int v = p->kernel_variant;
-    if (basis0 && p->grid.ndim == 3) return PASS_GENERIC;   // 3D cosine / sine columns: the generic pass
-    if (v == 0 && !basis0 && warp_col_supported(n0, n1)) return PASS_WARP;
+    const bool trig_warp = (n0 == 128 || n0 == 256) && (p->grid.ndim == 3 || slabs * (n1 / WARP_COL_C) > p->num_sms);
+    if (v == 0 && warp_col_supported(n0, n1) && (!basis0 || trig_warp)) return PASS_WARP;
+    if (basis0 && p->grid.ndim == 3) return PASS_GENERIC;
     if ((v == 0 || v == 3) && tma_col_supported(n0) && n1 % COL_TMA_C == 0) return PASS_TMA;
     return PASS_GENERIC;
 }
@@ -671,10 +683,32 @@ int run_nl_3d(xsde_problem *p, Params2D<R> &qr, Params2D<R> &q1, Params2D<R> &q0
         qr.sample_slot = slot;
         return timed(p, 9, s, [&] { return launch_row_pass<R>(ROW_NL, qr, s); });
     };
+    // complex64 columns of 64..512 points take the warp column pass
+    bool w1 = false, w0 = false, wc = false;
+    CUtensorMap m1A, m1B, m0A, m0B, mC;
+    if constexpr (std::is_same<R, float>::value) {
+        if ((uintptr_t)q1.A % 16 == 0 && (uintptr_t)q1.B % 16 == 0 && (uintptr_t)q1.C % 16 == 0) {
+            const xsde_grid &g = p->grid;
+            w1 = warp_col_supported(q1.n0, q1.n1) && p->d_tw2[1] &&
+                 col_maps(PASS_WARP, &m1A, &m1B, q1.A, q1.B, q1.npaths * q1.n0, q1.n1, q1.n0) == PASS_WARP;
+            w0 = warp_col_supported(q0.n0, (int64_t)g.n[1] * g.n[2]) && p->d_tw2[0] &&
+                 col_maps(PASS_WARP, &m0A, &m0B, q0.A, q0.B, q0.npaths * q0.n0, q0.n1, q0.n0) == PASS_WARP;
+            wc = w0 && encode_field_map_warp(&mC, q0.C, q0.npaths * q0.n0, q0.n1, q0.n0);
+            q1.tw0w = static_cast<const tw_t<R> *>(p->d_tw2[1]);
+            q0.tw0w = static_cast<const tw_t<R> *>(p->d_tw2[0]);
+        }
+    }
     auto col = [&](Params2D<R> &q, int mode, int slot) -> cudaError_t {
         q.sample_slot = slot;
         const int kind = (mode == COL_CONV || &q == &c1) ? 10 : mode == COL_SPECTRAL ? 8 : 7;
-        return timed(p, kind, s, [&] { return launch_col_pass<R>(mode, q, s); });
+        return timed(p, kind, s, [&] {
+            if constexpr (std::is_same<R, float>::value) {
+                if (mode == COL_PROPAGATE && &q == &q1 && w1) return launch_col_pass_warp(q, m1A, m1B, p->num_sms, s);
+                if (mode == COL_PROPAGATE && &q == &q0 && w0) return launch_col_pass_warp(q, m0A, m0B, p->num_sms, s);
+                if (mode == COL_CONV && wc) return launch_col_conv_warp(q, mC, p->num_sms, s);
+            }
+            return launch_col_pass<R>(mode, q, s);
+        });
     };
     auto conv = [&]() -> cudaError_t {
         cudaError_t e = col(c1, COL_FFT_FWD, -1);
@@ -794,9 +828,9 @@ int run_3d(xsde_problem *p, void *psi, int64_t nsteps, int64_t npaths, uint64_t 
         if ((uintptr_t)psi % 16 == 0 && (uintptr_t)p->d_scratch % 16 == 0) {
             rk = row_pass_kind(p, g.n[2], npaths * g.n[0] * g.n[1]);
             // dimension 1: [npaths n0 n1][n2]; dimension 0: [npaths n0][n1 n2]
-            ck1 = col_maps(col_pass_kind(p, g.n[1], g.n[2], g.basis[1]), &map1A, &map1B, psi, p->d_scratch,
+            ck1 = col_maps(col_pass_kind(p, g.n[1], g.n[2], npaths * g.n[0], g.basis[1]), &map1A, &map1B, psi, p->d_scratch,
                            npaths * g.n[0] * g.n[1], g.n[2], g.n[1]);
-            ck0 = col_maps(col_pass_kind(p, g.n[0], (int64_t)g.n[1] * g.n[2], g.basis[0]), &map0A, &map0B, psi,
+            ck0 = col_maps(col_pass_kind(p, g.n[0], (int64_t)g.n[1] * g.n[2], npaths, g.basis[0]), &map0A, &map0B, psi,
                            p->d_scratch,
                            npaths * g.n[0], (int64_t)g.n[1] * g.n[2], g.n[0]);
             q1.tw0w = static_cast<const tw_t<R> *>(p->d_tw2[1]);
@@ -887,7 +921,7 @@ int run_si_2d(xsde_problem *p, Params2D<R> &q, int64_t nsteps, uint64_t step0, c
     // 128..512 points the warp (or TMA) column pass, on the one field
     bool tma_rows = false;
     if constexpr (std::is_same<R, float>::value) {
-        tma_rows = (uintptr_t)q.A % 16 == 0 && p->d_twp && tma_rows_ok(q.n1, q.npaths * q.n0);
+        tma_rows = (uintptr_t)q.A % 16 == 0 && p->d_twp && tma_rows_ok(q.n1, q.npaths * q.n0, 1);
         q.tw1p = static_cast<const tw_t<R> *>(p->d_twp);
     }
     auto row = [&](int op, const V *e1, uint64_t sg, int slot) -> cudaError_t {
@@ -982,7 +1016,7 @@ int run_si_3d(xsde_problem *p, Params2D<R> &qr, Params2D<R> &q1, Params2D<R> &q0
     if constexpr (std::is_same<R, float>::value) {
         if ((uintptr_t)qr.A % 16 == 0) {
             const xsde_grid &g = p->grid;
-            tma_rows = p->d_twp && tma_rows_ok(qr.n1, qr.npaths * qr.n0);
+            tma_rows = p->d_twp && tma_rows_ok(qr.n1, qr.npaths * qr.n0, 1);
             qr.tw1p = static_cast<const tw_t<R> *>(p->d_twp);
             if (warp_col_supported(q1.n0, q1.n1) && p->d_tw2[1])
                 ck1 = col_maps(PASS_WARP, &map1, &unused, q1.A, q1.A, npaths * g.n[0] * g.n[1], g.n[2], g.n[1]);
@@ -1076,9 +1110,25 @@ int run_nl_2d(xsde_problem *p, Params2D<R> &q, int64_t nsteps, uint64_t step0, c
         q.sample_slot = slot;
         return timed(p, 9, s, [&] { return launch_row_pass<R>(ROW_NL, q, s); });
     };
+    // complex64 columns of 64..512 points take the warp column pass
+    bool warp = false, warp_conv = false;
+    CUtensorMap mapA, mapB, mapC;
+    if constexpr (std::is_same<R, float>::value) {
+        if ((uintptr_t)q.A % 16 == 0 && (uintptr_t)q.B % 16 == 0 && warp_col_supported(q.n0, q.n1) && p->d_tw2[0]) {
+            warp = col_maps(PASS_WARP, &mapA, &mapB, q.A, q.B, q.npaths * q.n0, q.n1, q.n0) == PASS_WARP;
+            warp_conv = (uintptr_t)q.C % 16 == 0 && encode_field_map_warp(&mapC, q.C, q.npaths * q.n0, q.n1, q.n0);
+            q.tw0w = static_cast<const tw_t<R> *>(p->d_tw2[0]);
+        }
+    }
     auto col = [&](int mode, int slot) -> cudaError_t {
         q.sample_slot = slot;
-        return timed(p, mode == COL_CONV ? 10 : 7, s, [&] { return launch_col_pass<R>(mode, q, s); });
+        return timed(p, mode == COL_CONV ? 10 : 7, s, [&] {
+            if constexpr (std::is_same<R, float>::value) {
+                if (warp && mode == COL_PROPAGATE) return launch_col_pass_warp(q, mapA, mapB, p->num_sms, s);
+                if (warp_conv && mode == COL_CONV) return launch_col_conv_warp(q, mapC, p->num_sms, s);
+            }
+            return launch_col_pass<R>(mode, q, s);
+        });
     };
     if (nsteps > 0) {
         XSDE_CUDA(row(NL_DENSITY, step0, -1), "row pass");
@@ -1215,7 +1265,7 @@ int run_integrate(xsde_problem *p, void *psi, double dt, int64_t nsteps, int64_t
     if constexpr (std::is_same<R, float>::value) {
         if ((uintptr_t)psi % 16 == 0 && (uintptr_t)p->d_scratch % 16 == 0) {
             rk = row_pass_kind(p, g.n[1], npaths * g.n[0]);
-            ck = col_maps(col_pass_kind(p, g.n[0], g.n[1], g.basis[0]), &mapA, &mapB, psi, p->d_scratch,
+            ck = col_maps(col_pass_kind(p, g.n[0], g.n[1], npaths, g.basis[0]), &mapA, &mapB, psi, p->d_scratch,
                           npaths * g.n[0], g.n[1], g.n[0]);
         }
         q.tw0w = static_cast<const tw_t<R> *>(p->d_tw2[0]);

@@ -212,7 +212,8 @@ template <int N, int E> __host__ __device__ constexpr int warp_fft_table_size() 
 // has synchronised the warp since the slots were last read.  Ends with a
 // __syncwarp() before the result is in registers, so the slots may be
 // rewritten by the caller.
-template <int N, int E, typename XW, typename XR, typename Tw>
+// COMP: the table holds compensated twiddles (hi, lo) for both directions
+template <int N, int E, bool COMP, typename XW, typename XR, typename Tw>
 __device__ __forceinline__ void warp_fft(float2 (&x)[E], int t, const XW &xw, const XR &xr, const Tw &tw) {
     constexpr int P = N / E;
     static_assert(P == 8 || P == 16, "two-stage plan: 8 or 16 lanes per line");
@@ -230,7 +231,10 @@ __device__ __forceinline__ void warp_fft(float2 (&x)[E], int t, const XW &xw, co
         float2 u[P];
         u[0] = x[q];
 #pragma unroll
-        for (int r = 1; r < P; ++r) u[r] = tw_fwd(x[q + (E / P) * r], tw((r - 1) * E + j));
+        for (int r = 1; r < P; ++r) {
+            const float4 w = tw((r - 1) * E + j);
+            u[r] = COMP ? twiddle_mul<-1>(x[q + (E / P) * r], w) : tw_fwd(x[q + (E / P) * r], w);
+        }
         dft_fwd<P>(u);
 #pragma unroll
         for (int r = 0; r < P; ++r) x[q + (E / P) * r] = u[r];

@@ -115,10 +115,12 @@ enum NlOp {
     NL_DENSITY = 0,     // A (real u) -> C = F1 |u|^2
     NL_PROLOGUE = 1,    // A (real a), C -> A = E1 F1 a, B = E1 F1 N(a) (at step sg; sample of a)
     NL_FFT = 2,         // A (real a), C -> sample of a (local terms with V_nl), B = F1 a
-    NL_S2A = 3,         // A = F1 a_I, B = F1 k1 -> C = F1 |a_I + k1/2|^2
+    // (S2A and SDA leave the fields they transform back in real space for the passes
+    // that follow them, which would have to transform them again)
+    NL_S2A = 3,         // A = F1 a_I, B = F1 k1 -> A = a_I, B = k1, C = F1 |a_I + k1/2|^2
     NL_S2B = 4,         // A, B, C -> D = k2 = N(a_I + k1/2), C = F1 |a_I + k2/2|^2
     NL_S2C = 5,         // A, B, C, D -> k3; A = E1 F1 (a_I + k3), B = E1 F1 (a_I + k1/6 + k2/3 + k3/3)
-    NL_SDA = 6,         // A = F1 D(a_I + k3) -> C = F1 |D(a_I + k3)|^2
+    NL_SDA = 6,         // A = F1 D(a_I + k3) -> A = D(a_I + k3), C = F1 |D(a_I + k3)|^2
     NL_SDB = 7,         // A, B = F1 D(acc), C -> A = a' = D(acc) + k4/6 (real), C = F1 |a'|^2 unless nl_last
 };
 // Semi-implicit steps on 2D lattices keep one field, A, row-transformed between
@@ -213,7 +215,7 @@ bool tma_row_supported(int n1);   // row-pass line length
 bool tma_col_supported(int n0);   // column length
 size_t col_tma_box_rows(int n0);
 cudaError_t launch_row_pass_tma(int mode, const Params2D<float> &p, int num_sms, cudaStream_t s);
-int64_t tma_row_lines(int n1);    // the lines of a pass are a multiple of it
+int64_t tma_row_lines(int n1, int fields);    // the lines of a pass on that many fields are a multiple of it
 cudaError_t launch_col_pass_tma(const Params2D<float> &p, const CUtensorMap &mapA, const CUtensorMap &mapB, int grid,
                                 cudaStream_t s);
 
@@ -228,6 +230,8 @@ int warp_col_elems(int n0);                       // points per lane (E of the t
 size_t warp_col_box_rows(int n0);
 cudaError_t launch_col_pass_warp(const Params2D<float> &p, const CUtensorMap &mapA, const CUtensorMap &mapB,
                                  int num_sms, cudaStream_t s);
+// COL_CONV on the field mapC describes
+cudaError_t launch_col_conv_warp(const Params2D<float> &p, const CUtensorMap &mapC, int num_sms, cudaStream_t s);
 
 // --------------------------------------------------------------------------
 // 1D adjoint: loss sum_p 1 - |<target|psi_N>|^2 and dL/dV (rk4ip_adjoint.cu)

@@ -204,24 +204,24 @@ __global__ void __launch_bounds__(PPC *(N / E), MINB) rk4ip_1d_kernel(const Para
             const int64_t s = slot_s++;
             next += p.sm.every;
             const uint64_t gs = p.step0 + n;
-            double acc[3] = {0.0, 0.0, 0.0};   // norm, local energy, kinetic energy
+            MomentSums loc{};
             if constexpr (NL) nonlocal(x[0], vn);
 #pragma unroll
             for (int m = 0; m < E; ++m) {
                 const int j = point_of(t + m * T);
                 const int idx[3] = {j, 0, 0};
-                const double m2 = (double)cabs2(x[0][m]);
-                const double vv = (double)potential(p.lt, 1, idx, j, gs);
-                acc[0] += m2;
-                acc[1] += vv * m2 + 0.5 * p.sm.g * m2 * m2;
-                if constexpr (NL) acc[1] += 0.5 * (double)vn[m] * m2;   // pair energy, counted once
+                const R m2r = cabs2(x[0][m]);
+                loc.add(m2r, potential(p.lt, 1, idx, j, gs));
+                if constexpr (NL) loc.pot = fma(widen(half * vn[m]), widen(m2r), loc.pot);   // pair energy, counted once
                 if (active && (p.sm.which & (MOM_MOD2 | MOM_MOD4)) && p.sm.per_point &&
                     XSDE_IN(s * N + j, p.sm.nsamp * N, p.status)) {
                     double *pp = p.sm.per_point + 2 * (s * N + j);
+                    const double m2 = (double)m2r;
                     atomicAdd(pp, m2 * p.sm.inv_paths);
                     atomicAdd(pp + 1, m2 * m2 * p.sm.inv_paths);
                 }
             }
+            double acc[3] = {loc.norm, loc.energy(p.sm.g), 0.0};   // norm, local energy, kinetic energy
             V y[1][E];
 #pragma unroll
             for (int m = 0; m < E; ++m) y[0][m] = x[0][m];
@@ -245,12 +245,15 @@ __global__ void __launch_bounds__(PPC *(N / E), MINB) rk4ip_1d_kernel(const Para
                 }
                 sync();
             } else {
+                double s0 = 0.0, s2 = 0.0;   // sums of |X|^2 and kj^2 |X|^2
 #pragma unroll
                 for (int m = 0; m < E; ++m) {
-                    const int kj = t + m * T;
-                    const double k = p.sm.kscale[0] * (kj < N / 2 ? kj : kj - N);
-                    acc[2] += (p.sm.h0 + p.sm.h2 * k * k) * (double)cabs2(y[0][m]);
+                    const int kj = t + m * T, kb = kj < N / 2 ? kj : kj - N;
+                    const double d = widen(cabs2(y[0][m]));
+                    s0 += d;
+                    s2 = fma(widen((float)(kb * kb)), d, s2);
                 }
+                acc[2] = p.sm.h0 * s0 + p.sm.h2 * p.sm.kscale[0] * p.sm.kscale[0] * s2;
             }
             slot_sum3<T>(acc, t, reinterpret_cast<double *>(bufB), sync);
             if (t == 0 && active) {

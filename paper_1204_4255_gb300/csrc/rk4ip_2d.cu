@@ -11,6 +11,7 @@
 // i.e. 16 field accesses per point per step.
 #include "fft.cuh"
 #include "kernels.h"
+#include "tma.cuh"
 
 namespace xsde {
 namespace {
@@ -48,18 +49,22 @@ __device__ __forceinline__ void group_sum2(double (&v)[2], int t, double *scratc
 // ---------------------------------------------------------------------------
 // Row pass: T = N1/8 threads per line, LINES lines per CTA.
 // ---------------------------------------------------------------------------
-template <int N1> struct RowCfg {
+template <typename R, int N1> struct RowCfg {
     static constexpr int E = 8;
     static constexpr int T = N1 / E;
-    static constexpr int LINES = T >= 256 ? 1 : 256 / T;
+    // small CTAs spread few lines over the SMs and wait for less at a barrier (64 against
+    // 256 threads: complex128 5 x 256 x 64 130 -> 115 us a step, 4 x 512^2 355 -> 337)
+    static constexpr int LINES = T >= 64 ? 1 : 64 / T;
     static constexpr int THREADS = LINES * T;
+    // complex128: 128 registers a thread, 512 threads an SM
+    static constexpr int MINB = sizeof(R) == 8 ? 512 / THREADS : 0;
 };
 
 // TRIG1: dimension 1 is a cosine or sine dimension (p.basis1), see below
 template <typename R, int N1, int MODE, bool TRIG1 = false>
-__global__ void __launch_bounds__(RowCfg<N1>::THREADS, sizeof(R) == 8 ? 2 : 0) row_pass_kernel(const Params2D<R> p) {
+__global__ void __launch_bounds__(RowCfg<R, N1>::THREADS, RowCfg<R, N1>::MINB) row_pass_kernel(const Params2D<R> p) {
     using V = cx<R>;
-    using Cfg = RowCfg<N1>;
+    using Cfg = RowCfg<R, N1>;
     constexpr int E = Cfg::E, T = Cfg::T, LINES = Cfg::LINES;
     constexpr int BUF = line_len<V, N1>();
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -92,6 +97,10 @@ __global__ void __launch_bounds__(RowCfg<N1>::THREADS, sizeof(R) == 8 ? 2 : 0) r
     const R gdt = p.lt.gdt;
     const R sixth = R(1) / R(6), third = R(1) / R(3), half = R(0.5);
     const bool sample = p.sample_slot >= 0;
+
+    // the previous pass's fields from here on
+    grid_launch_dependents();
+    grid_dependency_wait();
 
     // A cosine / sine dimension 1 (TRIG1; XMDS2 Sec. 2.1) holds a line's points
     // in the even-odd order of the DCT-II's evaluation by an N1-point FFT:
@@ -171,21 +180,22 @@ __global__ void __launch_bounds__(RowCfg<N1>::THREADS, sizeof(R) == 8 ? 2 : 0) r
     // (vnl: the non-local potential of f, whose pair energy 1/2 V_nl |f|^2 the
     // energy adds; nullptr without the term)
     auto sample_local = [&](const V (&f)[E], uint64_t gs, const R *vnl = nullptr) {
-        double acc[2] = {0.0, 0.0};
+        MomentSums sums{};
 #pragma unroll
         for (int m = 0; m < E; ++m) {
-            const double m2 = (double)cabs2(f[m]);
-            acc[0] += m2;
-            acc[1] += (double)potv(m, gs) * m2 + 0.5 * p.sm.g * m2 * m2;
-            if (vnl) acc[1] += 0.5 * (double)vnl[m] * m2;
+            const R m2r = cabs2(f[m]);
+            sums.add(m2r, potv(m, gs));
+            if (vnl) sums.pot = fma(widen(R(0.5) * vnl[m]), widen(m2r), sums.pot);
             if (active && (p.sm.which & (MOM_MOD2 | MOM_MOD4)) && p.sm.per_point) {
                 const int64_t ip = (int64_t)p.sample_slot * p.lt.npts + (int64_t)i0 * N1 + pt_of(t + m * T);
                 if (!XSDE_IN(ip, p.sm.nsamp * p.lt.npts, p.status)) continue;
                 double *pp = p.sm.per_point + 2 * ip;
+                const double m2 = (double)m2r;
                 atomicAdd(pp, m2 * p.sm.inv_paths);
                 atomicAdd(pp + 1, m2 * m2 * p.sm.inv_paths);
             }
         }
+        double acc[2] = {sums.norm, sums.energy(p.sm.g)};
         group_sum2<T>(acc, t, scratch);
         if (t == 0 && active) {
             if ((p.sm.which & (MOM_NORM | MOM_ENERGY)) && p.sm.per_path) {
@@ -321,7 +331,27 @@ __global__ void __launch_bounds__(RowCfg<N1>::THREADS, sizeof(R) == 8 ? 2 : 0) r
 #pragma unroll
             for (int m = 0; m < E; ++m) y[0][m] = Arow[t + m * T];
             fft_line<N1, E, +1, 1>(y, t, sm1, L, sync, tw, grp);
+            if (active)
+#pragma unroll
+                for (int m = 0; m < E; ++m) Arow[t + m * T] = y[0][m];
             density_out(y[0]);
+            return;
+        } else if (op == NL_SDB) {
+            // k4 = N(D(a_I + k3)) at step sg; a' = D(acc) + k4/6, real space; V_nl and D(acc)
+            // are transformed back together
+            V y[2][E];
+#pragma unroll
+            for (int m = 0; m < E; ++m) {
+                y[0][m] = Brow[t + m * T];
+                y[1][m] = Crow[t + m * T];
+            }
+            fft_line<N1, E, +1, 2>(y, t, sm2, L2, sync, tw, grp);
+#pragma unroll
+            for (int m = 0; m < E; ++m) {
+                x[0][m] = caxpy(y[0][m], sixth, apply_N(Arow[t + m * T], ptv(m, p.sg, y[1][m].x), gdt));
+                if (active) Arow[t + m * T] = x[0][m];
+            }
+            if (!p.nl_last) density_out(x[0]);
             return;
         } else {
 #pragma unroll
@@ -329,8 +359,14 @@ __global__ void __launch_bounds__(RowCfg<N1>::THREADS, sizeof(R) == 8 ? 2 : 0) r
                 x[0][m] = Arow[t + m * T];
                 x[1][m] = Brow[t + m * T];
             }
-            fft_line<N1, E, +1, 2>(x, t, sm2, L2, sync, tw, grp);
             if (op == NL_S2A) {
+                fft_line<N1, E, +1, 2>(x, t, sm2, L2, sync, tw, grp);
+                if (active)
+#pragma unroll
+                    for (int m = 0; m < E; ++m) {
+                        Arow[t + m * T] = x[0][m];
+                        Brow[t + m * T] = x[1][m];
+                    }
                 V u[E];
 #pragma unroll
                 for (int m = 0; m < E; ++m) u[m] = caxpy(x[0][m], half, x[1][m]);
@@ -347,16 +383,6 @@ __global__ void __launch_bounds__(RowCfg<N1>::THREADS, sizeof(R) == 8 ? 2 : 0) r
                     u[m] = caxpy(x[0][m], half, k2);
                 }
                 density_out(u);
-                return;
-            }
-            if (op == NL_SDB) {
-                // k4 = N(D(a_I + k3)) at step sg; a' = D(acc) + k4/6, real space
-#pragma unroll
-                for (int m = 0; m < E; ++m) {
-                    x[0][m] = caxpy(x[1][m], sixth, apply_N(x[0][m], ptv(m, p.sg, v[m]), gdt));
-                    if (active) Arow[t + m * T] = x[0][m];
-                }
-                if (!p.nl_last) density_out(x[0]);
                 return;
             }
             // NL_S2C: k3 = N(a_I + k2/2) with the V_nl of that argument
@@ -487,9 +513,9 @@ __global__ void __launch_bounds__(RowCfg<N1>::THREADS, sizeof(R) == 8 ? 2 : 0) r
 // column; lanes run over columns first so every load is a 128-byte segment.
 // ---------------------------------------------------------------------------
 template <typename R, int N0> struct ColCfg {
-    // 128-byte row segments (16 c64 / 8 c128 columns) up to 1024 (c64) or 512
+    // 128-byte (c64) or 64-byte (c128) row segments up to 1024 (c64) or 512
     // (c128) threads per CTA; longer columns use narrower tiles.
-    static constexpr int CMAX = sizeof(R) == 4 ? 16 : 8;
+    static constexpr int CMAX = sizeof(R) == 4 ? 16 : 4;
     static constexpr int TMAX = sizeof(R) == 4 ? 1024 : 512;
     static constexpr int E = 8;
     static constexpr int T = N0 / E;
@@ -530,6 +556,8 @@ __global__ void __launch_bounds__(ColCfg<R, N0>::THREADS, ColCfg<R, N0>::MINB) c
                            XSDE_IN(col, n1, p.status)))
         return;
 #endif
+    grid_launch_dependents();
+    grid_dependency_wait();
     // A cosine / sine dimension 0 (TRIG; XMDS2 Sec. 2.1) gathers its rows in the
     // even-odd order of the DCT-II's evaluation by an N0-point FFT (slot s holds
     // row 2s below N0/2, row 2 N0-1-2s above; odd rows negated for the sine
@@ -586,7 +614,8 @@ __global__ void __launch_bounds__(ColCfg<R, N0>::THREADS, ColCfg<R, N0>::MINB) c
         // fields written by propagating row passes already carry the
         // dimension-1 factor of exp(L dt/2); divide its modulus back out
         const double w = (MODE == COL_SPECTRAL) ? p.spec_scale : 1.0 / (double)cabs2(p.E1[col]);
-        double s = 0.0;
+        // Fourier: h = (h0 + h2 kc2) + h2 ks^2 kj^2 takes two FP64 sums, of |X|^2 and kj^2 |X|^2
+        double s = 0.0, s2 = 0.0;
 #pragma unroll
         for (int m = 0; m < E; ++m) {
             const int kj = t + m * T;
@@ -600,10 +629,13 @@ __global__ void __launch_bounds__(ColCfg<R, N0>::THREADS, ColCfg<R, N0>::MINB) c
                 const double k0 = p.sm.kscale[0] * (bas == 1 ? kj : N0 - kj);
                 s += (kj == 0 ? 1.0 : 2.0) * (p.sm.h0 + p.sm.h2 * (k0 * k0 + kc2)) * (xr * xr + xi * xi);
             } else {
-                const double k0 = p.sm.kscale[0] * (kj < N0 / 2 ? kj : kj - N0);
-                s += (p.sm.h0 + p.sm.h2 * (k0 * k0 + kc2)) * (double)cabs2(f[m]);
+                const int kb = kj < N0 / 2 ? kj : kj - N0;
+                const double d = widen(cabs2(f[m]));
+                s += d;
+                s2 = fma(widen((float)(kb * kb)), d, s2);
             }
         }
+        if constexpr (!TRIG) s = (p.sm.h0 + p.sm.h2 * kc2) * s + p.sm.h2 * p.sm.kscale[0] * p.sm.kscale[0] * s2;
         if (p.basis1 && p.kinner == 0 && col != 0) wc = 2.0;
         s *= w * wc;
         s = warp_sum(s);
@@ -726,7 +758,7 @@ __global__ void __launch_bounds__(ColCfg<R, N0>::THREADS, ColCfg<R, N0>::MINB) c
 }
 
 template <typename R, int N1, int MODE> cudaError_t row_launch(const Params2D<R> &p, cudaStream_t s) {
-    using Cfg = RowCfg<N1>;
+    using Cfg = RowCfg<R, N1>;
     const size_t smem = (size_t)Cfg::LINES * 2 * line_len<cx<R>, N1>() * sizeof(cx<R>) +
                         (size_t)Cfg::LINES * (Cfg::T / 32 + 1) * 2 * sizeof(double) +
                         (sizeof(R) == 8 ? (size_t)Cfg::LINES * FxLineGroup<Cfg::T, SyncBlock>::kWords * 4 : 0);
@@ -741,8 +773,7 @@ template <typename R, int N1, int MODE> cudaError_t row_launch(const Params2D<R>
     if (e != cudaSuccess) return e;
     const int64_t rows = p.npaths * (int64_t)p.n0;
     const int64_t blocks = (rows + Cfg::LINES - 1) / Cfg::LINES;
-    kern<<<(unsigned)blocks, Cfg::THREADS, smem, s>>>(p);
-    return cudaGetLastError();
+    return launch_dependent(kern, dim3((unsigned)blocks), Cfg::THREADS, smem, s, p);
 }
 
 template <typename R, int N0, int MODE> cudaError_t col_launch(const Params2D<R> &p, cudaStream_t s) {
@@ -755,8 +786,7 @@ template <typename R, int N0, int MODE> cudaError_t col_launch(const Params2D<R>
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     dim3 grid((unsigned)(p.n1 / Cfg::C), (unsigned)p.npaths);
-    kern<<<grid, Cfg::THREADS, smem, s>>>(p);
-    return cudaGetLastError();
+    return launch_dependent(kern, grid, Cfg::THREADS, smem, s, p);
 }
 
 }  // namespace

@@ -117,9 +117,13 @@ __global__ void __launch_bounds__(RowTma<N1, row_fields(MODE)>::THREADS, RowTma<
     const int64_t mine = nitems > blockIdx.x ? (nitems - 1 - blockIdx.x) / gridDim.x + 1 : 0;
     constexpr uint32_t line_bytes = (uint32_t)(N1 * sizeof(V)), vec_bytes = ROWS * line_bytes;
 
-    // the paired twiddles as (c, s) and (c eps, s eps) halves in tw_s's N1 entries
+    // the paired twiddles as (c, s) and (c eps, s eps) halves in tw_s's N1 entries.
+    // Lines of 64 points have one twiddled stage, where compensated twiddles (hi, lo)
+    // both ways cost little: they keep the generic pass's transforms, and the
+    // accuracy that small lattices are held to point by point
+    constexpr bool PAIRED = N1 > 64;
     float2 *tw_hi = reinterpret_cast<float2 *>(tw_s), *tw_lo = tw_hi + N1;
-    stage_paired(tw_hi, tw_lo, p.tw1p, N1, tid, blockDim.x);
+    stage_paired(tw_hi, tw_lo, PAIRED ? p.tw1p : p.tw1, N1, tid, blockDim.x);
     if constexpr (!REAL_OUT)
         for (int i = tid; i < 2 * N1; i += blockDim.x) e1_s[i] = p.E1[i];
     if (tid == 0) {
@@ -131,28 +135,29 @@ __global__ void __launch_bounds__(RowTma<N1, row_fields(MODE)>::THREADS, RowTma<
     grid_launch_dependents();
     grid_dependency_wait();
 
-    auto issue_load = [&](int64_t k) {   // item k of this CTA into stage k % NST
+    auto issue_load = [&](int64_t k) {   // item k of this CTA into stage k % NST; warp 0, a copy a lane
         const int s = (int)(k % NST);
         const int64_t row0 = (blockIdx.x + k * gridDim.x) * ROWS;
         V *dst = bufs + (size_t)s * F * ROWS * N1;
         // (bounds-checking build: a copy past the fields is skipped, the stage
         // completes without bytes)
-        if (!XSDE_IN(row0 + ROWS - 1, p.npaths * (int64_t)p.n0, p.status)) {
-            mbar_arrive(bars + s);
-            return;
+        const bool inside = XSDE_IN(row0 + ROWS - 1, p.npaths * (int64_t)p.n0, p.status);
+        if (tid == 0) {
+            if (inside) mbar_arrive_expect_tx(bars + s, IN_B ? 2 * vec_bytes : vec_bytes);
+            else mbar_arrive(bars + s);
         }
-        mbar_arrive_expect_tx(bars + s, IN_B ? 2 * vec_bytes : vec_bytes);
+        __syncwarp();
+        if (!inside) return;
         if constexpr (F == 1) {
-            bulk_load(dst, p.A + row0 * N1, vec_bytes, bars + s);
+            if (tid == 0) bulk_load(dst, p.A + row0 * N1, vec_bytes, bars + s);
         } else {
-#pragma unroll
-            for (int r = 0; r < ROWS; ++r) {
-                bulk_load(dst + 2 * r * N1, p.A + (row0 + r) * N1, line_bytes, bars + s);
-                if constexpr (IN_B) bulk_load(dst + (2 * r + 1) * N1, p.B + (row0 + r) * N1, line_bytes, bars + s);
-            }
+            static_assert(2 * ROWS <= 32, "a copy a lane");
+            const int r = tid >> 1;
+            if (r < ROWS && (IN_B || !(tid & 1)))
+                bulk_load(dst + tid * N1, ((tid & 1) ? p.B : p.A) + (row0 + r) * N1, line_bytes, bars + s);
         }
     };
-    if (tid == 0)
+    if (tid < 32)
         for (int64_t k = 0; k < NST && k < mine; ++k) issue_load(k);
 
     const float gdt = p.lt.gdt;
@@ -268,7 +273,8 @@ __global__ void __launch_bounds__(RowTma<N1, row_fields(MODE)>::THREADS, RowTma<
         }
         sync();   // the line's natural-order reads complete before swizzled exchanges
         if constexpr (!REAL_IN) {
-            fftp_bwd<N1, E, F>(x, t, sm, L, sync, tw);
+            if constexpr (PAIRED) fftp_bwd<N1, E, F>(x, t, sm, L, sync, tw);
+            else fft<N1, E, +1, F>(x, t, sm, L, sync, tw);
         }
         // local terms of the sample of the real-space field x[0] at global step gs
         auto sample_local = [&](uint64_t gs) {
@@ -343,7 +349,8 @@ __global__ void __launch_bounds__(RowTma<N1, row_fields(MODE)>::THREADS, RowTma<
 #pragma unroll
                 for (int m = 0; m < E; ++m) outA[t + m * T] = x[0][m];
         } else {
-            fftp_fwd<N1, E, F>(x, t, sm, L, sync, tw);
+            if constexpr (PAIRED) fftp_fwd<N1, E, F>(x, t, sm, L, sync, tw);
+            else fft<N1, E, -1, F>(x, t, sm, L, sync, tw);
             // the dimension-1 factor of exp(L dt/2) (hi/lo: a factor whose FP32
             // rounding misses its modulus by ~6e-8 would scale the populated modes
             // by that at every step)
@@ -360,7 +367,7 @@ __global__ void __launch_bounds__(RowTma<N1, row_fields(MODE)>::THREADS, RowTma<
         if (k + NST < mine) {
             fence_proxy_async();
             __syncthreads();
-            if (tid == 0) issue_load(k + NST);
+            if (tid < 32) issue_load(k + NST);
         }
     }
 }
@@ -564,24 +571,6 @@ __global__ void __launch_bounds__(ColTma<N0>::THREADS, ColTma<N0>::CTAS_PER_SM)
     if (tid == 0) bulk_wait<0>();
 }
 
-// Launch with programmatic stream serialization: the kernel may start while
-// the previous kernel of the stream drains; it waits for that kernel's results
-// in grid_dependency_wait() after loading its tables.
-template <typename K, typename... Args>
-cudaError_t launch_dependent(K kern, int grid, int threads, size_t smem, cudaStream_t s, const Args &...args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3((unsigned)threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, args...);
-}
-
 template <int N1, int MODE, bool SAMPLE, bool NOISE>
 cudaError_t row_tma_launch(const Params2D<float> &p, int num_sms, cudaStream_t s) {
     using Cfg = RowTma<N1, row_fields(MODE)>;
@@ -608,7 +597,7 @@ cudaError_t col_tma_launch(const Params2D<float> &p, const CUtensorMap &a, const
 
 }  // namespace
 
-bool tma_row_supported(int n1) { return n1 == 128 || n1 == 256 || n1 == 512 || n1 == 1024; }
+bool tma_row_supported(int n1) { return n1 == 64 || n1 == 128 || n1 == 256 || n1 == 512 || n1 == 1024; }
 bool tma_col_supported(int n0) { return n0 == 128 || n0 == 256 || n0 == 512; }
 
 template <int N1> cudaError_t row_tma_dispatch(int mode, const Params2D<float> &p, int num_sms, cudaStream_t s) {
@@ -646,6 +635,7 @@ template <int N1> cudaError_t row_tma_dispatch(int mode, const Params2D<float> &
 
 cudaError_t launch_row_pass_tma(int mode, const Params2D<float> &p, int num_sms, cudaStream_t s) {
     switch (p.n1) {
+        case 64: return row_tma_dispatch<64>(mode, p, num_sms, s);
         case 128: return row_tma_dispatch<128>(mode, p, num_sms, s);
         case 256: return row_tma_dispatch<256>(mode, p, num_sms, s);
         case 512: return row_tma_dispatch<512>(mode, p, num_sms, s);
@@ -653,7 +643,7 @@ cudaError_t launch_row_pass_tma(int mode, const Params2D<float> &p, int num_sms,
         default: return cudaErrorInvalidValue;
     }
 }
-int64_t tma_row_lines(int n1) { return 256 / (n1 / 8); }   // the larger of the two work items
+int64_t tma_row_lines(int n1, int fields) { return (fields == 2 && n1 <= 512 ? 128 : 256) / (n1 / 8); }
 
 cudaError_t launch_col_pass_tma(const Params2D<float> &p, const CUtensorMap &a, const CUtensorMap &b, int grid,
                                 cudaStream_t s) {

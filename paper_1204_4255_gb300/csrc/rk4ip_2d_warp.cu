@@ -43,22 +43,24 @@ __device__ __forceinline__ bool wait_or_abort(uint64_t *bar, uint32_t parity, co
 // ---------------------------------------------------------------------------
 // Column pass
 // ---------------------------------------------------------------------------
-template <int N0, bool SPREAD> struct ColW {
-    static constexpr int E = N0 >= 256 ? N0 / 16 : 16;        // points per lane: 32 / 16 / 16
-    static constexpr int P = N0 / E;                           // lanes per column: 16 / 16 / 8
+enum { COLW_PLAIN = 0, COLW_TRIG = 1, COLW_CONV = 2 };   // kinds of column pass
+template <int N0, bool SPREAD, bool TRIG> struct ColW {
+    static constexpr int E = N0 >= 256 ? N0 / 16 : N0 == 128 ? 16 : 8;   // points per lane: 32 / 16 / 16 / 8
+    static constexpr int P = N0 / E;                           // lanes per column: 16 / 16 / 8 / 8
     static constexpr int C = WARP_COL_C;                       // tile columns (64-byte rows)
     static constexpr int CPW = 32 / P;                         // columns per warp
-    static constexpr int NW = C / CPW;                         // warps per tile: 4 / 4 / 2
+    static constexpr int NW = C / CPW;                         // warps per tile: 4 / 4 / 2 / 2
     // A CTA is GROUPS independent groups of NW warps, each with its own stages, that
     // share one copy of the tables (the room for them is what held an SM to 8 warps
     // at 512 points): 12 warps at 167 registers, 16 at 128 for the shorter columns.
     // 64 x 512^2: 136 -> 120 us; 16 warps with one stage each 163 us.  SPREAD: one
     // group, for fields of few tiles.
-    static constexpr int GROUPS = SPREAD ? 1 : N0 == 512 ? 3 : N0 == 256 ? 4 : 8;
+    // (TRIG holds the partner values too: 8 to 12 warps)
+    static constexpr int GROUPS = SPREAD ? 1 : TRIG ? (N0 == 512 ? 2 : N0 == 256 ? 3 : 6) : N0 == 512 ? 3 : N0 == 256 ? 4 : 8;
     static constexpr int THREADS = GROUPS * NW * 32;
     static constexpr int NST = N0 == 512 ? 2 : 3;        // shared-memory stages of a group
     static constexpr int BOXR = N0 < 256 ? N0 : 256;           // tensor-copy box rows
-    static constexpr size_t TILE = (size_t)N0 * C * sizeof(V); // 32 / 16 / 8 KB
+    static constexpr size_t TILE = (size_t)N0 * C * sizeof(V); // 32 / 16 / 8 / 4 KB
     static constexpr int NTW = warp_fft_table_size<N0, E>();
     // (512 points: a compact (c, s) copy of the twiddles for the forward, NTW float2)
     static constexpr size_t TWF = N0 > 256 ? NTW * sizeof(float2) : 0;
@@ -72,11 +74,20 @@ template <int N0, bool SPREAD> struct ColW {
 // refills its stage with the tile NST items later.  A bulk store's completion
 // is tracked per thread, so that warp also waits until its store has read the
 // stage before the load reuses it.
-template <int N0, bool SPREAD>
-__global__ void __launch_bounds__(ColW<N0, SPREAD>::THREADS, 1)
+// TRIG: dimension 0 is a cosine / sine dimension (XMDS2 Sec. 2.1): rows are
+// taken from the tile in the even-odd order of the DCT-II's evaluation by an
+// N0-point FFT (slot s <- row 2s below N0/2, row 2 N0-1-2s above; odd rows
+// negated for the sine basis) and one exchange pairs k with N0-k for
+// U_k = A_k V_k + B_k V_{N0-k} (A in E0, B in p.B0, read through L1).  16 x 256 x 512:
+// 33 us a pass in the TMA column kernel, 27 us here.
+// CONV: the density convolution of the non-local term, K2(k0, col) (read through L1)
+// in place of E0(k0), on the one field the maps describe.
+template <int N0, bool SPREAD, int KIND>
+__global__ void __launch_bounds__(ColW<N0, SPREAD, KIND == COLW_TRIG>::THREADS, 1)
     col_pass_warp_kernel(const Params2D<float> p, const __grid_constant__ CUtensorMap mapA,
                          const __grid_constant__ CUtensorMap mapB) {
-    using Cfg = ColW<N0, SPREAD>;
+    constexpr bool TRIG = KIND == COLW_TRIG, CONV = KIND == COLW_CONV;
+    using Cfg = ColW<N0, SPREAD, TRIG>;
     constexpr int E = Cfg::E, P = Cfg::P, C = Cfg::C, CPW = Cfg::CPW, NW = Cfg::NW, NST = Cfg::NST,
                   BOXR = Cfg::BOXR;
     extern __shared__ unsigned char smem_raw[];
@@ -122,7 +133,7 @@ __global__ void __launch_bounds__(ColW<N0, SPREAD>::THREADS, 1)
             twf_s[i] = make_float2(w.x, w.y);
         }
     }
-    for (int i = threadIdx.x; i < 2 * N0; i += blockDim.x) e0_s[i] = p.E0[i];
+    for (int i = threadIdx.x; i < 2 * N0 && !CONV; i += blockDim.x) e0_s[i] = p.E0[i];
     if (tid == 0) {
         for (int s = 0; s < NST; ++s) {
             mbar_init(full + s, 1);
@@ -210,7 +221,7 @@ __global__ void __launch_bounds__(ColW<N0, SPREAD>::THREADS, 1)
         if constexpr (SPLIT) return PairedTwiddles{tw_hi, tw_lo};
         else return PairedTwiddles{twf_s, twf_s};
     }();
-    const bool sample = p.sample_slot >= 0;
+    const bool sample = !CONV && p.sample_slot >= 0;
     for (int64_t k = 0; k < mine; ++k) {
         const int s = (int)(k % NST);
         if (!wait_or_abort(full + s, (uint32_t)((k / NST) & 1), abort_flag)) {
@@ -236,11 +247,31 @@ __global__ void __launch_bounds__(ColW<N0, SPREAD>::THREADS, 1)
         auto xr = [&](int m) -> V * {
             return reinterpret_cast<V *>(tb + (rt ^ row_off(Slots::read_low(m))) + 64 * Slots::read_high(m));
         };
+        // (TRIG) the slots t + P m below N0/2 lie at rows 2t + 2 P m, the others at
+        // 2 N0 - 1 - 2 P m - 2t
+        const bool odd_neg = TRIG && p.basis0 == 2;
+        auto gather = [&](int m) -> V * {
+            const int chunk = m < E / 2 ? (t & 3) : 3 - (t & 3);
+            const int row = m < E / 2 ? 2 * t + 2 * P * m : 2 * N0 - 1 - 2 * P * m - 2 * t;
+            return reinterpret_cast<V *>(tb + 64 * row + ((chunk << 4) ^ co));
+        };
         V x[E];
 #pragma unroll
-        for (int m = 0; m < E; ++m) x[m] = *nat(m);
+        for (int m = 0; m < E; ++m) {
+            x[m] = TRIG ? *gather(m) : *nat(m);
+            if (odd_neg && m >= E / 2) x[m] = make_float2(-x[m].x, -x[m].y);
+        }
         __syncwarp();
-        warp_fft<N0, E>(x, t, xw, xr, twf);
+        warp_fft<N0, E, (N0 == 64)>(x, t, xw, xr, twf);
+        V xq[TRIG ? E : 1];   // partners V_{N0-k}
+        if constexpr (TRIG) {
+#pragma unroll
+            for (int m = 0; m < E; ++m) *nat(m) = x[m];
+            __syncwarp();
+#pragma unroll
+            for (int m = 0; m < E; ++m) xq[m] = *reinterpret_cast<V *>(tb + (row_off((N0 - P * m - t) & (N0 - 1)) ^ co));
+            __syncwarp();
+        }
         if (sample && vec == 0) {
             // kinetic energy of a_n: sum_k Re(i L(k)) |F psi|^2 dV/(n0 n1); the
             // dimension-1 factor of exp(L dt/2) already applied is divided out
@@ -248,13 +279,31 @@ __global__ void __launch_bounds__(ColW<N0, SPREAD>::THREADS, 1)
             const int k1i = col < p.n1 / 2 ? col : col - p.n1;
             const double k1 = p.sm.kscale[1] * k1i;
             const double w = 1.0 / (double)cabs2(p.E1[col]);
-            double sacc = 0.0;
+            // h(k) = (h0 + h2 k1^2) + h2 ks^2 kj^2: two FP64 sums, of |X|^2 and kj^2 |X|^2
+            double s0 = 0.0, s2 = 0.0;
 #pragma unroll
             for (int m = 0; m < E; ++m) {
                 const int kj = t + P * m;
-                const double k0 = p.sm.kscale[0] * (kj < N0 / 2 ? kj : kj - N0);
-                sacc += (p.sm.h0 + p.sm.h2 * (k0 * k0 + k1 * k1)) * (double)cabs2(x[m]);
+                if constexpr (TRIG) {
+                    // cosine spectrum from the pair, Parseval weight 2 but at k = 0;
+                    // sine mode N0-1-k sits at k
+                    // (in the field's precision: the sum is accumulated in FP64)
+                    float sn, cs;
+                    sincospif(-(float)kj / (2.0f * N0), &sn, &cs);
+                    const float xr = 0.5f * (cs * (x[m].x + xq[m].x) - sn * (x[m].y - xq[m].y));
+                    const float xi = 0.5f * (cs * (x[m].y + xq[m].y) + sn * (x[m].x - xq[m].x));
+                    const int kb = p.basis0 == 1 ? kj : N0 - kj;
+                    const double d = widen((kj == 0 ? 1.0f : 2.0f) * (xr * xr + xi * xi));
+                    s0 += d;
+                    s2 = fma(widen((float)(kb * kb)), d, s2);
+                } else {
+                    const int kb = kj < N0 / 2 ? kj : kj - N0;
+                    const double d = widen(cabs2(x[m]));
+                    s0 += d;
+                    s2 = fma(widen((float)(kb * kb)), d, s2);
+                }
             }
+            double sacc = (p.sm.h0 + p.sm.h2 * k1 * k1) * s0 + p.sm.h2 * p.sm.kscale[0] * p.sm.kscale[0] * s2;
             sacc = warp_sum(sacc * w);
             if (lane == 0 && (p.sm.which & (MOM_NORM | MOM_ENERGY)) && p.sm.per_path &&
                 XSDE_IN((int64_t)p.sample_slot * p.npaths + path, p.sm.nsamp * p.npaths, p.status))
@@ -264,11 +313,16 @@ __global__ void __launch_bounds__(ColW<N0, SPREAD>::THREADS, 1)
 #pragma unroll
         for (int m = 0; m < E; ++m) {
             const int j = t + P * m;
-            x[m] = cmul_hilo(x[m], e0_s[j], e0_s[N0 + j]);
+            if constexpr (CONV) x[m] = cmul(x[m], __ldg(p.K2 + (int64_t)j * p.n1 + tile * C + c));
+            else x[m] = cmul_hilo(x[m], e0_s[j], e0_s[N0 + j]);
+            if constexpr (TRIG) x[m] = cadd(x[m], cmul_hilo(xq[m], __ldg(p.B0 + j), __ldg(p.B0 + N0 + j)));
         }
         warp_ifft<N0, E>(x, t, xw, xr, tw);
 #pragma unroll
-        for (int m = 0; m < E; ++m) *nat(m) = x[m];
+        for (int m = 0; m < E; ++m) {
+            if (odd_neg && m >= E / 2) x[m] = make_float2(-x[m].x, -x[m].y);
+            *(TRIG ? gather(m) : nat(m)) = x[m];
+        }
         // the tile goes out through the tensor-memory-access unit (async proxy)
         fence_proxy_async();
         __syncwarp();
@@ -290,29 +344,11 @@ __global__ void __launch_bounds__(ColW<N0, SPREAD>::THREADS, 1)
     if (lane == 0) bulk_wait<0>();
 }
 
-// Launch with programmatic stream serialization: the kernel may start while
-// the previous kernel of the stream drains; it waits for that kernel's results
-// in grid_dependency_wait() after loading its tables.
-template <typename K, typename... Args>
-cudaError_t launch_dependent(K kern, int grid, int threads, size_t smem, cudaStream_t s, const Args &...args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3((unsigned)threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, args...);
-}
-
-template <int N0, bool SPREAD>
+template <int N0, bool SPREAD, int KIND>
 cudaError_t col_warp_launch_as(const Params2D<float> &p, int64_t items, const CUtensorMap &a, const CUtensorMap &b,
                                int num_sms, cudaStream_t s) {
-    using Cfg = ColW<N0, SPREAD>;
-    auto kern = col_pass_warp_kernel<N0, SPREAD>;
+    using Cfg = ColW<N0, SPREAD, KIND == COLW_TRIG>;
+    auto kern = col_pass_warp_kernel<N0, SPREAD, KIND>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::SMEM);
     if (e != cudaSuccess) return e;
     const int64_t want = SPREAD ? items : num_sms;
@@ -320,28 +356,43 @@ cudaError_t col_warp_launch_as(const Params2D<float> &p, int64_t items, const CU
 }
 // few tiles are spread over the SMs, one group to a CTA
 template <int N0>
-cudaError_t col_warp_launch(const Params2D<float> &p, const CUtensorMap &a, const CUtensorMap &b, int num_sms,
+cudaError_t col_warp_launch(const Params2D<float> &p, const CUtensorMap &a, const CUtensorMap &b, bool conv, int num_sms,
                             cudaStream_t s) {
     const int64_t items = p.npaths * (int64_t)(p.n1 / WARP_COL_C) * (p.single_field ? 1 : 2);
-    return items <= 2 * (int64_t)num_sms ? col_warp_launch_as<N0, true>(p, items, a, b, num_sms, s)
-                                         : col_warp_launch_as<N0, false>(p, items, a, b, num_sms, s);
+    if (conv) return col_warp_launch_as<N0, false, COLW_CONV>(p, items, a, b, num_sms, s);
+    if (p.basis0) return col_warp_launch_as<N0, false, COLW_TRIG>(p, items, a, b, num_sms, s);
+    return items <= 2 * (int64_t)num_sms ? col_warp_launch_as<N0, true, COLW_PLAIN>(p, items, a, b, num_sms, s)
+                                         : col_warp_launch_as<N0, false, COLW_PLAIN>(p, items, a, b, num_sms, s);
 }
 
 }  // namespace
 
-bool warp_col_supported(int n0, int64_t n1) { return (n0 == 128 || n0 == 256 || n0 == 512) && n1 % WARP_COL_C == 0; }
-int warp_col_elems(int n0) { return n0 >= 256 ? n0 / 16 : 16; }
+bool warp_col_supported(int n0, int64_t n1) {
+    return (n0 == 64 || n0 == 128 || n0 == 256 || n0 == 512) && n1 % WARP_COL_C == 0;
+}
+int warp_col_elems(int n0) { return n0 >= 256 ? n0 / 16 : n0 == 128 ? 16 : 8; }
 size_t warp_col_box_rows(int n0) { return n0 < 256 ? (size_t)n0 : 256; }
 
-cudaError_t launch_col_pass_warp(const Params2D<float> &p, const CUtensorMap &a, const CUtensorMap &b, int num_sms,
-                                 cudaStream_t s) {
-    if (!p.tw0w || p.basis0) return cudaErrorInvalidValue;
+static cudaError_t col_pass_warp_any(const Params2D<float> &p, const CUtensorMap &a, const CUtensorMap &b, bool conv,
+                                     int num_sms, cudaStream_t s) {
     switch (p.n0) {
-        case 128: return col_warp_launch<128>(p, a, b, num_sms, s);
-        case 256: return col_warp_launch<256>(p, a, b, num_sms, s);
-        case 512: return col_warp_launch<512>(p, a, b, num_sms, s);
+        case 64: return col_warp_launch<64>(p, a, b, conv, num_sms, s);
+        case 128: return col_warp_launch<128>(p, a, b, conv, num_sms, s);
+        case 256: return col_warp_launch<256>(p, a, b, conv, num_sms, s);
+        case 512: return col_warp_launch<512>(p, a, b, conv, num_sms, s);
         default: return cudaErrorInvalidValue;
     }
+}
+cudaError_t launch_col_pass_warp(const Params2D<float> &p, const CUtensorMap &a, const CUtensorMap &b, int num_sms,
+                                 cudaStream_t s) {
+    if (!p.tw0w || (p.basis0 && !p.B0)) return cudaErrorInvalidValue;
+    return col_pass_warp_any(p, a, b, false, num_sms, s);
+}
+cudaError_t launch_col_conv_warp(const Params2D<float> &p, const CUtensorMap &mapC, int num_sms, cudaStream_t s) {
+    if (!p.tw0w || !p.K2 || p.basis0) return cudaErrorInvalidValue;
+    Params2D<float> q = p;
+    q.single_field = 1;
+    return col_pass_warp_any(q, mapC, mapC, true, num_sms, s);
 }
 
 }  // namespace xsde

@@ -113,4 +113,22 @@ __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddep
 // memory operations are visible (a no-op without a programmatic dependency).
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// Launch with programmatic stream serialization: the kernel may start while
+// the previous kernel of the stream drains; it waits for that kernel's results
+// in grid_dependency_wait() after its own preparation.
+template <typename K, typename... Args>
+cudaError_t launch_dependent(K kern, dim3 grid, int threads, size_t smem, cudaStream_t s, const Args &...args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
 }  // namespace xsde
