@@ -917,8 +917,8 @@ int run_si_2d(xsde_problem *p, Params2D<R> &q, int64_t nsteps, uint64_t step0, c
     const V *E0f = static_cast<const V *>(p->d_Ef[0]), *E1f = static_cast<const V *>(p->d_Ef[1]);
     const int S = q.sm.every;
     auto is_sample = [&](int64_t k) { return S > 0 && k % S == 0; };
-    // complex64 lines of 128..1024 points take the TMA row pass, columns of
-    // 128..512 points the warp (or TMA) column pass, on the one field
+    // complex64 lines of 64..1024 points take the TMA row pass, columns of
+    // 64..512 points the warp (or TMA) column pass, on the one field
     bool tma_rows = false;
     if constexpr (std::is_same<R, float>::value) {
         tma_rows = (uintptr_t)q.A % 16 == 0 && p->d_twp && tma_rows_ok(q.n1, q.npaths * q.n0, 1);

@@ -567,4 +567,44 @@ template <typename V> struct TwiddleLdg {
     __device__ __forceinline__ V operator()(int m) const { return __ldg(p + m); }
 };
 
+// --- complex64 pairs through two buffers -----------------------------------------
+// fft<N, E, S, 2> whose exchanges alternate between two buffers of N 16-byte slots
+// (PAR: the first one's), so that an exchange waits once, between its writes and its
+// reads: a buffer is written again two exchanges later, after a barrier that every
+// reader has passed.  A transform's successor starts at pp_parity<N, E>() if it
+// follows one that started at 0; a forward / backward pair ends where it began.
+template <int N, int E> __host__ __device__ constexpr int pp_parity() {
+    int k = 0;
+    for (int ns = stage_radix<E>(N); ns < N; ns *= stage_radix<E>(N / ns)) ++k;
+    return k & 1;
+}
+template <int N, int E, int S, int Ns, int PAR, typename Sync, typename Tw>
+__device__ __forceinline__ void fft_pp_from(float2 (&v)[2][E], int t, float2 *const (&buf)[2], const Sync &sync, const Tw &tw) {
+    constexpr int R = stage_radix<E>(N / Ns), B = E / R, T = N / E;
+    const PairLine L{};
+    fft_stage<N, E, R, Ns, S, 2>(v, t, tw);
+    if constexpr (Ns * R < N) {
+        float2 *const sm[2] = {buf[PAR], nullptr};
+#pragma unroll
+        for (int q = 0; q < B; ++q) {
+            const int j = t + q * T, k = j & (Ns - 1), lb = L((j - k) * R + k);
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const float2 u[2] = {v[0][q + r * B], v[1][q + r * B]};
+                slot_put<PairLine, 2>(sm, L.join(lb, r * Ns), u);
+            }
+        }
+        sync();
+        const int lt = L(t);
+#pragma unroll
+        for (int m = 0; m < E; ++m) {
+            float2 u[2];
+            slot_get<PairLine, 2>(sm, L.join(lt, m * T), u);
+            v[0][m] = u[0];
+            v[1][m] = u[1];
+        }
+        fft_pp_from<N, E, S, Ns * R, PAR ^ 1>(v, t, buf, sync, tw);
+    }
+}
+
 }  // namespace xsde

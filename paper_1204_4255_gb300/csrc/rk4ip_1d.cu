@@ -54,6 +54,15 @@ __device__ __forceinline__ void slot_sum3(double (&v)[3], int t, double *scratch
     }
 }
 
+// Exchange buffers of a path's slot, of N values each: two, or four where the pair
+// transforms alternate between two, one barrier an exchange (complex64 paths of
+// several warps; cosine / sine lattices exchange between the transforms too and keep
+// two).  4096 paths, us a step: 1024 points 81.1 -> 72.4, 512 points 29.6 -> 28.4;
+// 1216 x 2048 50.6 -> 47.5
+template <typename R, int N, int E, bool TRIG> __host__ __device__ constexpr int slot_buffers() {
+    return sizeof(R) == 4 && N / E > 32 && !TRIG ? 4 : 2;
+}
+
 // the step's point term with the non-local potential vn added to V
 template <typename R> __device__ __forceinline__ PointTerm<R> with_vnl(PointTerm<R> pt, R dt, R vn) {
     pt.dtV += dt * vn;
@@ -80,7 +89,8 @@ __global__ void __launch_bounds__(PPC *(N / E), MINB) rk4ip_1d_kernel(const Para
     tw_t<R> *tws = reinterpret_cast<tw_t<R> *>(smem_raw);
     const int slot = threadIdx.x / T;
     const int t = threadIdx.x - slot * T;
-    V *bufA = reinterpret_cast<V *>(tws + N) + slot * 2 * BUF;
+    constexpr int SLOTBUF = slot_buffers<R, N, E, TRIG>() * BUF;
+    V *bufA = reinterpret_cast<V *>(tws + N) + slot * SLOTBUF;
     V *bufB = bufA + BUF;
     V *const sm2[2] = {bufA, bufB};
     V *const sm1[1] = {bufA};
@@ -89,7 +99,7 @@ __global__ void __launch_bounds__(PPC *(N / E), MINB) rk4ip_1d_kernel(const Para
     const LineLayout<V> L{};
     using Sync = SlotSync<T, PPC>;
     using Group = FxLineGroup<T, Sync>;
-    V *const bufs_end = reinterpret_cast<V *>(tws + N) + PPC * 2 * BUF;
+    V *const bufs_end = reinterpret_cast<V *>(tws + N) + PPC * SLOTBUF;
     const Group grp{reinterpret_cast<uint32_t *>(bufs_end) + slot * Group::kWords, t, sync};
 
     for (int i = threadIdx.x; i < N; i += blockDim.x) tws[i] = p.tw[i];
@@ -170,6 +180,11 @@ __global__ void __launch_bounds__(PPC *(N / E), MINB) rk4ip_1d_kernel(const Para
         auto with = [&](V *const (&sm)[NV]) {
             if constexpr (FX && !TRIG) {
                 fx_propagate<N, E, true, false, NV>(v, t, sm, X, sync, tw, grp, p.Etab, p.Ex);
+            } else if constexpr (NV == 2 && slot_buffers<R, N, E, TRIG>() == 4) {
+                V *const pp[2] = {bufA, bufA + 2 * BUF};
+                fft_pp_from<N, E, -1, 1, 0>(v, t, pp, sync, tw);
+                kmul(v);
+                fft_pp_from<N, E, +1, 1, pp_parity<N, E>()>(v, t, pp, sync, tw);
             } else {
                 fft_line<N, E, -1, NV>(v, t, sm, X, sync, tw, grp);
                 kmul(v);
@@ -367,7 +382,7 @@ __global__ void __launch_bounds__(PPC *(N / E), MINB) rk4ip_1d_kernel(const Para
 template <typename R, int N, int E, int PPC, int SCHEME = 0, bool NL = false, bool TRIG = false, int MINB = 1>
 cudaError_t launch_ppc(const Params1D<R> &p, cudaStream_t s) {
     constexpr int T = N / E;
-    const size_t smem = (size_t)N * sizeof(tw_t<R>) + (size_t)PPC * 2 * line_len<cx<R>, N>() * sizeof(cx<R>) +
+    const size_t smem = (size_t)N * sizeof(tw_t<R>) + (size_t)PPC * slot_buffers<R, N, E, TRIG>() * line_len<cx<R>, N>() * sizeof(cx<R>) +
                         (sizeof(R) == 8 ? (size_t)PPC * FxLineGroup<T, SlotSync<T, PPC>>::kWords * 4 : 0);
     const bool noise = p.lt.noise != NM_NONE;
     auto kern = noise ? rk4ip_1d_kernel<R, N, E, PPC, true, SCHEME, NL, TRIG, MINB>
@@ -508,7 +523,8 @@ int rk4ip_1d_elems(int variant) { return variant == 4 ? 4 : variant == 5 ? 2 : 8
 //   complex64    32 points,  152 paths: 3.28 / 3.02 / 1.57 / 1.14;  4096: 3.30 / 3.01 / 2.34 / 3.05
 //               128 points,  304 paths: 2.75 / 2.79 / 1.56 / 2.23;  4096: 7.66 / 8.08 / 7.31 / 18.1
 //               256 points,  304 paths: 2.69 / 2.73 / 2.01 / 3.32;  1216: 4.27 / 4.07 / 5.06 / 10.6
-//              1024 points,  152 paths: 4.76 / 4.29 / 4.13 / 7.60;   304: 7.24 / 6.35 / 6.87 / 15.2
+//               512 points,  152 paths: 3.11 capped / 2.68 / 2.41 / 3.48;  1216: 8.46 / 9.06 / 12.6 / 21.7
+//              1024 points,  152 paths: 3.87 uncapped / 4.06 / 6.50;   1216: 21.8 / 23.6 / 32.6 / 52.3
 //   complex128  256 points,    1 path :  41 /  40 /  21 /  11;      4096: 136 / 171 / 126 / 133
 //              1024 points,    1 path :  63 /  61 /  30 /  40;      4096: 600 / 1006 / 841 / 1083
 int rk4ip_1d_default(bool fp64, int n, int64_t npaths, int num_sms) {
@@ -520,7 +536,7 @@ int rk4ip_1d_default(bool fp64, int n, int64_t npaths, int num_sms) {
     if (n <= 32 && pts <= (int64_t)512 * num_sms) return 5;
     if (n <= 128) return 4;
     if (n <= 256) return npaths <= 2 * (int64_t)num_sms ? 4 : 0;
-    if (n <= 1024 && npaths <= num_sms) return 4;
+    if (n <= 512 && npaths <= num_sms) return 4;
     return npaths <= 2 * (int64_t)num_sms ? 6 : 0;   // variant 6: uncapped in complex64
 }
 #endif

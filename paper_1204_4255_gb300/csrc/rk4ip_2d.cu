@@ -119,34 +119,37 @@ __global__ void __launch_bounds__(RowCfg<R, N1>::THREADS, RowCfg<R, N1>::MINB) r
     };
     auto store_real = [&](V *f, int sl, V v) { f[pt_of(sl)] = negated(sl) ? mk<V>(-v.x, -v.y) : v; };
 
-    // raw potential of point (line, t + m T) at global step gs.  complex128: a
-    // harmonic trap is its line's part, once, plus three FP64 instructions a point
-    // (the FP64 pipe takes 16 clocks a warp instruction, conversions included)
-    R vline = R(0), xfirst = R(0), xstep = R(0), hlast = R(0);
-    if constexpr (sizeof(R) == 8) {
-        if (p.lt.pot == PM_HARMONIC) {
-            const R xa = p.lt.xmin[0] + R(la) * p.lt.dx[0];
-            vline = p.lt.hw2[0] * xa * xa;
-            if (p.ndim == 3) {
-                const R xb = p.lt.xmin[1] + R(lb) * p.lt.dx[1];
-                vline += p.lt.hw2[1] * xb * xb;
-            }
-            xstep = p.ndim == 3 ? p.lt.dx[2] : p.lt.dx[1];
-            hlast = p.ndim == 3 ? p.lt.hw2[2] : p.lt.hw2[1];
-            xfirst = (p.ndim == 3 ? p.lt.xmin[2] : p.lt.xmin[1]) + R(t) * xstep;
+    // raw potential of point (line, t + m T) at global step gs: a harmonic trap is
+    // its line's part, once, plus the last dimension's (no indexed coordinate array,
+    // which a run-time dimension count would put in local memory).  complex128: the
+    // coordinates of a thread's points by multiples of the thread spacing, three FP64
+    // instructions a point (a conversion would take the FP64 pipe another 16 clocks)
+    R vline = R(0), xlast = R(0), dlast = R(0), hlast = R(0);
+    if (p.lt.pot == PM_HARMONIC) {
+        const R xa = p.lt.xmin[0] + R(la) * p.lt.dx[0];
+        vline = p.lt.hw2[0] * xa * xa;
+        if (p.ndim == 3) {
+            const R xb = p.lt.xmin[1] + R(lb) * p.lt.dx[1];
+            vline += p.lt.hw2[1] * xb * xb;
         }
+        xlast = p.ndim == 3 ? p.lt.xmin[2] : p.lt.xmin[1];
+        dlast = p.ndim == 3 ? p.lt.dx[2] : p.lt.dx[1];
+        hlast = p.ndim == 3 ? p.lt.hw2[2] : p.lt.hw2[1];
     }
+    const R xfirst = sizeof(R) == 8 ? xlast + R(t) * dlast : R(0);
     auto pot = [&](int m, uint64_t gs) -> R {
-        if constexpr (sizeof(R) == 8 && !TRIG1) {
-            if (p.lt.pot == PM_HARMONIC) {
-                const R x = xfirst + R(m * T) * xstep;
-                return vline + hlast * x * x;
-            }
-        }
         const int ic = pt_of(t + m * T);
-        const int idx2[3] = {la, ic, 0};
-        const int idx3[3] = {la, lb, ic};
-        return potential(p.lt, p.ndim, p.ndim == 3 ? idx3 : idx2, (int64_t)i0 * N1 + ic, gs);
+        if (p.lt.pot == PM_HARMONIC) {
+            const R x = sizeof(R) == 8 && !TRIG1 ? xfirst + R(m * T) * dlast : xlast + R(ic) * dlast;
+            return vline + hlast * x * x;
+        }
+        if (p.lt.pot == PM_TABLE) {
+            int64_t r = p.lt.V_nt > 1 ? (int64_t)gs : 0;
+            if (r >= p.lt.V_nt) r = p.lt.V_nt - 1;
+            const int64_t iv = r * p.lt.npts + (int64_t)i0 * N1 + ic;
+            return XSDE_IN(iv, p.lt.V_nt * p.lt.npts, p.lt.status) ? p.lt.V[iv] : R(0);
+        }
+        return R(0);
     };
     // static potentials are evaluated once per element; tables with one row per
     // step are read for the step at hand
@@ -158,7 +161,11 @@ __global__ void __launch_bounds__(RowCfg<R, N1>::THREADS, RowCfg<R, N1>::MINB) r
 #pragma unroll
         for (int m = 0; m < E; ++m) Vst[m] = vtime ? R(0) : pot(m, 0);
     }
-    auto potv = [&](int m, uint64_t gs) -> R { return !KEEP_V || vtime ? pot(m, gs) : Vst[m]; };
+    auto potv = [&](int m, uint64_t gs) -> R {
+        if constexpr (KEEP_V)
+            if (!vtime) return Vst[m];
+        return pot(m, gs);
+    };
     // first: this pass is the first to use the step's noise, and keeps it
     auto pterm = [&](int m, uint64_t gs, bool first = false) -> PointTerm<R> {
         const int i1 = pt_of(t + m * T);

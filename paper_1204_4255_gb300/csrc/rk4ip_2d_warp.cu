@@ -9,11 +9,11 @@
 //                 two (or four) columns of the tile and transforms them with the
 //                 two-stage plan of fft2.cuh, exchanging in place inside its own
 //                 columns.  The last warp to finish a tile stores it and refills
-//                 the stage; several small CTAs per SM keep the SM busy while one
+//                 the stage; several groups of warps per SM keep it busy while one
 //                 of them waits.
 //
 // Every wait is bounded by the global timer; a wait that runs out records
-// ST_TIMEOUT, lets the CTA's other warps stop, waits (bounded) for this CTA's
+// ST_TIMEOUT, lets the group's other warps stop, waits (bounded) for the group's
 // copies in flight and returns.
 #include <type_traits>
 

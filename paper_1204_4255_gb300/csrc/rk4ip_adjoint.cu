@@ -54,7 +54,9 @@ __global__ void __launch_bounds__(N / E, sizeof(R) == 8 && E == 4 ? 512 / (N / E
     tw_t<R> *tws = reinterpret_cast<tw_t<R> *>(smem_raw);
     V *bufA = reinterpret_cast<V *>(tws + N);
     V *bufB = bufA + BUF;
-    double *red = reinterpret_cast<double *>(bufB + BUF);
+    // (complex64: a second pair of buffers, fft_pp_from)
+    constexpr int BUFS = sizeof(R) == 4 ? 4 : 2;
+    double *red = reinterpret_cast<double *>(bufA + BUFS * BUF);
     V *const sm2[2] = {bufA, bufB};
     const SyncBlock sync{};
     const TwiddleTable<tw_t<R>> tw{tws};
@@ -93,13 +95,14 @@ __global__ void __launch_bounds__(N / E, sizeof(R) == 8 && E == 4 ? 512 / (N / E
         if constexpr (sizeof(R) == 8) {
             fx_propagate<N, E, true, CONJ, 2>(x, t, sm2, L, sync, tw, grp, p.Etab, p.Ex);
         } else {
-            fft<N, E, -1, 2>(x, t, sm2, L, sync, tw);
+            V *const pp[2] = {bufA, bufA + 2 * BUF};
+            fft_pp_from<N, E, -1, 1, 0>(x, t, pp, sync, tw);
 #pragma unroll
             for (int m = 0; m < E; ++m)
 #pragma unroll
                 for (int iv = 0; iv < 2; ++iv)
                     x[iv][m] = CONJ ? cmulconj_hilo(x[iv][m], Ek[m], El[m]) : cmul_hilo(x[iv][m], Ek[m], El[m]);
-            fft<N, E, +1, 2>(x, t, sm2, L, sync, tw);
+            fft_pp_from<N, E, +1, 1, pp_parity<N, E>()>(x, t, pp, sync, tw);
         }
     };
     const size_t stride = (size_t)p.npaths * N;              // one field of all paths
@@ -284,7 +287,7 @@ __global__ void __launch_bounds__(N / E, sizeof(R) == 8 && E == 4 ? 512 / (N / E
 
 template <typename R, int N, int E> cudaError_t adj_launch(const AdjParams<R> &p, cudaStream_t s) {
     constexpr int T = N / E;
-    const size_t smem = (size_t)N * sizeof(tw_t<R>) + (size_t)2 * line_len<cx<R>, N>() * sizeof(cx<R>) +
+    const size_t smem = (size_t)N * sizeof(tw_t<R>) + (size_t)(sizeof(R) == 4 ? 4 : 2) * line_len<cx<R>, N>() * sizeof(cx<R>) +
                         (size_t)2 * ((T + 31) / 32) * sizeof(double) +
                         (sizeof(R) == 8 ? (size_t)FxLineGroup<T, SyncBlock>::kWords * 4 : 0);
     auto kern = rk4ip_adjoint_kernel<R, N, E>;
