@@ -39,9 +39,9 @@ METRIC = "RK4IP grid-point-steps/s"
 UNIT = "pt-steps/s"
 BYTES_PER_PT_PASS = {"c64": 32, "c128": 64}   # 2 fields in + 2 out per pass
 # DRAM read + write per launch measured by ncu for the default configuration
-# (profiles/gpe2d_passes_512x512x64_c64_full.md); reported only for that
+# (profiles/gpe2d_row_items_col_groups_512x512x64_c64.md); reported only for that
 # configuration and only while the kernels are unchanged since the capture.
-MEASURED_TRAFFIC = {("c64", 64, "col_propagate"): 481.7e6}
+MEASURED_TRAFFIC = {("c64", 64, "col_propagate"): 481.9e6}
 
 
 def _dist():
@@ -250,7 +250,8 @@ def c128_figure(P: int = 64, nsteps: int = 10) -> dict:
     return {"value": value, "unit": UNIT, "dtype": "c128", "workload": f"2D GPE 512x512 x {P}, {nsteps} RK4IP steps",
             "ms_per_rk4ip_step": ms / nsteps, "bound": "alu", "fp64_tflops": tflops, "fp64_fma_peak_tflops": f64,
             "fp64_frac": tflops / f64, "hbm_frac_at_256B": value * 256 / 1e9 / peak,
-            "flops_model": "8 * 5 log2(N_tot) + 100 per pt-step"}
+            "flops_model": "8 * 5 log2(N_tot) + 100 per pt-step",
+            "note": "the transforms run in 64-bit integers: fp64_frac is the FP64 model's FLOPs over the FP64 FMA rate and may exceed 1"}
 
 
 def gpe3d_figure(P: int = 8, nsteps: int = 20) -> dict:

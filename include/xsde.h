@@ -146,8 +146,8 @@ int64_t xsde_grid_points(const xsde_grid *grid);
  * or noise from the grid (they copy it).  Runs on 1D lattices and on any
  * dimensions of 2D and 3D lattices (RK4IP; a cosine / sine last dimension runs
  * the generic row passes, and a 2D one takes its samples between chunks of
- * steps from the real-space field; 3D cosine / sine columns run the generic
- * column passes); the semi-implicit scheme on 2D and 3D lattices,
+ * steps from the real-space field; cosine / sine columns of 128 and 256
+ * points run the warp column pass, other 3D ones the generic passes); the semi-implicit scheme on 2D and 3D lattices,
  * xsde_integrate_plain, xsde_integrate_adaptive, xsde_adjoint,
  * xsde_integrate_static_scratch and xsde_set_nonlocal report XSDE_EUNSUPPORTED
  * for such a problem.  A 1D cosine / sine problem has one launch shape
@@ -415,8 +415,8 @@ int xsde_synchronize(xsde_problem *prob, void *stream);
  *     are spread over more threads); where a bound applies a variant repeats
  *     another;
  *   2D and 3D lattices (4 variants): 0 uses, in complex64, the persistent
- *     TMA-pipelined row pass (lines of 128..1024 points) and the column pass
- *     with warp-synchronous two-stage transforms (columns of 128..512 points,
+ *     TMA-pipelined row pass (lines of 64..1024 points) and the column pass
+ *     with warp-synchronous two-stage transforms (columns of 64..512 points,
  *     a multiple of 8 columns; else the TMA column pass), 1 forces the generic
  *     passes, 2 uses the TMA row passes and the generic column passes, 3 the
  *     TMA row and TMA column passes;
