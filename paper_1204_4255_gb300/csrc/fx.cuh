@@ -147,11 +147,21 @@ template <int NV, int E> __device__ __forceinline__ void fx_largest(const longlo
     }
 }
 
+// magnitude of q's high word: |q| <= 2^32 (m + 1) for either sign (the shift floors;
+// abs() would give -2^60 + 1 a magnitude of 2^28, and sixteen of those sum to 2^32 = 0)
+__device__ __forceinline__ uint32_t fx_mag(long long q) {
+    const int h = (int)(q >> 32);
+    return (uint32_t)(h ^ (h >> 31));
+}
+
 // Shift every line right for a transform: by room, which takes S to 2^60.5, or
 // by what the first MID points' sums need (largest values below 2^32 mx) where
 // that is less; `room` keeps the difference for fx_refit.  S is taken over the
-// high words (one unit of them covers what the low words add): a thread's
-// 2E <= 16 of them stay below 2^32, and in units of 2^41 a line's stay below 2^32.
+// high words' magnitudes (one unit of them covers what the low words add), whose sum
+// over a thread's 2E <= 16 values stays below 2^32: from fx_load |q| < 2^60 and each
+// is at most 2^28 - 1; after a transform, whose values are at most 2^60.5 (1 - 2^-26)
+// in modulus by the margins taken here and in fx_largest, a value's two are at most
+// 2^29 - 8 together.  In units of 2^41 a line's sum stays below 2^32.
 template <int MID, int NV, int E, typename Group>
 __device__ __forceinline__ void fx_fit(longlong2 (&q)[NV][E], int (&ex)[NV], int (&room)[NV], const uint32_t (&mx)[NV],
                                        const Group &g) {
@@ -162,7 +172,7 @@ __device__ __forceinline__ void fx_fit(longlong2 (&q)[NV][E], int (&ex)[NV], int
         uint32_t a = 0;
 #pragma unroll
         for (int m = 0; m < E; ++m)
-            a += (uint32_t)abs((int)(q[iv][m].x >> 32)) + (uint32_t)abs((int)(q[iv][m].y >> 32));
+            a += fx_mag(q[iv][m].x) + fx_mag(q[iv][m].y);
         s[iv] = (a >> 9) + 2u;
     }
     g.sum(s);
