@@ -457,16 +457,17 @@ __device__ __forceinline__ double widen(float x) {
     return __hiloint2double((int)(hi | (b & 0x80000000u)), (int)(e == 0u ? 0u : b << 29));
 }
 __device__ __forceinline__ double widen(double x) { return x; }
-// FP64 sums of a sample's local terms: three FP64 instructions a point
+// FP64 sums of a sample's local terms, |psi|^2 and (V + g/2 |psi|^2) |psi|^2: three
+// FP64 instructions a point.  (|psi|^4 alone would leave FP64's range where the energy
+// does not, g = 0 above all.)
 struct MomentSums {
-    double norm, pot, quart;
+    double hg, norm = 0.0, energy = 0.0;
+    __device__ __forceinline__ explicit MomentSums(double g) : hg(0.5 * g) {}
     template <typename R> __device__ __forceinline__ void add(R m2, R v) {
         const double d = widen(m2);
         norm += d;
-        pot = fma(widen(v), d, pot);
-        quart = fma(d, d, quart);
+        energy = fma(fma(hg, d, widen(v)), d, energy);
     }
-    __device__ __forceinline__ double energy(double g) const { return pot + 0.5 * g * quart; }
 };
 
 __device__ __forceinline__ double warp_sum(double x) {

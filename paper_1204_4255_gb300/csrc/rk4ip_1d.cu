@@ -219,7 +219,7 @@ __global__ void __launch_bounds__(PPC *(N / E), MINB) rk4ip_1d_kernel(const Para
             const int64_t s = slot_s++;
             next += p.sm.every;
             const uint64_t gs = p.step0 + n;
-            MomentSums loc{};
+            MomentSums loc(p.sm.g);
             if constexpr (NL) nonlocal(x[0], vn);
 #pragma unroll
             for (int m = 0; m < E; ++m) {
@@ -227,7 +227,7 @@ __global__ void __launch_bounds__(PPC *(N / E), MINB) rk4ip_1d_kernel(const Para
                 const int idx[3] = {j, 0, 0};
                 const R m2r = cabs2(x[0][m]);
                 loc.add(m2r, potential(p.lt, 1, idx, j, gs));
-                if constexpr (NL) loc.pot = fma(widen(half * vn[m]), widen(m2r), loc.pot);   // pair energy, counted once
+                if constexpr (NL) loc.energy = fma(widen(half * vn[m]), widen(m2r), loc.energy);   // pair energy, counted once
                 if (active && (p.sm.which & (MOM_MOD2 | MOM_MOD4)) && p.sm.per_point &&
                     XSDE_IN(s * N + j, p.sm.nsamp * N, p.status)) {
                     double *pp = p.sm.per_point + 2 * (s * N + j);
@@ -236,7 +236,7 @@ __global__ void __launch_bounds__(PPC *(N / E), MINB) rk4ip_1d_kernel(const Para
                     atomicAdd(pp + 1, m2 * m2 * p.sm.inv_paths);
                 }
             }
-            double acc[3] = {loc.norm, loc.energy(p.sm.g), 0.0};   // norm, local energy, kinetic energy
+            double acc[3] = {loc.norm, loc.energy, 0.0};   // norm, local energy, kinetic energy
             V y[1][E];
 #pragma unroll
             for (int m = 0; m < E; ++m) y[0][m] = x[0][m];

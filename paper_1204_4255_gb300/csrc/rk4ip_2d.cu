@@ -187,12 +187,12 @@ __global__ void __launch_bounds__(RowCfg<R, N1>::THREADS, RowCfg<R, N1>::MINB) r
     // (vnl: the non-local potential of f, whose pair energy 1/2 V_nl |f|^2 the
     // energy adds; nullptr without the term)
     auto sample_local = [&](const V (&f)[E], uint64_t gs, const R *vnl = nullptr) {
-        MomentSums sums{};
+        MomentSums sums(p.sm.g);
 #pragma unroll
         for (int m = 0; m < E; ++m) {
             const R m2r = cabs2(f[m]);
             sums.add(m2r, potv(m, gs));
-            if (vnl) sums.pot = fma(widen(R(0.5) * vnl[m]), widen(m2r), sums.pot);
+            if (vnl) sums.energy = fma(widen(R(0.5) * vnl[m]), widen(m2r), sums.energy);
             if (active && (p.sm.which & (MOM_MOD2 | MOM_MOD4)) && p.sm.per_point) {
                 const int64_t ip = (int64_t)p.sample_slot * p.lt.npts + (int64_t)i0 * N1 + pt_of(t + m * T);
                 if (!XSDE_IN(ip, p.sm.nsamp * p.lt.npts, p.status)) continue;
@@ -202,7 +202,7 @@ __global__ void __launch_bounds__(RowCfg<R, N1>::THREADS, RowCfg<R, N1>::MINB) r
                 atomicAdd(pp + 1, m2 * m2 * p.sm.inv_paths);
             }
         }
-        double acc[2] = {sums.norm, sums.energy(p.sm.g)};
+        double acc[2] = {sums.norm, sums.energy};
         group_sum2<T>(acc, t, scratch);
         if (t == 0 && active) {
             if ((p.sm.which & (MOM_NORM | MOM_ENERGY)) && p.sm.per_path) {

@@ -278,7 +278,7 @@ __global__ void __launch_bounds__(RowTma<N1, row_fields(MODE)>::THREADS, RowTma<
         }
         // local terms of the sample of the real-space field x[0] at global step gs
         auto sample_local = [&](uint64_t gs) {
-            MomentSums acc{};
+            MomentSums acc(p.sm.g);
 #pragma unroll
             for (int m = 0; m < E; ++m) {
                 const float m2 = cabs2(x[0][m]);
@@ -292,7 +292,7 @@ __global__ void __launch_bounds__(RowTma<N1, row_fields(MODE)>::THREADS, RowTma<
                     atomicAdd(pp + 1, d * d * p.sm.inv_paths);
                 }
             }
-            double sum[2] = {acc.norm, acc.energy(p.sm.g)};
+            double sum[2] = {acc.norm, acc.energy};
             line_sum2<T>(sum, t, line, scratch);
             if (t == 0) {
                 if ((p.sm.which & (MOM_NORM | MOM_ENERGY)) && p.sm.per_path &&

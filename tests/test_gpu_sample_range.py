@@ -1,0 +1,48 @@
+"""Norm and energy samples at the ends of the number range."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+def _problem(shape, dtype, g, basis=(), scheme=0, noise=0):
+    from paper_1204_4255_gb300 import xsde
+    lo = tuple(0.0 if basis and basis[d] else -6.0 for d in range(len(shape)))
+    P = xsde.Problem(shape, lo, (6.0,) * len(shape), dtype, basis=basis)
+    P.set_operators(g=g, pot_kind=xsde.XSDE_POT_HARMONIC if shape else xsde.XSDE_POT_NONE, omega=(1.0,) * len(shape),
+                    noise_kind=noise, seed=9, amplitude=0.02 if noise else 0.0)
+    if scheme:
+        xsde.xsde_set_scheme(P.prob, scheme)
+    return P
+
+
+def _field(shape, npaths, seed=1):
+    rng = np.random.default_rng(seed)
+    ax = [np.linspace(-6.0, 6.0, n, endpoint=False) for n in shape]
+    r2 = sum(np.meshgrid(*[x ** 2 for x in ax], indexing="ij"))
+    return np.exp(-0.3 * r2) * np.exp(0.2j * rng.standard_normal((npaths,) + shape))
+
+
+def _samples(shape, dtype, g, psi, steps=2, every=1, **more):
+    import torch
+    from paper_1204_4255_gb300 import xsde
+    P = _problem(shape, dtype, g, **more)
+    pp = torch.zeros((steps // every + 1, len(psi), 2), dtype=torch.float64, device="cuda") if every else None
+    if every:
+        P.moments(every, xsde.XSDE_MOM_NORM | xsde.XSDE_MOM_ENERGY, pp)
+    t = torch.from_numpy(np.ascontiguousarray(psi)).to(torch.complex64 if dtype == "c64" else torch.complex128).cuda()
+    P.integrate(t, 1e-4, steps)
+    P.synchronize()
+    P.close()
+    return t.cpu().numpy(), pp.cpu().numpy() if every else None
+
+
+@pytest.mark.parametrize("shape", [(64,), (512,), (32, 64), (16, 16, 32)])
+def test_energy_of_large_linear_fields(shape):
+    """without a nonlinearity the energy is quadratic in the field: 1e100 times the
+    field has 1e200 times the energy (|psi|^4 leaves FP64's range there)"""
+    psi = _field(shape, 2)
+    _, one = _samples(shape, "c128", 0.0, psi)
+    _, big = _samples(shape, "c128", 0.0, psi * 2.0 ** 332)
+    assert np.isfinite(big).all()
+    assert np.allclose(big * 2.0 ** -664, one, rtol=1e-12, atol=0)
