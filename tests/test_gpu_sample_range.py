@@ -46,3 +46,16 @@ def test_energy_of_large_linear_fields(shape):
     _, big = _samples(shape, "c128", 0.0, psi * 2.0 ** 332)
     assert np.isfinite(big).all()
     assert np.allclose(big * 2.0 ** -664, one, rtol=1e-12, atol=0)
+
+
+@pytest.mark.parametrize("shape", [(64,), (1024,), (16, 16), (64, 128), (64, 512), (16, 32, 64)])
+def test_norm_of_small_complex64_fields(shape):
+    """|psi|^2 near 1e-40 is a whole number of 2^-149; each point's is off by at most
+    two halves (its squares' and their sum's rounding) and then counts in full"""
+    amp = 2.0 ** -66
+    psi = (_field(shape, 2) * amp).astype(np.complex64).astype(np.complex128)
+    _, pp = _samples(shape, "c64", 0.0, psi)
+    want = (np.abs(psi) ** 2).reshape(2, -1).sum(1) * np.prod([12.0 / n for n in shape])
+    # and the steps leave the norm within 1e-5
+    tol = np.prod(shape) * 1.5 * 2.0 ** -149 * np.prod([12.0 / n for n in shape]) / want + 1e-5
+    assert (np.abs(pp[:, :, 0] / want - 1.0) < tol).all(), (pp[:, :, 0], want)
