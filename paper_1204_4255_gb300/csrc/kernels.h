@@ -457,6 +457,11 @@ __device__ __forceinline__ double widen(float x) {
     hi = a == 0u ? 0u : a >= 0x7f800000u ? hi | 0x7ff00000u : hi;
     return __hiloint2double((int)(hi | (b & 0x80000000u)), (int)(b << 29));
 }
+// a whole number k >= 0 below 2^24
+__device__ __forceinline__ double widen_whole(int k) {
+    const uint32_t b = __float_as_uint((float)k);
+    return __hiloint2double(k == 0 ? 0 : (int)((b >> 3) + 0x38000000u), (int)(b << 29));
+}
 __device__ __forceinline__ double widen(double x) { return x; }
 // FP64 sums of a sample's local terms, |psi|^2 and (V + g/2 |psi|^2) |psi|^2: three
 // FP64 instructions a point.  (|psi|^4 alone would leave FP64's range where the energy

@@ -266,7 +266,7 @@ __global__ void __launch_bounds__(PPC *(N / E), MINB) rk4ip_1d_kernel(const Para
                     const int kj = t + m * T, kb = kj < N / 2 ? kj : kj - N;
                     const double d = widen(cabs2(y[0][m]));
                     s0 += d;
-                    s2 = fma(widen((float)(kb * kb)), d, s2);
+                    s2 = fma(widen_whole(kb * kb), d, s2);
                 }
                 acc[2] = p.sm.h0 * s0 + p.sm.h2 * p.sm.kscale[0] * p.sm.kscale[0] * s2;
             }

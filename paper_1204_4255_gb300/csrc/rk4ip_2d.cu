@@ -639,7 +639,7 @@ __global__ void __launch_bounds__(ColCfg<R, N0>::THREADS, ColCfg<R, N0>::MINB) c
                 const int kb = kj < N0 / 2 ? kj : kj - N0;
                 const double d = widen(cabs2(f[m]));
                 s += d;
-                s2 = fma(widen((float)(kb * kb)), d, s2);
+                s2 = fma(widen_whole(kb * kb), d, s2);
             }
         }
         if constexpr (!TRIG) s = (p.sm.h0 + p.sm.h2 * kc2) * s + p.sm.h2 * p.sm.kscale[0] * p.sm.kscale[0] * s2;

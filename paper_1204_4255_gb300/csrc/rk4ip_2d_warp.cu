@@ -82,7 +82,9 @@ template <int N0, bool SPREAD, bool TRIG> struct ColW {
 // 33 us a pass in the TMA column kernel, 27 us here.
 // CONV: the density convolution of the non-local term, K2(k0, col) (read through L1)
 // in place of E0(k0), on the one field the maps describe.
-template <int N0, bool SPREAD, int KIND>
+// SAMPLE: this pass writes a sample; a template flag, so that the common pass does not
+// carry the sampling code (its registers are all taken).
+template <int N0, bool SPREAD, int KIND, bool SAMPLE>
 __global__ void __launch_bounds__(ColW<N0, SPREAD, KIND == COLW_TRIG>::THREADS, 1)
     col_pass_warp_kernel(const Params2D<float> p, const __grid_constant__ CUtensorMap mapA,
                          const __grid_constant__ CUtensorMap mapB) {
@@ -221,7 +223,6 @@ __global__ void __launch_bounds__(ColW<N0, SPREAD, KIND == COLW_TRIG>::THREADS, 
         if constexpr (SPLIT) return PairedTwiddles{tw_hi, tw_lo};
         else return PairedTwiddles{twf_s, twf_s};
     }();
-    const bool sample = !CONV && p.sample_slot >= 0;
     for (int64_t k = 0; k < mine; ++k) {
         const int s = (int)(k % NST);
         if (!wait_or_abort(full + s, (uint32_t)((k / NST) & 1), abort_flag)) {
@@ -272,7 +273,7 @@ __global__ void __launch_bounds__(ColW<N0, SPREAD, KIND == COLW_TRIG>::THREADS, 
             for (int m = 0; m < E; ++m) xq[m] = *reinterpret_cast<V *>(tb + (row_off((N0 - P * m - t) & (N0 - 1)) ^ co));
             __syncwarp();
         }
-        if (sample && vec == 0) {
+        if (SAMPLE && vec == 0) {
             // kinetic energy of a_n: sum_k Re(i L(k)) |F psi|^2 dV/(n0 n1); the
             // dimension-1 factor of exp(L dt/2) already applied is divided out
             const int col = tile * C + c;
@@ -295,12 +296,12 @@ __global__ void __launch_bounds__(ColW<N0, SPREAD, KIND == COLW_TRIG>::THREADS, 
                     const int kb = p.basis0 == 1 ? kj : N0 - kj;
                     const double d = widen((kj == 0 ? 1.0f : 2.0f) * (xr * xr + xi * xi));
                     s0 += d;
-                    s2 = fma(widen((float)(kb * kb)), d, s2);
+                    s2 = fma(widen_whole(kb * kb), d, s2);
                 } else {
                     const int kb = kj < N0 / 2 ? kj : kj - N0;
                     const double d = widen(cabs2(x[m]));
                     s0 += d;
-                    s2 = fma(widen((float)(kb * kb)), d, s2);
+                    s2 = fma(widen_whole(kb * kb), d, s2);
                 }
             }
             double sacc = (p.sm.h0 + p.sm.h2 * k1 * k1) * s0 + p.sm.h2 * p.sm.kscale[0] * p.sm.kscale[0] * s2;
@@ -344,11 +345,13 @@ __global__ void __launch_bounds__(ColW<N0, SPREAD, KIND == COLW_TRIG>::THREADS, 
     if (lane == 0) bulk_wait<0>();
 }
 
-template <int N0, bool SPREAD, int KIND>
+template <int N0, bool SPREAD, int KIND, bool SAMPLE = false>
 cudaError_t col_warp_launch_as(const Params2D<float> &p, int64_t items, const CUtensorMap &a, const CUtensorMap &b,
                                int num_sms, cudaStream_t s) {
+    if constexpr (KIND != COLW_CONV && !SAMPLE)
+        if (p.sample_slot >= 0) return col_warp_launch_as<N0, SPREAD, KIND, true>(p, items, a, b, num_sms, s);
     using Cfg = ColW<N0, SPREAD, KIND == COLW_TRIG>;
-    auto kern = col_pass_warp_kernel<N0, SPREAD, KIND>;
+    auto kern = col_pass_warp_kernel<N0, SPREAD, KIND, SAMPLE>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::SMEM);
     if (e != cudaSuccess) return e;
     const int64_t want = SPREAD ? items : num_sms;
