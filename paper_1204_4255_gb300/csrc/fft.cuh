@@ -317,10 +317,16 @@ __device__ __forceinline__ void fx_factor(double2 (&v)[NV][E], const double2 *F,
 }
 
 // forward transform, factors F (CONJ: their conjugates), and (BACK) the backward
-// transform, with one conversion in and one out where F has limbs (fex != kFxNone)
-template <int N, int E, bool BACK, bool CONJ, int NV, typename Layout, typename Sync, typename Tw, typename Group>
+// transform, with one conversion in and one out where F has limbs (fex != kFxNone).
+// seen(q, ex) looks at the spectrum on the way
+struct FxUnseen {
+    template <typename Q, typename X> __device__ __forceinline__ void operator()(const Q &, const X &) const {}
+};
+template <int N, int E, bool BACK, bool CONJ, int NV, typename Layout, typename Sync, typename Tw, typename Group,
+          typename Seen = FxUnseen>
 __device__ __forceinline__ void fx_propagate(double2 (&v)[NV][E], int t, double2 *const (&sm)[NV], const Layout &L,
-                                             const Sync &sync, const Tw &tw, const Group &g, const double2 *F, int fex) {
+                                             const Sync &sync, const Tw &tw, const Group &g, const double2 *F, int fex,
+                                             const Seen &seen = {}) {
     constexpr int T = N / E, MID = fx_middle<E>(N);
     auto at = [&](int m) { return t + m * T; };
     longlong2 q[NV][E], *qs[NV];
@@ -329,6 +335,7 @@ __device__ __forceinline__ void fx_propagate(double2 (&v)[NV][E], int t, double2
     for (int i = 0; i < NV; ++i) qs[i] = reinterpret_cast<longlong2 *>(sm[i]);
     fx_load<MID, NV, E>(v, q, ex, room, g);
     fx_fft_from<N, E, -1, 1, NV>(q, ex, room, t, qs, L, sync, tw, g);
+    seen(q, ex);
     if (fex != kFxNone) {
         if constexpr (BACK) {
             uint32_t mx[NV];

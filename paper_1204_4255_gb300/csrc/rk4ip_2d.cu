@@ -726,18 +726,21 @@ __global__ void __launch_bounds__(ColCfg<R, N0>::THREADS, ColCfg<R, N0>::MINB) c
             x[0][m] = load(p.A, t + m * T);
             x[1][m] = load(p.B, t + m * T);
         }
-        // complex128: a pass that takes no sample stays in fixed point between
-        // the two transforms
+        // complex128 stays in fixed point between the two transforms, and a sample
+        // reads the spectrum there: the field does not depend on being sampled
         if constexpr (sizeof(R) == 8 && !TRIG) {
-            if (!sample) {
-                fx_propagate<N0, E, true, false, 2>(x, t, sm2, L, sync, tw, grp, p.E0, p.E0x);
+            fx_propagate<N0, E, true, false, 2>(x, t, sm2, L, sync, tw, grp, p.E0, p.E0x, [&](const auto &q, const auto &ex) {
+                if (!sample) return;
+                V f[2][E];
+                fx_store<2, E>(q, ex, f);
+                kinetic(f[0], f[0]);
+            });
 #pragma unroll
-                for (int m = 0; m < E; ++m) {
-                    store(p.A, t + m * T, x[0][m]);
-                    store(p.B, t + m * T, x[1][m]);
-                }
-                return;
+            for (int m = 0; m < E; ++m) {
+                store(p.A, t + m * T, x[0][m]);
+                store(p.B, t + m * T, x[1][m]);
             }
+            return;
         }
         fft_line<N0, E, -1, 2>(x, t, sm2, L, sync, tw, grp);
         V xq[2][E];

@@ -1,4 +1,5 @@
-"""Norm and energy samples at the ends of the number range."""
+"""Norm and energy samples at the ends of the number range, and fields that do not
+depend on being sampled."""
 import numpy as np
 import pytest
 
@@ -59,3 +60,12 @@ def test_norm_of_small_complex64_fields(shape):
     # and the steps leave the norm within 1e-5
     tol = np.prod(shape) * 1.5 * 2.0 ** -149 * np.prod([12.0 / n for n in shape]) / want + 1e-5
     assert (np.abs(pp[:, :, 0] / want - 1.0) < tol).all(), (pp[:, :, 0], want)
+
+
+@pytest.mark.parametrize("dtype", ["c64", "c128"])
+@pytest.mark.parametrize("shape", [(64,), (512,), (16, 64), (64, 256), (128, 128)])
+def test_sampling_leaves_the_field_alone(shape, dtype):
+    psi = _field(shape, 3)
+    seen, _ = _samples(shape, dtype, 2.0, psi, steps=4, every=2)
+    unseen, _ = _samples(shape, dtype, 2.0, psi, steps=4, every=0)
+    assert np.array_equal(seen, unseen)
