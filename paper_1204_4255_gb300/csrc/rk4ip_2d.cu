@@ -534,7 +534,9 @@ template <typename R, int N0> struct ColCfg {
     static_assert(THREADS % 32 == 0, "column tiles are whole warps");
 };
 
-template <typename R, int N0, int MODE, bool TRIG = false>
+// SAMPLED: the pass may write a sample (complex128 propagation without it is its own
+// instantiation: the sampling code's registers cost it 1 %)
+template <typename R, int N0, int MODE, bool TRIG = false, bool SAMPLED = true>
 __global__ void __launch_bounds__(ColCfg<R, N0>::THREADS, ColCfg<R, N0>::MINB) col_pass_kernel(const Params2D<R> p) {
     using V = cx<R>;
     using Cfg = ColCfg<R, N0>;
@@ -556,7 +558,7 @@ __global__ void __launch_bounds__(ColCfg<R, N0>::THREADS, ColCfg<R, N0>::MINB) c
     const int64_t path = blockIdx.y;
     const int n1 = p.n1;
     const int64_t base = path * (int64_t)N0 * n1 + col;
-    const bool sample = p.sample_slot >= 0;
+    const bool sample = SAMPLED && p.sample_slot >= 0;
 #if XSDE_BOUNDS
     // the column's last element inside the field (one decision for the CTA)
     if (!__syncthreads_and(XSDE_IN(base + (int64_t)(N0 - 1) * n1, p.npaths * (int64_t)N0 * n1, p.status) &&
@@ -791,6 +793,8 @@ template <typename R, int N0, int MODE> cudaError_t col_launch(const Params2D<R>
     const size_t smem = (size_t)2 * N0 * Cfg::C * sizeof(cx<R>) + (Cfg::THREADS / 32 + 1) * sizeof(double) +
                         (sizeof(R) == 8 ? (size_t)FxColGroup<Cfg::C, Cfg::T>::kWords * 4 : 0);
     auto kern = col_pass_kernel<R, N0, MODE>;
+    if constexpr (sizeof(R) == 8 && MODE == COL_PROPAGATE)
+        if (p.sample_slot < 0) kern = col_pass_kernel<R, N0, MODE, false, false>;
     if constexpr (MODE != COL_FFT_BWD && MODE != COL_SINGLE && MODE != COL_CONV)
         if (p.basis0) kern = col_pass_kernel<R, N0, MODE, true>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
