@@ -965,9 +965,16 @@ int run_si_2d(xsde_problem *p, Params2D<R> &q, int64_t nsteps, uint64_t step0, c
         k.spec_scale = (double)q.n1 * (double)q.n1;
         return timed(p, 8, s, [&] { return launch_col_pass<R>(COL_SPECTRAL, k, s); });
     };
-    // straight into step 0 where its state is not sampled: F1 D a_0 / n1
-    const bool start = tma_rows && nsteps > 0 && !is_sample(0);
+    // straight into step 0: F1 D a_0 / n1; its sample comes from the real-space field, so
+    // that the field does not depend on being sampled there
+    const bool start = tma_rows && nsteps > 0;
     if (start) {
+        if (is_sample(0)) {
+            q.sg = step0;
+            q.sample_slot = 0;
+            XSDE_CUDA(timed(p, 2 + ROW_FFT_ONLY, s, [&] { return launch_row_pass<R>(ROW_FFT_ONLY, q, s); }), "row pass");
+            XSDE_CUDA(timed(p, 8, s, [&] { return launch_col_pass<R>(COL_SPECTRAL, q, s); }), "col pass");
+        }
         XSDE_CUDA(row(SI_START, E1h, step0, -1), "row pass");
         XSDE_CUDA(col(E0h), "col pass");
     } else {
@@ -1065,8 +1072,17 @@ int run_si_3d(xsde_problem *p, Params2D<R> &qr, Params2D<R> &q1, Params2D<R> &q0
         k.spec_scale = (double)qr.n1 * (double)qr.n1;
         return timed(p, 8, s, [&] { return launch_col_pass<R>(COL_SPECTRAL, k, s); });
     };
-    const bool start = tma_rows && nsteps > 0 && !is_sample(0);   // as run_si_2d
+    const bool start = tma_rows && nsteps > 0;   // as run_si_2d
     if (start) {
+        if (is_sample(0)) {
+            qr.sg = step0;
+            qr.sample_slot = 0;
+            XSDE_CUDA(timed(p, 2 + ROW_FFT_ONLY, s, [&] { return launch_row_pass<R>(ROW_FFT_ONLY, qr, s); }), "row pass");
+            q1.sample_slot = -1;
+            XSDE_CUDA(timed(p, 8, s, [&] { return launch_col_pass<R>(COL_FFT_FWD, q1, s); }), "col pass");
+            q0.sample_slot = 0;
+            XSDE_CUDA(timed(p, 8, s, [&] { return launch_col_pass<R>(COL_SPECTRAL, q0, s); }), "col pass");
+        }
         XSDE_CUDA(row(SI_START, false, step0, -1), "row pass");
         XSDE_CUDA(cols(false), "col pass");
     } else {

@@ -69,3 +69,12 @@ def test_sampling_leaves_the_field_alone(shape, dtype):
     seen, _ = _samples(shape, dtype, 2.0, psi, steps=4, every=2)
     unseen, _ = _samples(shape, dtype, 2.0, psi, steps=4, every=0)
     assert np.array_equal(seen, unseen)
+
+
+@pytest.mark.parametrize("dtype", ["c64", "c128"])
+@pytest.mark.parametrize("shape", [(64, 64), (64, 256), (32, 1024), (16, 32, 128)])
+def test_first_sample_leaves_a_semi_implicit_field_alone(shape, dtype):
+    psi = _field(shape, 2)
+    seen, _ = _samples(shape, dtype, 2.0, psi, steps=3, every=5, scheme=1)
+    unseen, _ = _samples(shape, dtype, 2.0, psi, steps=3, every=0, scheme=1)
+    assert np.array_equal(seen, unseen)
