@@ -247,12 +247,28 @@ void split_hi_lo(const std::complex<double> &z, float2 *hi, float2 *lo) {
     *lo = make_float2((float)(z.real() - (double)hr), (float)(z.imag() - (double)hm));
 }
 // c 2^62 as two signed limbs (fx.cuh); |c| may pass 1 by the rounding of a modulus
-void fx_limbs(double c, int *hi, int *lo) {
+void fx_limbs(long double c, int *hi, int *lo) {
     const int64_t q = std::llround(std::ldexp(c, 62));
     int64_t l = (int64_t)(int32_t)(uint32_t)(uint64_t)q;
     if (l == INT32_MIN) ++l;   // the kernels negate the limbs
     *lo = (int)l;
     *hi = (int)((q - (int64_t)(int32_t)(uint32_t)(uint64_t)q) >> 32);
+}
+// exp(-2 pi i m/n), n a multiple of 8, as limbs: the first octant in long double, the rest
+// by symmetry.  (FP64 values, off by up to 3e-16, are what the error of lines of many
+// twiddled stages would consist of: 20 steps of one mode on 64 points at 2 points a
+// thread 6.8e-15, against 4.3e-15 of FP64 transforms at 8 points a thread.)
+int4 fx_root(long m, int n) {
+    const long a = ((m % n) + n) % n, q = 4 * a / n, r = a - q * (n / 4);
+    const long double unit = 2.0L * 3.14159265358979323846264338327950288L / n;
+    const bool far = 8 * r > n;
+    const long double x = unit * (far ? n / 4 - r : r);
+    const long double c = far ? std::sin(x) : std::cos(x), sn = far ? std::cos(x) : std::sin(x);
+    int4 w;
+    // (c - i s) (-i)^q
+    fx_limbs(q == 0 ? c : q == 1 ? -sn : q == 2 ? -c : sn, &w.x, &w.y);
+    fx_limbs(q == 0 ? -sn : q == 1 ? -c : q == 2 ? sn : c, &w.z, &w.w);
+    return w;
 }
 int4 fx_limbs(const std::complex<double> &z) {
     int4 w;
@@ -285,9 +301,8 @@ template <typename V> int upload_raw(const std::vector<V> &tmp, void **dptr, cud
     return XSDE_OK;
 }
 
-// twiddle table exp(-2 pi i m/n), m < n: complex128 Q62 limbs (FP64 values for
+// twiddle table exp(-2 pi i m/n), m < n: complex128 Q62 limbs (fx_root; FP64 values for
 // the adaptive integrator); FP32 (hi, lo) split
-void make_twiddle(const std::complex<double> &z, int4 *out) { *out = fx_limbs(z); }
 void make_twiddle(const std::complex<double> &z, double2 *out) { *out = make_double2(z.real(), z.imag()); }
 void make_twiddle(const std::complex<double> &z, float4 *out) {
     float2 hi, lo;
@@ -306,26 +321,30 @@ void make_twiddle_paired(const std::complex<double> &z, float4 *out) {
 
 void make_twiddle64(const std::complex<double> &z, float4 *out) { make_twiddle(z, out); }
 
+// the table entry of exp(-2 pi i m/n)
+template <bool PAIRED = false, typename TW> void make_root(long m, int n, TW *out) {
+    if constexpr (std::is_same<TW, int4>::value) {
+        *out = fx_root(m, n);
+    } else {
+        const std::complex<double> z = std::polar(1.0, -2.0 * M_PI * (double)m / n);
+        if constexpr (PAIRED) make_twiddle_paired(z, out);
+        else make_twiddle(z, out);
+    }
+}
+
 // per-stage layout of fft.cuh: stage (Ns, R) holds w_n^(r k n/(Ns R)) at
 // [stage_table_offset(n, Ns) + (r-1) Ns + k]; n entries are allocated (the
 // table needs at most n - 1).  PAIRED (complex64): entries for fftp_*.
 template <typename R, int E = 8, bool PAIRED = false, typename TW = tw_t<R>>
 int upload_twiddles(int n, void **dptr, cudaStream_t s) {
     std::vector<TW> tmp(n);
-    auto put = [&](const std::complex<double> &z, TW *out) {
-        if constexpr (PAIRED) make_twiddle_paired(z, out);
-        else make_twiddle(z, out);
-    };
-    put(std::complex<double>(0.0, 0.0), &tmp[n - 1]);
     for (int ns = 1; ns < n;) {
         const int rad = stage_radix<E>(n / ns);
         if (ns > 1) {
             const int off = stage_table_offset<E>(n, ns);
             for (int r = 1; r < rad; ++r)
-                for (int k = 0; k < ns; ++k) {
-                    const long m = (long)r * k * (n / (ns * rad));
-                    put(std::polar(1.0, -2.0 * M_PI * (double)m / n), &tmp[off + (r - 1) * ns + k]);
-                }
+                for (int k = 0; k < ns; ++k)
+                    make_root<PAIRED>((long)r * k * (n / (ns * rad)), n, &tmp[off + (r - 1) * ns + k]);
         }
         ns *= rad;
     }
@@ -2485,16 +2504,14 @@ int static_integrate(xsde_problem *p, void *psi, double dt, int64_t nsteps, int6
         const int n = g.n[d];
         tw_t<R> *tw = reinterpret_cast<tw_t<R> *>(hdim[d]);
         V *e = reinterpret_cast<V *>(hdim[d] + kStaticTwBytes);
-        make_twiddle(std::complex<double>(0.0, 0.0), &tw[n - 1]);
+        tw[n - 1] = tw_t<R>{};   // (the stages take n - 1 at most)
         for (int ns = 1; ns < n;) {
             const int rad = stage_radix<8>(n / ns);
             if (ns > 1) {
                 const int off = stage_table_offset(n, ns);
                 for (int r = 1; r < rad; ++r)
-                    for (int k = 0; k < ns; ++k) {
-                        const long m = (long)r * k * (n / (ns * rad));
-                        make_twiddle(std::polar(1.0, -2.0 * M_PI * (double)m / n), &tw[off + (r - 1) * ns + k]);
-                    }
+                    for (int k = 0; k < ns; ++k)
+                        make_root((long)r * k * (n / (ns * rad)), n, &tw[off + (r - 1) * ns + k]);
             }
             ns *= rad;
         }

@@ -18,12 +18,14 @@
 // 256 points and more therefore start with the larger of the scales that S and
 // the first stages' own growth (their product of radices times the largest value)
 // allow, and shift by what is still needed once, between two stages, after a look
-// at the largest value there.  Measured against 113-bit arithmetic (one RK4IP step,
-// relative 2-norm, FP64 pipe / fixed point): Gaussian 4.9e-16 / 3.6e-16 at 256
-// points, 6.1e-16 / 5.1e-16 at 2048; white noise 6.0e-16 / 5.0e-16 at 512, 6.3e-16 /
-// 5.5e-16 at 1024.  Non-finite values make their whole line NaN; what lies below
-// 2^-59 of a line's largest component is truncated (an FP64 transform loses it below
-// 2^-53 of the line's norm).
+// at the largest value there.  The roots of unity are rounded to 2^-62 (fx_root in
+// api.cu): FP64 ones would be most of the error.  Measured against 64-bit-mantissa
+// arithmetic (one RK4IP step, relative 2-norm, FP64 transforms / fixed point): Gaussian
+// 3.5e-16 / 1.1e-16 at 64 points, 5.0e-16 / 1.3e-16 at 256, 6.7e-16 / 2.3e-16 at 2048;
+// white noise 3.8e-16 / 1.8e-16 at 64, 5.9e-16 / 2.4e-16 at 512, 6.4e-16 / 3.1e-16 at
+// 1024; 20 steps of one mode at 64 points 4.3e-15 / 5.7e-16.  Non-finite values make their
+// whole line NaN; what lies below 2^-59 of a line's largest component is truncated (an
+// FP64 transform loses it below 2^-53 of the line's norm).
 #pragma once
 
 #include <cstdint>

@@ -8,7 +8,7 @@ dimension, each within u log2 n of the exact one.
 import numpy as np
 import pytest
 
-from test_gpu_fixed_point import _free, _rel, _run, U
+from test_gpu_fixed_point import _field, _free, _rel, _run, CLD, U
 
 pytestmark = pytest.mark.gpu
 
@@ -55,3 +55,15 @@ def test_denormal_fields_propagate(shape):
     unit = 2.0 ** -74
     rms = float(np.sqrt((np.abs(got * 2.0 ** 1000 - ref) ** 2).mean())) / unit
     assert rms < (2.0 if len(shape) == 1 else 2.0 * np.sqrt(shape[-1])), rms
+
+
+@pytest.mark.parametrize("variant", [0, 1, 4, 5])
+@pytest.mark.parametrize("n", [16, 32, 64, 128, 256, 512])
+@pytest.mark.parametrize("kind", ["noise", "mode"])
+def test_forward_and_backward_transforms_are_inverses(n, variant, kind):
+    """With L = 0 a step is two forward / backward pairs.  Each pair rounds to FP64 once
+    (0.42 u rms of the values), and its two transforms round integers whose unit is at most
+    half a unit of FP64 at the line's size (0.3 u each): 0.9 u for two pairs, in quadrature.
+    2 u is the bound."""
+    psi = _field(kind, (16, n))
+    assert _rel(_run(psi, 10.0, 0j, 0j, 1e-4, variant), psi.astype(CLD)) < 2 * U
