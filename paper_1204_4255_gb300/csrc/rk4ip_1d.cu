@@ -518,13 +518,18 @@ template <typename R> cudaError_t launch_rk4ip_1d(int n, int variant, const Para
 int rk4ip_1d_variants() { return 7; }
 int rk4ip_1d_elems(int variant) { return variant == 4 ? 4 : variant == 5 ? 2 : 8; }
 // The shape that variant 0 stands for: few paths are spread over more threads
-// (4 or 2 points each), ensembles keep 8 points a thread.  Measured (GB300, us a
-// step; 8 points capped at 128 registers / uncapped / 4 points / 2 points):
-//   complex64    32 points,  152 paths: 3.28 / 3.02 / 1.57 / 1.14;  4096: 3.30 / 3.01 / 2.34 / 3.05
-//               128 points,  304 paths: 2.75 / 2.79 / 1.56 / 2.23;  4096: 7.66 / 8.08 / 7.31 / 18.1
-//               256 points,  304 paths: 2.69 / 2.73 / 2.01 / 3.32;  1216: 4.27 / 4.07 / 5.06 / 10.6
-//               512 points,  152 paths: 3.11 capped / 2.68 / 2.41 / 3.48;  1216: 8.46 / 9.06 / 12.6 / 21.7
-//              1024 points,  152 paths: 3.87 uncapped / 4.06 / 6.50;   1216: 21.8 / 23.6 / 32.6 / 52.3
+// (4 or 2 points each), ensembles keep 8 points a thread: uncapped while every path
+// is resident at 255 registers (2048 points an SM), capped at 128 beyond.  Measured
+// (GB300, us a step; 8 points capped / uncapped / 4 points / 2 points):
+//   complex64    32 points,  152 paths: 2.58 / 2.29 / 1.19 / 1.05; 65536: 20.2 / 21.6 / 19.0 / 33.2
+//                64 points, 8192 paths: 5.62 / 5.55 / 5.34 / 10.8; 16384: 9.58 / 9.63 / 10.5 / 20.8
+//               128 points,  304 paths: 3.15 / 2.82 / 1.66 / 1.79;  4096: 7.58 / 7.76 / 7.39 / 15.3;
+//                                                                  16384: 25.3 / 26.8 / 27.9 / 58.9
+//               256 points,  304 paths: 3.29 / 2.99 / 1.99 / 2.66;   608: 3.28 / 2.99 / 2.76 / 4.80;
+//                                                                   1216: 4.48 / 4.12 / 4.83 / 9.57
+//               512 points,  152 paths: 3.23 / 3.08 / 2.40 / 3.45;  1216: 8.23 / 8.91 / 12.5 / 21.7
+//              1024 points,  304 paths: 6.25 / 5.88 / 8.03 / 13.0;  1216: 21.2 / 23.3 / 32.1 / 51.9
+//              2048 points,  152 paths: 7.23 / 7.02 / 8.16 / 14.0;   304: 12.0 / 14.0 / 16.3 / 27.9
 //   complex128  256 points,    1 path :  41 /  40 /  21 /  11;      4096: 136 / 171 / 126 / 133
 //              1024 points,    1 path :  63 /  61 /  30 /  40;      4096: 600 / 1006 / 841 / 1083
 int rk4ip_1d_default(bool fp64, int n, int64_t npaths, int num_sms) {
@@ -533,11 +538,11 @@ int rk4ip_1d_default(bool fp64, int n, int64_t npaths, int num_sms) {
         if (n <= 256) return pts < (int64_t)4096 * num_sms ? 5 : 4;
         return npaths <= num_sms ? 4 : 6;   // variant 6: capped in complex128
     }
-    if (n <= 32 && pts <= (int64_t)512 * num_sms) return 5;
-    if (n <= 128) return 4;
-    if (n <= 256) return npaths <= 2 * (int64_t)num_sms ? 4 : 0;
+    if (n <= 32) return pts <= (int64_t)512 * num_sms ? 5 : 4;
+    if (n <= 128 && pts <= (int64_t)3500 * num_sms) return 4;
+    if (n <= 256 && npaths <= 4 * (int64_t)num_sms) return 4;
     if (n <= 512 && npaths <= num_sms) return 4;
-    return npaths <= 2 * (int64_t)num_sms ? 6 : 0;   // variant 6: uncapped in complex64
+    return pts <= (int64_t)2048 * num_sms ? 6 : 0;   // variant 6: uncapped in complex64
 }
 #endif
 XSDE_1D_UNIT(float)
