@@ -280,10 +280,10 @@ int4 fx_limbs(const std::complex<double> &z) {
 // largest modulus takes the limbs' whole range.  The limbs have one absolute
 // precision, so a table whose moduli differ by more than 4 (strong damping or
 // growth over the spectrum) keeps FP64 products: kFxNone.
-int fx_exponent(const std::vector<std::complex<double>> &h) {
+int fx_exponent(const std::complex<double> *h, size_t n) {
     double big = 0.0, small = HUGE_VAL;
-    for (const auto &z : h) {
-        const double a = std::abs(z);
+    for (size_t i = 0; i < n; ++i) {
+        const double a = std::abs(h[i]);
         if (!std::isfinite(a)) return kFxNone;
         big = std::max(big, a);
         small = std::min(small, a);
@@ -365,25 +365,25 @@ int upload_twiddles_2stage(int n, int E, void **dptr, cudaStream_t s) {
 
 // factor table [2 n]: complex64 hi [n], lo [n]; complex128 values [n], limbs [n]
 // (zero, and *fex = kFxNone, where fx_exponent gives none)
-void fill_factors(const std::vector<std::complex<double>> &h, float2 *out, int *fex) {
-    for (size_t i = 0; i < h.size(); ++i) split_hi_lo(h[i], &out[i], &out[h.size() + i]);
+void fill_factors(const std::complex<double> *h, size_t n, float2 *out, int *fex) {
+    for (size_t i = 0; i < n; ++i) split_hi_lo(h[i], &out[i], &out[n + i]);
     if (fex) *fex = kFxNone;
 }
-void fill_factors(const std::vector<std::complex<double>> &h, double2 *out, int *fex) {
+void fill_factors(const std::complex<double> *h, size_t n, double2 *out, int *fex) {
     static_assert(sizeof(int4) == sizeof(double2), "limbs take the place of lo");
-    const int e = fex ? fx_exponent(h) : kFxNone;
-    for (size_t i = 0; i < h.size(); ++i) {
+    const int e = fex ? fx_exponent(h, n) : kFxNone;
+    for (size_t i = 0; i < n; ++i) {
         out[i] = make_double2(h[i].real(), h[i].imag());
         const int4 w = e == kFxNone ? make_int4(0, 0, 0, 0)
                                     : fx_limbs(std::complex<double>(std::ldexp(h[i].real(), -e), std::ldexp(h[i].imag(), -e)));
-        std::memcpy(&out[h.size() + i], &w, sizeof w);
+        std::memcpy(&out[n + i], &w, sizeof w);
     }
     if (fex) *fex = e;
 }
 template <typename V>
 int upload(const std::vector<std::complex<double>> &h, void **dptr, cudaStream_t s, int *fex = nullptr) {
     std::vector<V> tmp(2 * h.size());
-    fill_factors(h, tmp.data(), fex);
+    fill_factors(h.data(), h.size(), tmp.data(), fex);
     return upload_raw(tmp, dptr, s);
 }
 
@@ -2488,8 +2488,9 @@ int static_arrays_for(int dev, StaticArrays **out) {
     return XSDE_OK;
 }
 
-// host staging of the tables (per thread, no heap)
+// host staging of the tables and of one dimension's factors (per thread, no heap)
 thread_local unsigned char t_host_tables[kStaticTableBytes];
+thread_local std::complex<double> t_host_factors[kStaticMaxN];
 
 template <typename R>
 int static_integrate(xsde_problem *p, void *psi, double dt, int64_t nsteps, int64_t npaths, int64_t path_offset,
@@ -2515,14 +2516,13 @@ int static_integrate(xsde_problem *p, void *psi, double dt, int64_t nsteps, int6
             }
             ns *= rad;
         }
-        thread_local std::vector<std::complex<double>> f;   // grows to the longest dimension once
-        f.resize(n);
+        std::complex<double> *f = t_host_factors;
         for (int i = 0; i < n; ++i) {
             const double k = kval(g, d, i);
             f[i] = d == 0 ? std::exp((c0 + c2 * (k * k)) * (0.5 * dt)) / ((double)g.n[0] * g.n[1])
                           : std::exp(c2 * (k * k) * (0.5 * dt));
         }
-        fill_factors(f, e, &fex[d]);
+        fill_factors(f, n, e, &fex[d]);
     }
     XSDE_CUDA(cudaMemcpyAsync(sa.tables, t_host_tables, kStaticTableBytes, cudaMemcpyHostToDevice, s),
               "xsde_integrate_static_scratch: tables");
