@@ -643,14 +643,24 @@ int ensure_scratch(xsde_problem *p, size_t need, cudaStream_t s) {
         p->d_scratch = nullptr;
         p->scratch_bytes = 0;
     }
-    XSDE_CUDA(cudaMalloc(&p->d_scratch, need), "cudaMalloc(scratch)");
+    cudaError_t e = cudaMalloc(&p->d_scratch, need);
+    if (e == cudaErrorMemoryAllocation && p->d_noise) {   // the normals can be drawn again: their buffer goes first
+        cudaGetLastError();
+        XSDE_CUDA(cudaStreamSynchronize(s), "cudaStreamSynchronize(scratch)");
+        cudaFree(p->d_noise);
+        p->d_noise = nullptr;
+        p->noise_bytes = 0;
+        e = cudaMalloc(&p->d_scratch, need);
+    }
+    XSDE_CUDA(e, "cudaMalloc(scratch)");
     p->scratch_bytes = need;
     return XSDE_OK;
 }
 
 // The buffer of a noisy 2D / 3D RK4IP step's scaled normals (Params2D::Z), grown and
 // never shrunk; nullptr (every pass draws for itself) for other problems, where it
-// cannot be had, or where the stream is being captured and it would have to grow.
+// would take more than a quarter of the memory that is free (other problems' fields come
+// first), or where the stream is being captured and it would have to grow.
 void *noise_buffer(xsde_problem *p, int64_t npaths, cudaStream_t s) {
     if (p->noise.kind == XSDE_NOISE_NONE || p->scheme != XSDE_SCHEME_RK4IP || p->grid.ndim < 2) return nullptr;
     const size_t real = elem_bytes(p->dtype) / 2;
@@ -658,6 +668,11 @@ void *noise_buffer(xsde_problem *p, int64_t npaths, cudaStream_t s) {
     if (p->noise_bytes >= need) return p->d_noise;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    size_t avail = 0, total = 0;
+    if (cudaMemGetInfo(&avail, &total) != cudaSuccess || need > (avail + p->noise_bytes) / 4) {
         cudaGetLastError();
         return nullptr;
     }
