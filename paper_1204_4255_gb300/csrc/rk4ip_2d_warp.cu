@@ -56,7 +56,7 @@ template <int N0, bool SPREAD, bool TRIG> struct ColW {
     // 64 x 512^2: 136 -> 120 us; 16 warps with one stage each 163 us.  SPREAD: one
     // group, for fields of few tiles.
     // (TRIG holds the partner values too: 8 to 12 warps)
-    static constexpr int GROUPS = SPREAD ? 1 : TRIG ? (N0 == 512 ? 2 : N0 == 256 ? 3 : 6) : N0 == 512 ? 3 : N0 == 256 ? 4 : 8;
+    static constexpr int GROUPS = SPREAD ? 1 : TRIG ? (N0 == 256 ? 3 : 6) : N0 == 512 ? 3 : N0 == 256 ? 4 : 8;
     static constexpr int THREADS = GROUPS * NW * 32;
     static constexpr int NST = N0 == 512 ? 2 : 3;        // shared-memory stages of a group
     static constexpr int BOXR = N0 < 256 ? N0 : 256;           // tensor-copy box rows
@@ -363,7 +363,10 @@ cudaError_t col_warp_launch(const Params2D<float> &p, const CUtensorMap &a, cons
                             cudaStream_t s) {
     const int64_t items = p.npaths * (int64_t)(p.n1 / WARP_COL_C) * (p.single_field ? 1 : 2);
     if (conv) return col_warp_launch_as<N0, false, COLW_CONV>(p, items, a, b, num_sms, s);
-    if (p.basis0) return col_warp_launch_as<N0, false, COLW_TRIG>(p, items, a, b, num_sms, s);
+    if (p.basis0) {
+        if constexpr (N0 == 128 || N0 == 256) return col_warp_launch_as<N0, false, COLW_TRIG>(p, items, a, b, num_sms, s);
+        else return cudaErrorInvalidValue;   // (col_pass_kind takes other passes)
+    }
     return items <= 2 * (int64_t)num_sms ? col_warp_launch_as<N0, true, COLW_PLAIN>(p, items, a, b, num_sms, s)
                                          : col_warp_launch_as<N0, false, COLW_PLAIN>(p, items, a, b, num_sms, s);
 }
