@@ -31,8 +31,10 @@
  *     step n at point j of global path p comes from counter (j, p, n+1, 0) and
  *     key (seed_lo, seed_hi) through u = (x + 0.5) 2^-32 and Box-Muller:
  *     z0 = sqrt(-2 ln u0) cos(2 pi u1), z1 = sqrt(-2 ln u0) sin(2 pi u1).
- *     Real noise uses z0, complex noise (z0 + i z1)/sqrt(2).  Results are
- *     therefore independent of launch shape and of how paths are split.
+ *     Real noise uses z0, complex noise (z0 + i z1)/sqrt(2).  The noise is
+ *     therefore independent of launch shape and of how paths are split, and a
+ *     path's result is too, to rounding: kernel variant 0 picks its launch
+ *     shape by the number of paths as well (xsde_set_kernel_variant).
  *
  * Errors: every call returns an xsde_status; on failure xsde_last_error()
  * returns a thread-local message.  No C++ exception crosses this boundary.
@@ -413,13 +415,21 @@ int xsde_synchronize(xsde_problem *prob, void *stream);
  *     complex128; variant 6 is that shape with the other choice; variant 0 takes
  *     one of these shapes by precision, length and number of paths (few paths
  *     are spread over more threads); where a bound applies a variant repeats
- *     another;
+ *     another.  Shapes of 8, 4 and 2 points round differently, so that a path
+ *     agrees bit for bit between ensembles of different sizes (the shares of an
+ *     ensemble split over ranks) only where they run with the same variant
+ *     other than 0;
  *   2D and 3D lattices (4 variants): 0 uses, in complex64, the persistent
  *     TMA-pipelined row pass (lines of 64..1024 points) and the column pass
  *     with warp-synchronous two-stage transforms (columns of 64..512 points,
  *     a multiple of 8 columns; else the TMA column pass), 1 forces the generic
  *     passes, 2 uses the TMA row passes and the generic column passes, 3 the
- *     TMA row and TMA column passes;
+ *     TMA row and TMA column passes.  Variant 0's choice depends on the number of
+ *     paths for cosine / sine columns of 128 and 256 points on 2D lattices only
+ *     (the warp pass where there are more tiles than SMs, else the TMA pass).
+ *     The variants are those of RK4IP steps without the non-local term: the
+ *     semi-implicit scheme and the non-local term have one launch shape, by
+ *     lattice and alignment, whatever variant was set before;
  *   0D lattices (1 variant).
  * Out-of-range variants report XSDE_EINVAL.  xsde_autotune picks one by
  * timing. */

@@ -3,8 +3,10 @@
 Stochastic paths and independent instances need no exchange while they are
 integrated (XMDS2 runs its paths as separate MPI processes, Sec. 2.5): each
 rank advances a contiguous range of global path indices, and the Philox
-counters carry the global index (``path_offset``), so a path's noise, and
-therefore its result, does not depend on how the ensemble is split.  The only
+counters carry the global index (``path_offset``), so a path's noise does not
+depend on how the ensemble is split, and its result does not beyond rounding
+(bit for bit where every rank sets the same kernel variant other than 0: the
+default also goes by the number of local paths).  The only
 collective is the combination of the ensemble moments, once per sample set,
 in FP64.  Works with any process group (NCCL for device tensors, gloo for
 host tensors); no arithmetic of the time step happens here.

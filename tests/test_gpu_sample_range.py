@@ -1,12 +1,12 @@
-"""Norm and energy samples at the ends of the number range, and fields that do not
-depend on being sampled."""
+"""Norm and energy samples at the ends of the number range, fields that do not depend on
+being sampled, and paths in ensembles of different sizes."""
 import numpy as np
 import pytest
 
 pytestmark = pytest.mark.gpu
 
 
-def _problem(shape, dtype, g, basis=(), scheme=0, noise=0):
+def _problem(shape, dtype, g, basis=(), scheme=0, noise=0, variant=0):
     from paper_1204_4255_gb300 import xsde
     lo = tuple(0.0 if basis and basis[d] else -6.0 for d in range(len(shape)))
     P = xsde.Problem(shape, lo, (6.0,) * len(shape), dtype, basis=basis)
@@ -14,6 +14,8 @@ def _problem(shape, dtype, g, basis=(), scheme=0, noise=0):
                     noise_kind=noise, seed=9, amplitude=0.02 if noise else 0.0)
     if scheme:
         xsde.xsde_set_scheme(P.prob, scheme)
+    if variant:
+        xsde.xsde_set_kernel_variant(P.prob, variant)
     return P
 
 
@@ -78,3 +80,22 @@ def test_first_sample_leaves_a_semi_implicit_field_alone(shape, dtype):
     seen, _ = _samples(shape, dtype, 2.0, psi, steps=3, every=5, scheme=1)
     unseen, _ = _samples(shape, dtype, 2.0, psi, steps=3, every=0, scheme=1)
     assert np.array_equal(seen, unseen)
+
+
+@pytest.mark.parametrize("dtype", ["c64", "c128"])
+@pytest.mark.parametrize("shape,npaths,basis,variant", [((32,), 3000, (), 4), ((64,), 12000, (), 4), ((256,), 3000, (), 1),
+                                                        ((512,), 320, (), 5), ((1024,), 310, (), 4), ((128, 64), 40, (1, 0), 3),
+                                                        ((256, 128), 20, (2, 0), 3), ((64, 64), 32, (), 0)])
+def test_a_path_and_the_ensemble_it_runs_in(shape, npaths, basis, variant, dtype):
+    """Variant 0 takes its launch shape by the number of paths too, so a path alone and
+    in a large ensemble agree to rounding (two steps, each within 1e-6 or 1e-14); with a
+    variant set, and on Fourier lattices of 2D, bit for bit."""
+    psi = np.ascontiguousarray(np.broadcast_to(_field(shape, 4), (4,) + shape))
+    many = np.tile(psi, (npaths // 4,) + (1,) * len(shape))
+    for v in {0, variant}:
+        whole, _ = _samples(shape, dtype, 2.0, many, every=0, basis=basis, variant=v)
+        part, _ = _samples(shape, dtype, 2.0, psi, every=0, basis=basis, variant=v)
+        for got in (whole[:4], whole[-4:]):
+            assert np.linalg.norm(got - part) <= (1e-6 if dtype == "c64" else 1e-14) * np.linalg.norm(part)
+            if v or (len(shape) > 1 and not basis):
+                assert np.array_equal(got, part)
