@@ -176,7 +176,10 @@ __global__ void __launch_bounds__(PPC *(N / E), MINB) rk4ip_1d_kernel(const Para
     // D = F^-1 exp(L dt/2) F on NV vectors
     auto propagate = [&](auto &v) {
         constexpr int NV = sizeof(v) / sizeof(v[0]);
-        const ExchangeLayout<V, NV> X{};
+        // (one warp a path: two 8-byte slots a pair are the faster ones from 128 points on, us a
+        // step of 2704 x 128 cosine 8.68 -> 8.09, 2704 x 256 sine 14.2 -> 13.3, 4096 x 256 13.4 ->
+        // 13.3; 2704 x 64 cosine 3.97 against 4.53)
+        const std::conditional_t<(T <= 32 && N >= 128), LineLayout<V>, ExchangeLayout<V, NV>> X{};
         auto with = [&](V *const (&sm)[NV]) {
             if constexpr (FX && !TRIG) {
                 fx_propagate<N, E, true, false, NV>(v, t, sm, X, sync, tw, grp, p.Etab, p.Ex);
