@@ -1260,7 +1260,7 @@ int run_integrate(xsde_problem *p, void *psi, double dt, int64_t nsteps, int64_t
         q.Ex = p->E_x[0];
         const bool shape0 = p->scheme != XSDE_SCHEME_RK4IP || p->nonlocal || g.basis[0] != XSDE_BASIS_FOURIER;
         int variant = p->kernel_variant;
-        if (variant == 0 && !shape0) variant = rk4ip_1d_default(sizeof(R) == 8, g.n[0], npaths, p->num_sms);
+        if (variant == 0 && !shape0) variant = rk4ip_1d_default(sizeof(R) == 8, lt.noise != NM_NONE, g.n[0], npaths, p->num_sms);
         const int elems = shape0 ? 8 : rk4ip_1d_elems(variant);
         q.tw = static_cast<const tw_t<R> *>(elems == 8 ? p->d_tw[0] : p->d_tw1d[elems == 4 ? 0 : 1]);
         q.lt = lt;

@@ -86,7 +86,7 @@ int measure_fma_peaks(double *fp32_tflops, double *fp64_tflops);
 cudaError_t launch_wait_timeout(uint64_t wait_ns, int *status, cudaStream_t s);
 int rk4ip_1d_variants();
 int rk4ip_1d_elems(int variant);
-int rk4ip_1d_default(bool fp64, int n, int64_t npaths, int num_sms);
+int rk4ip_1d_default(bool fp64, bool noise, int n, int64_t npaths, int num_sms);
 template <typename R> cudaError_t launch_rk4ip_1d(int n, int variant, const Params1D<R> &p, cudaStream_t s);
 
 // --------------------------------------------------------------------------

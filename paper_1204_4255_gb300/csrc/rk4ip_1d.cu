@@ -535,17 +535,20 @@ int rk4ip_1d_elems(int variant) { return variant == 4 ? 4 : variant == 5 ? 2 : 8
 //              2048 points,  152 paths: 7.23 / 7.02 / 8.16 / 14.0;   304: 12.0 / 14.0 / 16.3 / 27.9
 //   complex128  256 points,    1 path :  41 /  40 /  21 /  11;      4096: 136 / 171 / 126 / 133
 //              1024 points,    1 path :  63 /  61 /  30 /  40;      4096: 600 / 1006 / 841 / 1083
-int rk4ip_1d_default(bool fp64, int n, int64_t npaths, int num_sms) {
+// (With noise, whose draws hide the exchanges, 4 points stay ahead at 128 points: 8192 paths
+// 17.3 us a step against 19.0 capped.)
+int rk4ip_1d_default(bool fp64, bool noise, int n, int64_t npaths, int num_sms) {
     const int64_t pts = npaths * n;
     if (fp64) {
         if (n <= 256) return pts < (int64_t)4096 * num_sms ? 5 : 4;
         return npaths <= num_sms ? 4 : 6;   // variant 6: capped in complex128
     }
     if (n <= 32) return pts <= (int64_t)512 * num_sms ? 5 : 4;
-    if (n <= 128 && pts <= (int64_t)3500 * num_sms) return 4;
-    if (n <= 256 && npaths <= 4 * (int64_t)num_sms) return 4;
+    if (n <= 128 && (noise || pts <= (int64_t)3500 * num_sms)) return 4;
+    if (n <= 256 && npaths <= (noise ? 2 : 4) * (int64_t)num_sms) return 4;
     if (n <= 512 && npaths <= num_sms) return 4;
-    return pts <= (int64_t)2048 * num_sms ? 6 : 0;   // variant 6: uncapped in complex64
+    // variant 6: uncapped in complex64
+    return pts <= (int64_t)2048 * num_sms && (!noise || npaths <= 2 * (int64_t)num_sms) ? 6 : 0;
 }
 #endif
 XSDE_1D_UNIT(float)

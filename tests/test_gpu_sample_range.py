@@ -90,7 +90,7 @@ def test_a_path_and_the_ensemble_it_runs_in(shape, npaths, basis, variant, dtype
     """Variant 0 takes its launch shape by the number of paths too, so a path alone and
     in a large ensemble agree to rounding (two steps, each within 1e-6 or 1e-14); with a
     variant set, and on Fourier lattices of 2D, bit for bit."""
-    psi = np.ascontiguousarray(np.broadcast_to(_field(shape, 4), (4,) + shape))
+    psi = _field(shape, 4)
     many = np.tile(psi, (npaths // 4,) + (1,) * len(shape))
     for v in {0, variant}:
         whole, _ = _samples(shape, dtype, 2.0, many, every=0, basis=basis, variant=v)
