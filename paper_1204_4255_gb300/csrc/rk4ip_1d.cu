@@ -178,8 +178,9 @@ __global__ void __launch_bounds__(PPC *(N / E), MINB) rk4ip_1d_kernel(const Para
         constexpr int NV = sizeof(v) / sizeof(v[0]);
         // (one warp a path: two 8-byte slots a pair are the faster ones from 128 points on, us a
         // step of 2704 x 128 cosine 8.68 -> 8.09, 2704 x 256 sine 14.2 -> 13.3, 4096 x 256 13.4 ->
-        // 13.3; 2704 x 64 cosine 3.97 against 4.53)
-        const std::conditional_t<(T <= 32 && N >= 128), LineLayout<V>, ExchangeLayout<V, NV>> X{};
+        // 13.3; 2704 x 64 cosine 3.97 against 4.53, 8192 x 128 noisy at 4 points 17.5 against 17.9)
+        constexpr bool NARROW = T <= 32 && N >= 128 && !(NOISE && E < 8);
+        const std::conditional_t<NARROW, LineLayout<V>, ExchangeLayout<V, NV>> X{};
         auto with = [&](V *const (&sm)[NV]) {
             if constexpr (FX && !TRIG) {
                 fx_propagate<N, E, true, false, NV>(v, t, sm, X, sync, tw, grp, p.Etab, p.Ex);
@@ -525,11 +526,11 @@ int rk4ip_1d_elems(int variant) { return variant == 4 ? 4 : variant == 5 ? 2 : 8
 // is resident at 255 registers (2048 points an SM), capped at 128 beyond.  Measured
 // (GB300, us a step; 8 points capped / uncapped / 4 points / 2 points):
 //   complex64    32 points,  152 paths: 2.58 / 2.29 / 1.19 / 1.05; 65536: 20.2 / 21.6 / 19.0 / 33.2
-//                64 points, 8192 paths: 5.62 / 5.55 / 5.34 / 10.8; 16384: 9.58 / 9.63 / 10.5 / 20.8
-//               128 points,  304 paths: 3.15 / 2.82 / 1.66 / 1.79;  4096: 7.58 / 7.76 / 7.39 / 15.3;
-//                                                                  16384: 25.3 / 26.8 / 27.9 / 58.9
-//               256 points,  304 paths: 3.29 / 2.99 / 1.99 / 2.66;   608: 3.28 / 2.99 / 2.76 / 4.80;
-//                                                                   1216: 4.48 / 4.12 / 4.83 / 9.57
+//                64 points, 8192 paths: 5.31 / 5.47 / 5.28 / 10.8; 16384: 8.95 / 9.45 / 10.4 / 20.8
+//               128 points,  304 paths: 2.59 / 2.37 / 1.51 / 1.79;  4096: 7.33 / 7.44 / 7.21 / 15.4;
+//                                                                  16384: 24.5 / 25.7 / 27.3 / 59.0
+//               256 points,  304 paths: 2.68 / 2.47 / 1.99 / 2.65;   608: 2.67 / 2.48 / 2.77 / 4.81;
+//                                                                   2432: 7.67 / 7.75 / 9.98 / 19.1
 //               512 points,  152 paths: 3.23 / 3.08 / 2.40 / 3.45;  1216: 8.23 / 8.91 / 12.5 / 21.7
 //              1024 points,  304 paths: 6.25 / 5.88 / 8.03 / 13.0;  1216: 21.2 / 23.3 / 32.1 / 51.9
 //              2048 points,  152 paths: 7.23 / 7.02 / 8.16 / 14.0;   304: 12.0 / 14.0 / 16.3 / 27.9
@@ -545,7 +546,7 @@ int rk4ip_1d_default(bool fp64, bool noise, int n, int64_t npaths, int num_sms) 
     }
     if (n <= 32) return pts <= (int64_t)512 * num_sms ? 5 : 4;
     if (n <= 128 && (noise || pts <= (int64_t)3500 * num_sms)) return 4;
-    if (n <= 256 && npaths <= (noise ? 2 : 4) * (int64_t)num_sms) return 4;
+    if (n <= 256 && npaths <= 2 * (int64_t)num_sms) return 4;
     if (n <= 512 && npaths <= num_sms) return 4;
     // variant 6: uncapped in complex64
     return pts <= (int64_t)2048 * num_sms && (!noise || npaths <= 2 * (int64_t)num_sms) ? 6 : 0;
