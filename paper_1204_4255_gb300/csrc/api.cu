@@ -246,24 +246,36 @@ void split_hi_lo(const std::complex<double> &z, float2 *hi, float2 *lo) {
     *hi = make_float2(hr, hm);
     *lo = make_float2((float)(z.real() - (double)hr), (float)(z.imag() - (double)hm));
 }
-// c 2^62 as two signed limbs (fx.cuh); |c| may pass 1 by the rounding of a modulus
-void fx_limbs(long double c, int *hi, int *lo) {
-    const int64_t q = std::llround(std::ldexp(c, 62));
+// q = c 2^62 as two signed limbs (fx.cuh); |c| may pass 1 by the rounding of a modulus
+void fx_limbs(int64_t q, int *hi, int *lo) {
     int64_t l = (int64_t)(int32_t)(uint32_t)(uint64_t)q;
     if (l == INT32_MIN) ++l;   // the kernels negate the limbs
     *lo = (int)l;
     *hi = (int)((q - (int64_t)(int32_t)(uint32_t)(uint64_t)q) >> 32);
 }
-// exp(-2 pi i m/n), n a multiple of 8, as limbs: the first octant in long double, the rest
-// by symmetry.  (FP64 values, off by up to 3e-16, are what the error of lines of many
+// cos and sin of 2 pi r/2048, r <= 256, in Q62, from long double (a library call each where
+// that is software: once a process, and every length's roots are among them)
+struct FxOctant {
+    static constexpr int N = 2048;
+    int64_t c[N / 8 + 1], s[N / 8 + 1];
+    FxOctant() {
+        for (int r = 0; r <= N / 8; ++r) {
+            const long double x = 2.0L * 3.14159265358979323846264338327950288L * r / N;
+            c[r] = std::llround(std::ldexp(std::cos(x), 62));
+            s[r] = std::llround(std::ldexp(std::sin(x), 62));
+        }
+    }
+};
+// exp(-2 pi i m/n), n a power of two in [16, 2048], as limbs: the first octant, the rest by
+// symmetry.  (FP64 values, off by up to 3e-16, are what the error of lines of many
 // twiddled stages would consist of: 20 steps of one mode on 64 points at 2 points a
 // thread 6.8e-15, against 4.3e-15 of FP64 transforms at 8 points a thread.)
 int4 fx_root(long m, int n) {
-    const long a = ((m % n) + n) % n, q = 4 * a / n, r = a - q * (n / 4);
-    const long double unit = 2.0L * 3.14159265358979323846264338327950288L / n;
-    const bool far = 8 * r > n;
-    const long double x = unit * (far ? n / 4 - r : r);
-    const long double c = far ? std::sin(x) : std::cos(x), sn = far ? std::cos(x) : std::sin(x);
+    static const FxOctant oct;
+    constexpr int N = FxOctant::N;
+    const int a = (int)((m % n + n) % n) * (N / n), q = a / (N / 4), r = a % (N / 4);
+    const bool far = r > N / 8;
+    const int64_t c = far ? oct.s[N / 4 - r] : oct.c[r], sn = far ? oct.c[N / 4 - r] : oct.s[r];
     int4 w;
     // (c - i s) (-i)^q
     fx_limbs(q == 0 ? c : q == 1 ? -sn : q == 2 ? -c : sn, &w.x, &w.y);
@@ -272,8 +284,8 @@ int4 fx_root(long m, int n) {
 }
 int4 fx_limbs(const std::complex<double> &z) {
     int4 w;
-    fx_limbs(z.real(), &w.x, &w.y);
-    fx_limbs(z.imag(), &w.z, &w.w);
+    fx_limbs((int64_t)std::llround(std::ldexp(z.real(), 62)), &w.x, &w.y);
+    fx_limbs((int64_t)std::llround(std::ldexp(z.imag(), 62)), &w.z, &w.w);
     return w;
 }
 // Exponent e for a table of complex128 factors as limbs, f = limbs 2^e: the
