@@ -25,7 +25,7 @@
 // white noise 3.8e-16 / 1.8e-16 at 64, 5.9e-16 / 2.4e-16 at 512, 6.4e-16 / 3.1e-16 at
 // 1024; 20 steps of one mode at 64 points 4.3e-15 / 5.7e-16.  Non-finite values make their
 // whole line NaN; what lies below 2^-59 of a line's largest component is truncated (an
-// FP64 transform loses it below 2^-53 of the line's norm).
+// FP64 transform loses it below 2^-53 of the line's norm), and denormals count as zero.
 #pragma once
 
 #include <cstdint>
@@ -88,11 +88,13 @@ constexpr int kFxTop = 59;        // bit that the largest exponent's leading one
 
 __device__ __forceinline__ uint32_t fx_hi(double v) { return (uint32_t)__double2hiint(v); }
 
-// v 2^-(em - 1023 - kFxTop), truncated; em, the line's largest exponent field, is at
-// least kFxTop + 2, so that field 0 (zeros, and denormals, far below) is shifted out
+// v 2^-(em - 1023 - kFxTop), truncated (the exponent field of v is at most em;
+// field 0, zeros and denormals, gives 0: bringing denormals into range first costs every
+// line 1 to 5 %, a branch between the reduction and the conversions)
 __device__ __forceinline__ long long fx_from(double v, int em) {
     const long long b = __double_as_longlong(v);
-    const int r = em - (int)((fx_hi(v) >> 20) & 0x7ffu);
+    const int e = (int)((fx_hi(v) >> 20) & 0x7ffu);
+    const int r = e ? em - e : 64;
     unsigned long long m = (((unsigned long long)b & 0xfffffffffffffull) | 0x10000000000000ull) << (kFxTop - 52);
     asm("shr.u64 %0, %0, %1;" : "+l"(m) : "r"(r));   // amounts past 63 give 0
     const long long s = b >> 63;
@@ -204,7 +206,7 @@ __device__ __forceinline__ void fx_refit(longlong2 (&q)[NV][E], int (&ex)[NV], c
 }
 
 template <int MID, int NV, int E, typename Group>
-__device__ __forceinline__ void fx_load(double2 (&x)[NV][E], longlong2 (&q)[NV][E], int (&ex)[NV], int (&room)[NV],
+__device__ __forceinline__ void fx_load(const double2 (&x)[NV][E], longlong2 (&q)[NV][E], int (&ex)[NV], int (&room)[NV],
                                         const Group &g) {
     uint32_t mx[NV];
 #pragma unroll
@@ -218,16 +220,8 @@ __device__ __forceinline__ void fx_load(double2 (&x)[NV][E], longlong2 (&q)[NV][
     g.max(mx);
 #pragma unroll
     for (int iv = 0; iv < NV; ++iv) {
-        int em = (int)(mx[iv] >> 20);
+        const int em = (int)(mx[iv] >> 20);
         ex[iv] = em == 0x7ff ? kFxBad : em - 1023 - kFxTop;
-        if (em < kFxTop + 2) {
-            // smaller values, denormals (of field 1's exponent) among them: into the range, exactly
-#pragma unroll
-            for (int m = 0; m < E; ++m) x[iv][m] = make_double2(x[iv][m].x * 0x1p128, x[iv][m].y * 0x1p128);
-            em = max(em, 1);
-            ex[iv] = em - 1023 - kFxTop;
-            em += 128;
-        }
 #pragma unroll
         for (int m = 0; m < E; ++m) {
             q[iv][m].x = fx_from(x[iv][m].x, em);

@@ -65,7 +65,7 @@ def test_norm_of_small_complex64_fields(shape):
 
 
 @pytest.mark.parametrize("dtype", ["c64", "c128"])
-@pytest.mark.parametrize("shape", [(64,), (512,), (16, 64), (64, 256), (128, 128)])
+@pytest.mark.parametrize("shape", [(64,), (512,), (16, 64), (64, 256), (128, 128), (16, 32, 64)])
 def test_sampling_leaves_the_field_alone(shape, dtype):
     psi = _field(shape, 3)
     seen, _ = _samples(shape, dtype, 2.0, psi, steps=4, every=2)
