@@ -152,21 +152,14 @@ template <int NV, int E> __device__ __forceinline__ void fx_largest(const longlo
     }
 }
 
-// magnitude of q's high word: |q| <= 2^32 (m + 1) for either sign (the shift floors;
-// abs() would give -2^60 + 1 a magnitude of 2^28, and sixteen of those sum to 2^32 = 0)
-__device__ __forceinline__ uint32_t fx_mag(long long q) {
-    const int h = (int)(q >> 32);
-    return (uint32_t)(h ^ (h >> 31));
-}
-
 // Shift every line right for a transform: by room, which takes S to 2^60.5, or
 // by what the first MID points' sums need (largest values below 2^32 mx) where
 // that is less; `room` keeps the difference for fx_refit.  S is taken over the
-// high words' magnitudes (one unit of them covers what the low words add), whose sum
-// over a thread's 2E <= 16 values stays below 2^32: from fx_load |q| < 2^60 and each
-// is at most 2^28 - 1; after a transform, whose values are at most 2^60.5 (1 - 2^-26)
-// in modulus by the margins taken here and in fx_largest, a value's two are at most
-// 2^29 - 8 together.  In units of 2^41 a line's sum stays below 2^32.
+// high words' magnitudes (one unit of them covers what the low words add), of which a
+// 32-bit sum takes eight: a component just above -2^60 has 2^28 (the shift floors), and
+// sixteen of those would be 2^32, zero; after a transform, of values of at most 2^60.5 in
+// modulus, a value's two are at most 2^29 + 2.  In units of 2^41 a line's sum stays
+// below 2^32.
 template <int MID, int NV, int E, typename Group>
 __device__ __forceinline__ void fx_fit(longlong2 (&q)[NV][E], int (&ex)[NV], int (&room)[NV], const uint32_t (&mx)[NV],
                                        const Group &g) {
@@ -174,11 +167,11 @@ __device__ __forceinline__ void fx_fit(longlong2 (&q)[NV][E], int (&ex)[NV], int
     uint32_t s[NV];
 #pragma unroll
     for (int iv = 0; iv < NV; ++iv) {
-        uint32_t a = 0;
+        uint32_t a[2] = {0u, 0u};   // four points each
 #pragma unroll
         for (int m = 0; m < E; ++m)
-            a += fx_mag(q[iv][m].x) + fx_mag(q[iv][m].y);
-        s[iv] = (a >> 9) + 2u;
+            a[m / 4] += (uint32_t)abs((int)(q[iv][m].x >> 32)) + (uint32_t)abs((int)(q[iv][m].y >> 32));
+        s[iv] = E > 4 ? (((a[0] >> 1) + (a[1] >> 1)) >> 8) + 2u : (a[0] >> 9) + 2u;
     }
     g.sum(s);
     int sh[NV];
