@@ -148,8 +148,10 @@ int64_t xsde_grid_points(const xsde_grid *grid);
  * or noise from the grid (they copy it).  Runs on 1D lattices and on any
  * dimensions of 2D and 3D lattices (RK4IP; a cosine / sine last dimension runs
  * the generic row passes, and a 2D one takes its samples between chunks of
- * steps from the real-space field; cosine / sine columns of 128 and 256
- * points run the warp column pass, other 3D ones the generic passes); the semi-implicit scheme on 2D and 3D lattices,
+ * steps from the real-space field; complex64 cosine / sine columns of 128 and
+ * 256 points run the warp column pass, on 2D lattices where there are more tiles
+ * than SMs, else the TMA column pass; other 3D ones the generic passes); the
+ * semi-implicit scheme on 2D and 3D lattices,
  * xsde_integrate_plain, xsde_integrate_adaptive, xsde_adjoint,
  * xsde_integrate_static_scratch and xsde_set_nonlocal report XSDE_EUNSUPPORTED
  * for such a problem.  A 1D cosine / sine problem has one launch shape
@@ -198,7 +200,19 @@ int xsde_noise_normals(const xsde_noise *noise, xsde_dtype dtype, int64_t npts, 
 /* ---- problem -------------------------------------------------------------- */
 
 /* A problem binds a lattice, a precision and the operators; it owns the
- * device workspace (Fourier tables, one scratch field) that integration needs. */
+ * device workspace that integration needs: Fourier tables, one scratch field
+ * (2D and 3D lattices; three with the non-local term), and for noisy RK4IP steps
+ * on them a buffer of the step's normals (a real, with complex noise a complex
+ * value a point and path).  That buffer is taken when it is at most a quarter of
+ * the free device memory and given up when the scratch field cannot be had
+ * otherwise; without it every pass draws its normals again, the same ones.
+ *
+ * complex128 transforms run on 64-bit integers with one exponent a line of a
+ * dimension: what lies below 2^-59 of the line's largest component is truncated,
+ * denormal components (below 2.3e-308) count as zero, and a NaN or infinity makes
+ * its line NaN.  A field's result does not depend on
+ * whether RK4IP steps are sampled; a semi-implicit run splits the propagator of
+ * a step at its samples after the first and rounds differently there. */
 int xsde_problem_create(const xsde_grid *grid, xsde_dtype dtype, xsde_problem **out);
 void xsde_problem_destroy(xsde_problem *prob);
 
@@ -413,8 +427,8 @@ int xsde_synchronize(xsde_problem *prob, void *stream);
  *     complex64 (at most 128 registers a thread, a few values spilled: more
  *     warps to hide the exchanges' latency) and with all its registers in
  *     complex128; variant 6 is that shape with the other choice; variant 0 takes
- *     one of these shapes by precision, length and number of paths (few paths
- *     are spread over more threads); where a bound applies a variant repeats
+ *     one of these shapes by precision, length, noise and number of paths (few
+ *     paths are spread over more threads); where a bound applies a variant repeats
  *     another.  Shapes of 8, 4 and 2 points round differently, so that a path
  *     agrees bit for bit between ensembles of different sizes (the shares of an
  *     ensemble split over ranks) only where they run with the same variant
